@@ -162,6 +162,7 @@ cudaError_t launch_adjoint(int D, const AdjParams& p, int grid, cudaStream_t s) 
 // partial last spot chunk costs it more than the FMA kernel); the FMA-pipe
 // kernels otherwise. Variant 1 / 2 force one family (2 needs D <= 21).
 constexpr int kTcFwdMinSpots = 64, kTcAdjMinSpots = 256;
+
 bool use_tc_fwd(const ash_hologram* h) {
   if (!h->tc_ok || h->variant == 1) return false;
   return h->variant == 2 || (h->tc_na == 1 && h->g.N >= kTcFwdMinSpots);
@@ -170,6 +171,19 @@ bool use_tc_adj(const ash_hologram* h) {
   if (!h->tc_ok || h->variant == 1) return false;
   return h->variant == 2 || (h->tc_na == 1 && h->g.N >= kTcAdjMinSpots);
 }
+// The separable transforms serve the automatic choice for polynomial bases of
+// degree <= 4. The mixed terms of a tile shrink with the square (third order:
+// the cube) of the grid's side; below these sides most tiles need 16 or more
+// row strips and the others are faster (forward, us before / after: 256^2
+// N = 200 D = 10 18 / 40, 384^2 N = 200 D = 11 29 / 35, 512^2 N = 300 D = 10
+// 62 / 40; degree 2, 256^2 N = 100: 15 / 14). A step costs the same however
+// few of its 128 spots are used: with fewer than 64 it pays only where most
+// tiles need one strip (742 x 486 N = 27: 26 / 34; 1024^2 N = 20: 52 / 36).
+constexpr int kSepMinSide = 400, kSepMinSide2 = 200, kSepFewSpots = 64, kSepFewSide = 900;
+bool sep_pays(int ord, int side, int N) {
+  return ord <= 2 ? side >= kSepMinSide2 : side >= (N < kSepFewSpots ? kSepFewSide : kSepMinSide);
+}
+bool use_sep_fwd(const ash_hologram* h) { return h->sep_ok && h->variant == 0; }
 // The coefficient-gradient moments on the tensor cores need one K-atom,
 // D <= 12 and a polynomial basis of total degree <= 4 (the tile polynomials);
 // from N = 64, as the forward whose structure they share.
@@ -258,6 +272,10 @@ constexpr int kSrcImg = 2;
 
 cudaError_t enqueue_tc_coeff(ash_hologram* h, cudaStream_t s) {
   if (!h->tc_ok) return cudaSuccess;
+  if (h->sep_ok) {
+    const cudaError_t e = sep_build_params(h->g, h->sep_tab, h->coeff, h->sep_poly, h->sep_strips, h->sep_cost, s);
+    if (e != cudaSuccess) return e;
+  }
   return tc_build_coeff(h->g, h->tc_layout, h->coeff, h->anchors, h->czs, h->rot, s);
 }
 
@@ -277,6 +295,21 @@ TcFwdParams tc_fwd_params(const ash_hologram* h, float2* E) {
   p.err = h->err_word;
   p.claim = h->tfwd_nfull >= 0 ? h->tfwd_claim : nullptr;
   p.n_full = h->tfwd_nfull;
+  return p;
+}
+
+SepFwdParams sep_fwd_params(const ash_hologram* h, float2* E) {
+  SepFwdParams p{};
+  p.g = h->g;
+  p.nb = sep_blocks(h->g.N);
+  p.poly = h->sep_poly;
+  p.strips = h->sep_strips;
+  p.cost = h->sep_cost;
+  p.fimg = h->fimg;
+  p.part = h->sep_part;
+  p.E = E;
+  p.G = h->sep_G;
+  p.err = h->err_word;
   return p;
 }
 
@@ -311,11 +344,15 @@ cudaError_t launch_gradc(int D, const GradCParams& p, dim3 grid, cudaStream_t s)
 // forward transform into E (device complex [N]).
 ash_status enqueue_forward(ash_hologram* h, int source, const float* phase, const float2* field, float2* E,
                            cudaStream_t s) {
-  if (use_tc_fwd(h)) {
+  if (use_sep_fwd(h) || use_tc_fwd(h)) {
     cudaError_t e = cudaSuccess;
     if (source != kSrcImg) {
       e = tc_field_img(h->g, h->amp_img, source == kSrcPhase ? phase : nullptr, field, h->fimg, s);
       if (e != cudaSuccess) return cuda_fail(e, "nearfield image launch");
+    }
+    if (use_sep_fwd(h)) {
+      e = sep_launch_forward(sep_fwd_params(h, E), s);
+      return e == cudaSuccess ? ASH_OK : cuda_fail(e, "separable forward launch");
     }
     const TcFwdParams tp = tc_fwd_params(h, E);
     e = tc_launch_forward(h->tc_na, tp, h->tfwd.G, s);
@@ -380,7 +417,7 @@ ash_status enqueue_adjoint(ash_hologram* h, const float2* y, float2* g_out, floa
 // metrics. When both transforms run on the tensor cores the adjoint also
 // writes the next forward's nearfield (kEpiFimg), so only the first forward
 // converts a phase.
-bool wgs_fused_field(const ash_hologram* h) { return use_tc_fwd(h) && use_tc_adj(h); }
+bool wgs_fused_field(const ash_hologram* h) { return (use_sep_fwd(h) || use_tc_fwd(h)) && use_tc_adj(h); }
 
 ash_status enqueue_wgs_body(ash_hologram* h, int iters, cudaStream_t s) {
   const bool tc = wgs_fused_field(h);
@@ -768,6 +805,17 @@ ash_status create_impl(ash_hologram** out, int nx, int ny, int row0, int ny_full
       }
     }
   }
+  if (h->tc_ok && spec) {
+    int ord = 0;
+    for (const MonoTerm& m : spec->terms) ord = m.px + m.py > ord ? m.px + m.py : ord;
+    const int side = nx < ny_full ? nx : ny_full;
+    if (ord <= kSepMaxOrd && sep_pays(ord, side, N)) {
+      ce = sep_prepare();
+      if (ce != cudaSuccess) return fail(cuda_fail(ce, "separable kernel preparation"));
+      h->sep_ok = true;
+      h->sep_G = sms;
+    }
+  }
   h->gradc_gy = (N + kGradThreads * kGradSpots - 1) / (kGradThreads * kGradSpots);
   {
     const int slots = sms * (h->li.gradc_ctas_per_sm > 0 ? h->li.gradc_ctas_per_sm : 1);
@@ -798,6 +846,14 @@ ash_status create_impl(ash_hologram** out, int nx, int ny, int row0, int ny_full
     if ((st = ws(h, &h->tfwd_claim, (size_t)kTcClaimInts)) != ASH_OK) return fail(st);
     if ((st = ws(h, &h->tadj_begin, tadj_begin.size())) != ASH_OK) return fail(st);
     if ((st = ws(h, &h->tadj_groups, tadj_groups.size() + 1)) != ASH_OK) return fail(st);
+  }
+  if (h->sep_ok) {
+    const size_t npad = (size_t)sep_blocks(N) * kSepSpots;
+    if ((st = ws(h, &h->sep_tab, (size_t)g.T * D * kSepTab)) != ASH_OK) return fail(st);
+    if ((st = ws(h, &h->sep_poly, (size_t)g.T * 4 * npad)) != ASH_OK) return fail(st);
+    if ((st = ws(h, &h->sep_strips, (size_t)g.T * sep_blocks(N))) != ASH_OK) return fail(st);
+    if ((st = ws(h, &h->sep_cost, (size_t)g.T * sep_blocks(N) + 1)) != ASH_OK) return fail(st);
+    if ((st = ws(h, &h->sep_part, (size_t)kSepFwdRows * h->sep_G * npad)) != ASH_OK) return fail(st);
   }
   if (h->tgrad_ok) {
     if ((st = ws(h, &h->tpoly, tc_tpoly_floats(g, h->tgrad_ord))) != ASH_OK) return fail(st);
@@ -883,6 +939,7 @@ ash_status create_impl(ash_hologram** out, int nx, int ny, int row0, int ny_full
     // pixels outside the grid stay 0 in every nearfield image
     CREATE_CUDA(cudaMemsetAsync(h->fimg, 0, tc_fimg_float4s(g) * sizeof(float4), s));
   }
+  if (h->sep_ok) CREATE_CUDA(sep_build_table(g, h->terms, h->term_off, h->sep_tab, s));
   CREATE_CUDA(enqueue_tc_coeff(h, s));
   k_amp_image<<<g.T, g.NT, 0, s>>>(g, amp, h->amp_img);
   CREATE_CUDA(cudaGetLastError());
@@ -1202,8 +1259,9 @@ int ash_wgs_launches(const ash_hologram* h, int iters) {
   // forward: tensor-core (nearfield image unless fused, kernel, reduce if
   // split) or FMA (kernel, reduction); adjoint: kernel (+ fix-up)
   const bool fused = wgs_fused_field(h);
-  const int fwd_first = use_tc_fwd(h) ? 2 + (h->tfwd_split ? 1 : 0) : 2;
-  const int fwd = use_tc_fwd(h) ? (fused ? 1 : 2) + (h->tfwd_split ? 1 : 0) : 2;
+  const bool sep = use_sep_fwd(h);
+  const int fwd_first = sep ? 3 : use_tc_fwd(h) ? 2 + (h->tfwd_split ? 1 : 0) : 2;
+  const int fwd = sep ? (fused ? 2 : 3) : use_tc_fwd(h) ? (fused ? 1 : 2) + (h->tfwd_split ? 1 : 0) : 2;
   const int adj = use_tc_adj(h) ? 1 + (h->tadj_split ? 1 : 0) : 1 + (h->split_tiles ? 1 : 0);
   return fwd_first + iters * (1 + adj + fwd) + 1;   // + metrics
 }

@@ -11,6 +11,7 @@
 #include "common.cuh"
 #include "launch.h"
 #include "mono.h"
+#include "sep_launch.h"
 #include "tc_launch.h"
 
 struct ash_hologram {
@@ -61,6 +62,14 @@ struct ash_hologram {
   float* tgrad_part = nullptr;  // [tgrad.G][2][128][DC]
   int tgrad_ord = 0;            // total degree of the basis polynomials
   float* tpoly = nullptr;       // tile polynomials of the basis
+  // separable tile transforms (polynomial bases of total degree <= 4)
+  bool sep_ok = false;
+  int sep_G = 0;                // forward CTAs
+  float* sep_tab = nullptr;     // basis polynomials per tile
+  float4* sep_poly = nullptr;   // phase polynomials per (tile, spot)
+  unsigned char* sep_strips = nullptr;   // per (tile, spot block): log2 of its row strips
+  int* sep_cost = nullptr;      // prefix of its steps' cost
+  float2* sep_part = nullptr;   // [kSepFwdRows sep_G][128 nb]
   float2* split = nullptr;
   float* gradc_partial = nullptr;
   float2* E = nullptr;

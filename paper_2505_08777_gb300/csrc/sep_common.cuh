@@ -1,0 +1,134 @@
+// Separable tile transforms: shared layout, parameter blocks and device pieces.
+//
+// Over a 32 x 32 pixel tile a basis of total degree <= 4 gives every spot a
+// phase that is a polynomial of degree <= 4 in the pixel's offsets
+// u = (col - 16) / 16, v = (row - 16) / 16 from the tile's pixel (16, 16):
+//
+//   C_n . Z = 2 pi (base + px(u) + py(v)) + r(u, v),
+//   r(u, v) = u R1(v) + u^2 R2(v) + u^3 R3(v),   R_k(0) = 0.
+//
+// px and py (tilts, defocus, the pure powers) can be of any size; r holds
+// only the mixed terms, which over one tile are small. So the kernel
+// factors, exp(-i C.Z) = Y(v) X(u) exp(-i r), and with exp(-i r) as a cubic
+// in u (its coefficients Q_k are polynomials of R1 .. R3 per row) the sum
+// over a tile's pixels is
+//
+//   sum_v Y(v) sum_k Q_k(v) [ sum_u X(u) u^k f(u, v) ],
+//
+// where the bracket is a matrix product over the tile's columns: it runs on
+// the tensor cores (tcgen05, kind::f16, fp32 accumulators in TMEM), and a
+// (spot, tile) pair costs 32 + 32 sine / cosine pairs instead of 1024.
+//
+// fp32 accuracy from f16 operands (split-f16): every operand value |x| <= 1
+// is x = hi + lo with hi on the grid 2^-11 (exact in f16) and lo = f16(x -
+// hi), so that |x - hi - lo| <= 2^-25; the product is hi hi + hi lo + lo hi.
+// The nearfield is scaled by a power of two per tile to meet |x| <= 1.
+#pragma once
+
+#include "common.cuh"
+#include "sep_launch.h"
+#include "tc_common.cuh"
+#include "tc_launch.h"
+
+namespace ash {
+
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+  float2 d;
+  asm("{\n\t.reg .b64 ra, rb, rd;\n\t"
+      "mov.b64 ra, {%2, %3};\n\t"
+      "mov.b64 rb, {%4, %5};\n\t"
+      "add.rn.f32x2 rd, ra, rb;\n\t"
+      "mov.b64 {%0, %1}, rd;\n\t}"
+      : "=f"(d.x), "=f"(d.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return d;
+}
+__device__ __forceinline__ float2 dup2(float a) { return make_float2(a, a); }
+__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
+
+// hi of the split: x rounded to the grid 2^-11 (adding 1.5 * 2^12 leaves no
+// finer bits), for |x| <= 1.
+__device__ __forceinline__ float2 split_hi2(float2 x) {
+  return add2(add2(x, dup2(6144.0f)), dup2(-6144.0f));
+}
+// (a, b) as a pair of f16, a in the low half.
+__device__ __forceinline__ uint32_t pack_f16(float a, float b) {
+  uint32_t d;
+  asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(b), "f"(a));
+  return d;
+}
+
+// Instruction descriptor of kind::f16 with f16 operands and an fp32
+// accumulator, both operands K-major, shape M x N.
+__host__ __device__ constexpr uint32_t umma_idesc_f16(int M, int N) {
+  return (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+}
+__device__ __forceinline__ void umma_f16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
+                                         uint32_t accumulate) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
+      "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate));
+}
+
+// 8 consecutive fp32 columns of this thread's TMEM lane, without waiting.
+__device__ __forceinline__ void tmem_ld8_nowait(uint32_t taddr, uint32_t* r) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr));
+}
+
+// Byte offset of the 16-byte chunk c (0..7) of row r in a K-major operand of
+// 128-byte rows (64 f16) with the 128-byte swizzle.
+__device__ __forceinline__ uint32_t swz_chunk(int r, int c) { return (uint32_t)(r * 128 + ((c ^ (r & 7)) << 4)); }
+
+// A (tile, spot)'s phase polynomial as stored by k_sep_params, in the pixel
+// offsets mx = col - 16, my = row - 16 from the tile's pixel (16, 16).
+struct SepPoly {
+  float base;                  // at that pixel, radians, about [-pi, pi]
+  float ax, ay;                // turns per pixel along columns and rows,
+  float axl, ayl;              // and what their rounding left, radians
+  float x2, x3, x4;            // mx^2, mx^3, mx^4, radians
+  float y2, y3, y4;            // my^2, my^3, my^4, radians
+  // mixed terms u^k my^l (u = mx / 16), radians; n31 negated
+  float c11, c21, c12, c22, n31, c13;
+};
+
+__device__ __forceinline__ uint32_t pack_bf16_rz(float lo, float hi) {
+  return (__float_as_uint(lo) >> 16) | (__float_as_uint(hi) & 0xffff0000u);
+}
+
+__device__ __forceinline__ SepPoly sep_unpack(float4 a, float4 b, float4 c, float4 d) {
+  SepPoly p;
+  p.base = a.x;
+  p.ax = a.y;
+  p.ay = a.z;
+  const uint32_t lo = __float_as_uint(a.w);
+  p.axl = __uint_as_float(lo << 16);
+  p.ayl = __uint_as_float(lo & 0xffff0000u);
+  p.x2 = b.x; p.x3 = b.y; p.x4 = b.z; p.y2 = b.w;
+  p.y3 = c.x; p.y4 = c.y; p.c11 = c.z; p.c21 = c.w;
+  p.c12 = d.x; p.c22 = d.y; p.n31 = d.z; p.c13 = d.w;
+  return p;
+}
+
+// sin and cos of two angles of at most about 2 pi through the MUFU.
+__device__ __forceinline__ void cis2(float2 x, float2& c, float2& s) {
+  s.x = __sinf(x.x);
+  c.x = __cosf(x.x);
+  s.y = __sinf(x.y);
+  c.y = __cosf(x.y);
+}
+
+// The angles base + 2 pi a m + m (al + q2 m + q3 m^2 + q4 m^3), less a whole
+// number of turns of a m, for two offsets m; a - rint(a m) / m is exact. `na`
+// is -a (the packed operations take no sign).
+__device__ __forceinline__ float2 sep_angle(float a, float na, float al, float q2, float q3, float q4, float2 base,
+                                            float2 m) {
+  const float2 k = add2(fma2(dup2(na), m, dup2(12582912.0f)), dup2(-12582912.0f));   // -rint(a m)
+  const float2 r = fma2(dup2(a), m, k);
+  const float2 q = fma2(fma2(fma2(dup2(q4), m, dup2(q3)), m, dup2(q2)), m, dup2(al));
+  return fma2(r, dup2(6.283185307179586f), fma2(q, m, base));
+}
+
+}  // namespace ash

@@ -1,0 +1,636 @@
+// Separable forward transform (see sep_common.cuh): the tables it works from,
+// the kernel and the sum of its CTAs' partial fields.
+#include "sep_common.cuh"
+
+namespace ash {
+
+namespace {
+
+// --- tables ---------------------------------------------------------------------
+
+// One thread per (tile, mode): sum coef x^a y^b about pixel (16, 16) in fp64.
+__global__ void k_sep_table(const Geometry G, const MonoTerm* __restrict__ terms, const int* __restrict__ term_off,
+                            float* __restrict__ tab) {
+  const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= (long long)G.T * G.D) return;
+  const int d = (int)(e % G.D), tile = (int)(e / G.D);
+  const double R = grid_radius(G);
+  const double xc = grid_x(G, (double)((tile % G.tiles_x) * kTileX) + 16.0);
+  const double yc = grid_y(G, (double)((tile / G.tiles_x) * kTileY) + 16.0);
+  double b[5][5] = {};
+  for (int t = term_off[d]; t < term_off[d + 1]; ++t) {
+    const MonoTerm m = terms[t];
+    // coefficients of (xc + x)^px and (yc + y)^py
+    double fx[5], fy[5];
+    auto expand = [](int n, double c, double* f) {
+      for (int k = 0; k <= 4; ++k) f[k] = 0.0;
+      double binom = 1.0;
+      for (int k = 0; k <= n && k <= 4; ++k) {
+        double p = binom;
+        for (int q = 0; q < n - k; ++q) p *= c;
+        f[k] = p;
+        binom = binom * (n - k) / (k + 1);
+      }
+    };
+    expand(m.px, xc, fx);
+    expand(m.py, yc, fy);
+    for (int k = 0; k <= 4; ++k)
+      for (int l = 0; k + l <= 4; ++l) b[k][l] += m.coef * fx[k] * fy[l];
+  }
+  const double turn = 0.15915494309189533576888376337251, s = 16.0 / R;
+  double pw[5] = {1.0, s, s * s, s * s * s, s * s * s * s};
+  float* o = tab + (size_t)e * kSepTab;
+  const double hl[3] = {b[0][0] * turn, b[1][0] * turn / R, b[0][1] * turn / R};
+  for (int k = 0; k < 3; ++k) {
+    o[2 * k] = (float)hl[k];
+    o[2 * k + 1] = (float)(hl[k] - (double)o[2 * k]);
+  }
+  o[6] = (float)(b[2][0] * pw[2] * turn);
+  o[7] = (float)(b[3][0] * pw[3] * turn);
+  o[8] = (float)(b[4][0] * pw[4] * turn);
+  o[9] = (float)(b[0][2] * pw[2] * turn);
+  o[10] = (float)(b[0][3] * pw[3] * turn);
+  o[11] = (float)(b[0][4] * pw[4] * turn);
+  // mixed terms in radians
+  o[12] = (float)(b[1][1] * pw[2]);
+  o[13] = (float)(b[2][1] * pw[3]);
+  o[14] = (float)(b[1][2] * pw[3]);
+  o[15] = (float)(b[2][2] * pw[4]);
+  o[16] = (float)(b[3][1] * pw[4]);
+  o[17] = (float)(b[1][3] * pw[4]);
+}
+
+// acc (hi, lo) += c (bh + bl), with the rounding errors of the product and
+// the sum kept in lo.
+__device__ __forceinline__ void acc_hl(float& hi, float& lo, float c, float bh, float bl) {
+  const float p = __fmul_rn(c, bh);
+  const float e = __fmaf_rn(c, bl, __fmaf_rn(c, bh, -p));
+  const float s = __fadd_rn(hi, p);
+  const float z = __fsub_rn(s, hi);
+  lo = __fadd_rn(lo, __fadd_rn(e, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, z)), __fsub_rn(p, z))));
+  hi = s;
+}
+
+// CTA (tile, block): thread = spot. Bound: the table is read once per CTA
+// from shared memory and 64 B per (tile, spot) are written.
+__global__ void __launch_bounds__(kSepSpots) k_sep_params(const Geometry G, const float* __restrict__ tab,
+                                                          const float* __restrict__ coeff, float4* __restrict__ poly,
+                                                          unsigned char* __restrict__ strips, int npad) {
+  __shared__ float st[kMaxModes * kSepTab];
+  __shared__ int sred[4];
+  const int tile = blockIdx.x, b = blockIdx.y, t = threadIdx.x, D = G.D;
+  for (int k = t; k < D * kSepTab; k += kSepSpots) st[k] = __ldg(tab + (size_t)tile * D * kSepTab + k);
+  __syncthreads();
+  const int n = b * kSepSpots + t;
+  float base = 0.0f, axh = 0.0f, axl = 0.0f, ayh = 0.0f, ayl = 0.0f;
+  float q[12] = {};
+  if (n < G.N) {
+    for (int d = 0; d < D; ++d) {
+      const float c = __ldg(coeff + (size_t)n * D + d);
+      const float* o = st + d * kSepTab;
+      // base: every product and sum reduced modulo one turn (base_turns)
+      const float p = __fmul_rn(c, o[0]);
+      const float e = __fmaf_rn(c, o[0], -p);
+      const float r = __fsub_rn(p, rint_fma_pipe(p));
+      base = __fadd_rn(base, __fadd_rn(r, __fmaf_rn(c, o[1], e)));
+      base = __fsub_rn(base, rint_fma_pipe(base));
+      acc_hl(axh, axl, c, o[2], o[3]);
+      acc_hl(ayh, ayl, c, o[4], o[5]);
+#pragma unroll
+      for (int k = 0; k < 12; ++k) q[k] = __fmaf_rn(c, o[6 + k], q[k]);
+    }
+    const float x = __fadd_rn(axh, axl), y = __fadd_rn(ayh, ayl);
+    axl = __fsub_rn(axl, __fsub_rn(x, axh));
+    ayl = __fsub_rn(ayl, __fsub_rn(y, ayh));
+    axh = x;
+    ayh = y;
+  }
+  // radians per pixel offset (u = mx / 16, v = my / 16)
+  constexpr float tp = 6.283185307179586f, h = 0.0625f;
+  const size_t o = (size_t)tile * 4 * npad + n;
+  poly[o] = make_float4(tp * base, axh, ayh, __uint_as_float(pack_bf16_rz(tp * axl, tp * ayl)));
+  poly[o + npad] = make_float4(tp * q[0] * (h * h), tp * q[1] * (h * h * h), tp * q[2] * (h * h * h * h),
+                               tp * q[3] * (h * h));
+  poly[o + 2 * (size_t)npad] = make_float4(tp * q[4] * (h * h * h), tp * q[5] * (h * h * h * h), q[6] * h, q[7] * h);
+  poly[o + 3 * (size_t)npad] = make_float4(q[8] * (h * h), q[9] * (h * h), -q[10] * h, q[11] * (h * h * h));
+  // Row strips: the cubic in u takes u^4 R1^4 / 24 etc. as u^2 (off by at most
+  // 1/4) and drops the rest; with 2^k strips R_k about a strip's middle row is
+  // at most |dR_k/dv| / 2^k. The fewest strips that drop less than kSepTol.
+  auto dropped = [](float R1, float R2, float R3) {
+    const float s = R1 * R1;
+    const float e4 = s * s * (1.0f / 24.0f) + 0.5f * s * R2 + 0.5f * R2 * R2;
+    const float e5 = s * s * R1 * (1.0f / 120.0f) + s * R1 * R2 * (1.0f / 6.0f) + 0.5f * R1 * R2 * R2 + 0.5f * s * R3 +
+                     R2 * R3;
+    return 0.25f * e4 + R1 * R3 + e5;
+  };
+  const float a11 = fabsf(q[6]), a21 = fabsf(q[7]), a12 = fabsf(q[8]), a22 = fabsf(q[9]), a31 = fabsf(q[10]),
+              a13 = fabsf(q[11]);
+  int k = 0;
+  if (!(dropped(a11 + a12 + a13, a21 + a22, a31) <= kSepTol)) {
+    float f = 0.5f;
+    for (k = 1; k < 5; ++k, f *= 0.5f)
+      if (dropped(f * (a11 + 2.0f * a12 + 3.0f * a13), f * (a21 + 2.0f * a22), f * a31) <= kSepTol) break;
+  }
+  k = __reduce_max_sync(0xffffffffu, k);
+  if ((t & 31) == 0) sred[t >> 5] = k;
+  __syncthreads();
+  if (t == 0) strips[(size_t)tile * gridDim.y + b] = (unsigned char)max(max(sred[0], sred[1]), max(sred[2], sred[3]));
+}
+
+// Cost prefix of the (tile, spot block) units, cost[u] .. cost[u + 1]: unit u
+// runs 2^strips[u] steps of kSepStepCost. One CTA of 1024 threads.
+__global__ void k_sep_scan(const unsigned char* __restrict__ strips, int U, int* __restrict__ cost) {
+  __shared__ int wsum[32];
+  const int t = threadIdx.x, per = (U + 1023) / 1024;
+  const int a = min(U, t * per), b = min(U, a + per);
+  int sum = 0;
+  for (int u = a; u < b; ++u) sum += sep_step_cost(strips[u]) << strips[u];
+  int inc = sum;
+  for (int h = 1; h < 32; h <<= 1) {
+    const int v = __shfl_up_sync(0xffffffffu, inc, h);
+    if ((t & 31) >= h) inc += v;
+  }
+  if ((t & 31) == 31) wsum[t >> 5] = inc;
+  __syncthreads();
+  if (t < 32) {
+    int v = wsum[t];
+    for (int h = 1; h < 32; h <<= 1) {
+      const int x = __shfl_up_sync(0xffffffffu, v, h);
+      if (t >= h) v += x;
+    }
+    wsum[t] = v;
+  }
+  __syncthreads();
+  int acc = inc - sum + (t >= 32 ? wsum[(t >> 5) - 1] : 0);
+  for (int u = a; u < b; ++u) {
+    cost[u] = acc;
+    acc += sep_step_cost(strips[u]) << strips[u];
+  }
+  if (t == 1023) cost[U] = acc;
+}
+
+// --- forward --------------------------------------------------------------------
+
+// One CTA per SM, 20 warps in three roles. The generators (warps 8-15)
+// prepare the steps' operands, the summers (warps 0-7) read the results, one
+// thread (warp 17) lists the steps and fetches their phase polynomials, and
+// one (warp 16) issues the MMAs (issuing blocks while the tensor core is
+// busy, so no generator does it). A step: A = X(u) of 128 spots, rows [Re X(0..31) | Im X(0..31)];
+// B = the tile's nearfield times u^k, k = 0..3, rows (k / 2, row pair, k % 2,
+// re / im, row of the pair), [Re f | -Im f] and [Im f | Re f]. D[spot][256]
+// then holds the four complex sums of every tile row, to which the summers
+// apply Q_k(v) and Y(v). The low parts of the operands enter for k = 0, 1
+// only: |Q_2|, |Q_3| < 0.01. A, B and D have two buffers each, so the
+// generators, the tensor core and the summers work on different steps.
+constexpr int kFwdThreads = 640;
+// Registers: 20 warps launch with 96 a thread; the summers take 120, the
+// generators keep 96, the last warpgroup drops to 40.
+static_assert(2 * 120 + 2 * 96 + 40 <= 5 * 96);
+constexpr uint32_t kFA = 16384, kFB = 32768, kFBlo = 16384, kFSlot = 4 * 2048;
+constexpr uint32_t kFwdBuf = kFB + kFBlo;                            // one B buffer
+constexpr size_t kFwdB = 4 * kFA, kFwdSlots = kFwdB + 2 * kFwdBuf;   // slots: phase polynomials of 128 spots, 4 steps
+constexpr size_t kFwdTail = kFwdSlots + 4 * kFSlot;                  // barriers, TMEM slot, maxima, step records
+constexpr size_t kFwdSmem = 1024 + kFwdTail + 256;
+
+// A step: spot block b (-1: no more steps) of a tile, strip s of 2^ls, and the
+// B buffer that holds (or is to hold) the tile.
+struct SepStep {
+  int tile, b, s, ls, bb;
+};
+
+// Offset my of a strip's middle row (0 for the whole tile).
+__device__ __forceinline__ float strip_mid(int s, int ls) {
+  const int n = 32 >> ls;
+  return ls == 0 ? 0.0f : (float)(s * n - 16) + 0.5f * (float)(n - 1);
+}
+
+__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+// The tensor core's fp32 accumulator truncates: measured over 256^2 to
+// 1920 x 1152 pixels, fields came out smaller by 2.8e-7 of themselves whatever
+// the input, and by 5e-8 at random. The scale makes up for the first.
+constexpr float kTruncation = 1.0f + 2.4e-7f;
+
+// Sums over row pairs of c Tr, s Ti, c Ti, s Tr, with Y = c - i s.
+struct SepSum {
+  float2 cr, si, ci, sr;
+  __device__ __forceinline__ void zero() { cr = si = ci = sr = make_float2(0.0f, 0.0f); }
+};
+
+// acc += Y(v) sum_k Q_k(v) D_k(v) over one pair of rows, offsets m; x and z
+// hold D_0, D_1 and D_2, D_3 of the pair (re, im; both rows). `one` >= 0: only
+// that row of the pair counts.
+__device__ __forceinline__ void sep_sum_pair(const SepPoly& q, float R1s, float R2s, float n3s, const uint32_t* x,
+                                             const uint32_t* z, float2 m, int one, SepSum& acc) {
+  auto D = [](const uint32_t* a, int i) { return make_float2(__uint_as_float(a[2 * i]), __uint_as_float(a[2 * i + 1])); };
+  const float2 R1 = fma2(fma2(fma2(dup2(q.c13), m, dup2(q.c12)), m, dup2(q.c11)), m, dup2(-R1s));
+  const float2 R2 = fma2(fma2(dup2(q.c22), m, dup2(q.c21)), m, dup2(-R2s));
+  const float2 n3 = fma2(dup2(q.n31), m, dup2(-n3s));   // -R3
+  // exp(-i r) = 1 - i R1 u + q2 u^2 + q3 u^3, with the u^4 term taken as u^2
+  const float2 n1 = mul2(R1, dup2(-1.0f)), s = mul2(R1, R1);
+  const float2 q2r = fma2(s, fma2(s, dup2(1.0f / 24.0f), dup2(-0.5f)), mul2(R2, mul2(R2, dup2(-0.5f))));
+  const float2 q2i = mul2(R2, fma2(s, dup2(0.5f), dup2(-1.0f)));
+  const float2 q3r = mul2(n1, R2), q3i = fma2(mul2(R1, s), dup2(1.0f / 6.0f), n3);
+  const float2 ur = fma2(q3i, D(z, 3), mul2(q2i, D(z, 1)));
+  float2 Tr = fma2(q3r, D(z, 2), fma2(q2r, D(z, 0), fma2(R1, D(x, 3), D(x, 0))));
+  Tr = fma2(ur, dup2(-1.0f), Tr);
+  float2 Ti = fma2(q2r, D(z, 1), fma2(n1, D(x, 2), D(x, 1)));
+  Ti = fma2(q3r, D(z, 3), fma2(q3i, D(z, 2), fma2(q2i, D(z, 0), Ti)));
+  float2 c, sn;
+  cis2(sep_angle(q.ay, -q.ay, q.ayl, q.y2, q.y3, q.y4, dup2(q.base), m), c, sn);
+  if (one >= 0) {
+    const float2 w = one ? make_float2(0.0f, 1.0f) : make_float2(1.0f, 0.0f);
+    c = mul2(c, w);
+    sn = mul2(sn, w);
+  }
+  acc.cr = fma2(c, Tr, acc.cr);
+  acc.si = fma2(sn, Ti, acc.si);
+  acc.ci = fma2(c, Ti, acc.ci);
+  acc.sr = fma2(sn, Tr, acc.sr);
+}
+
+// The row pairs [p0, p0 + np) of D at TMEM address ta (np 1 or even).
+__device__ __forceinline__ void sep_sum_rows(const SepPoly& q, float ms, uint32_t ta, int p0, int np, int one,
+                                             SepSum& acc) {
+  const float R1s = ms * (q.c11 + ms * (q.c12 + ms * q.c13)), R2s = ms * (q.c21 + ms * q.c22), n3s = ms * q.n31;
+  uint32_t x[16], z[16];
+  if (np == 1) {
+    tmem_ld8_nowait(ta + (uint32_t)(p0 * 8), x);
+    tmem_ld8_nowait(ta + (uint32_t)(128 + p0 * 8), z);
+    tmem_wait();
+    const float m0 = (float)(2 * p0 - 16);
+    sep_sum_pair(q, R1s, R2s, n3s, x, z, make_float2(m0, m0 + 1.0f), one, acc);
+    return;
+  }
+  for (int k = 0; k < np; k += 2) {
+    tmem_ld16_nowait(ta + (uint32_t)((p0 + k) * 8), x);
+    tmem_ld16_nowait(ta + (uint32_t)(128 + (p0 + k) * 8), z);
+    tmem_wait();
+    const float m0 = (float)(2 * (p0 + k) - 16);
+    sep_sum_pair(q, R1s, R2s, n3s, x, z, make_float2(m0, m0 + 1.0f), -1, acc);
+    sep_sum_pair(q, R1s, R2s, n3s, x + 8, z + 8, make_float2(m0 + 2.0f, m0 + 3.0f), -1, acc);
+  }
+}
+
+// (c, s) split into f16 pairs (hi, lo); s negated by the caller's angle.
+__device__ __forceinline__ void split_pack(float2 v, uint32_t& hi, uint32_t& lo) {
+  const float2 h = split_hi2(v), l = fma2(h, dup2(-1.0f), v);
+  hi = pack_f16(h.x, h.y);
+  lo = pack_f16(l.x, l.y);
+}
+
+__device__ __forceinline__ void put16(uint8_t* base, int r, int c, const uint32_t (&v)[4], uint32_t flip = 0) {
+  *reinterpret_cast<uint4*>(base + swz_chunk(r, c)) = make_uint4(v[0] ^ flip, v[1] ^ flip, v[2] ^ flip, v[3] ^ flip);
+}
+
+__global__ void __launch_bounds__(kFwdThreads, 1) k_sep_forward(const SepFwdParams p) {
+  extern __shared__ uint8_t raw[];
+  uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(raw) + 1023) & ~(uintptr_t)1023);
+  uint64_t* full = reinterpret_cast<uint64_t*>(sm + kFwdTail);   // [2] MMAs of a step done
+  uint64_t* empty = full + 2;                                    // [4] its D and slot read
+  uint64_t* ready = full + 6;                                    // [4] its operands written
+  uint64_t* listed = full + 10;                                  // [4] its record and polynomials written
+  uint32_t* slot = reinterpret_cast<uint32_t*>(full + 14);
+  uint32_t* smax = slot + 2;                                     // [8]
+  float* scales = reinterpret_cast<float*>(smax + 8);            // [4] 2^e of the steps' tiles
+  SepStep* steps = reinterpret_cast<SepStep*>(scales + 4);       // [4]
+  const int t = threadIdx.x, w = t >> 5, lane = t & 31;
+  const int row = t & 127;
+  const int nb = p.nb, npad = nb * kSepSpots, U = p.g.T * nb;
+  if (w == 0) tmem_alloc(slot, 512);
+  if (t == 0) {
+    for (int k = 0; k < 14; ++k) mbar_init(full + k, k >= 2 && k < 6 ? 8 : 1);
+    fence_mbar_init();
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *slot;
+  bool ok = true;
+
+  if (w < 8) {
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 120;");
+    // --- summers: spot `row`, half of a step's row pairs ---
+    const int half = t >> 7;
+    float2* part = p.part + (size_t)(kSepFwdRows * blockIdx.x + half) * npad + row;
+    // no other thread touches these partial sums
+    for (int b = 0; b < nb; ++b) part[b * kSepSpots] = make_float2(0.0f, 0.0f);
+    const uint32_t tlane = tmem + ((uint32_t)((w & 3) * 32) << 16);
+    SepSum acc;
+    acc.zero();
+    int pb = -1;          // block and scale of the sums held
+    float psc = 1.0f, pscale = 1.0f;
+    for (uint32_t it = 0;; ++it) {
+      ok = ok && mbar_wait(&ready[it & 3], (it >> 2) & 1, kTcWaitPolls);
+      ok = __all_sync(0xffffffffu, ok);
+      if (!ok) break;
+      const SepStep r = steps[it & 3];
+      const float scale = scales[it & 3];
+      if (r.b != pb || scale != psc) {
+        if (pb >= 0) {
+          float2* o = part + pb * kSepSpots;
+          atomicAdd(&o->x, ((acc.cr.x + acc.cr.y) + (acc.si.x + acc.si.y)) * pscale);
+          atomicAdd(&o->y, ((acc.ci.x + acc.ci.y) - (acc.sr.x + acc.sr.y)) * pscale);
+        }
+        acc.zero();
+        pb = r.b;
+        pscale = scale * kTruncation;
+        psc = scale;
+      }
+      if (r.b < 0) break;
+      const float4* sq = reinterpret_cast<const float4*>(sm + kFwdSlots + (it & 3) * kFSlot) + row;
+      const SepPoly q = sep_unpack(sq[0], sq[128], sq[256], sq[384]);
+      const int rows = 32 >> r.ls, pairs = rows >= 2 ? rows >> 1 : 1;
+      const int np = pairs >= 2 ? pairs >> 1 : (half ? 0 : 1), p0 = ((r.s * rows) >> 1) + half * np;
+      ok = ok && mbar_wait(&full[it & 1], (it >> 1) & 1, kTcWaitPolls);
+      ok = __all_sync(0xffffffffu, ok);
+      if (!ok) break;
+      tc_fence_after();
+      if (np > 0)
+        sep_sum_rows(q, strip_mid(r.s, r.ls), tlane + 256u * (it & 1), p0, np, rows == 1 ? (r.s & 1) : -1, acc);
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&empty[it & 3]);
+    }
+  } else if (w >= 16) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
+    if (w == 16 && lane == 0) {
+      // --- MMA issue ---
+      uint32_t it = 0;
+      for (;; ++it) {
+        const int d = it & 1;
+        ok = ok && mbar_wait(&ready[it & 3], (it >> 2) & 1, kTcWaitPolls);
+        if (it >= 2) ok = ok && mbar_wait(&empty[(it - 2) & 3], ((it - 2) >> 2) & 1, kTcWaitPolls);
+        if (!ok) break;
+        const SepStep r = steps[it & 3];
+        if (r.b < 0) break;
+        tc_fence_after();
+        // the columns of the step's rows in each half of D (N >= 16)
+        const int rows = 32 >> r.ls, p0 = (r.s * rows) >> 1;
+        const int n = rows >= 4 ? rows * 4 : 16, col = (n == 16 ? (p0 & ~1) : p0) * 8;
+        const uint32_t dst = tmem + (uint32_t)(256 * d + col), idesc = umma_idesc_f16(128, n);
+        // (descriptors count 16-byte units)
+        const uint64_t a = umma_desc(smem_u32(sm) + (uint32_t)d * 2 * kFA);
+        const uint64_t b = umma_desc(smem_u32(sm + kFwdB) + (uint32_t)r.bb * kFwdBuf + (uint32_t)col * 128);
+        // the small products first: the accumulator truncates every sum
+        const uint64_t al = a + (kFA >> 4), bl = b + (kFB >> 4), b1 = b + 128 * 8;
+#pragma unroll
+        for (int ks = 0; ks < 8; ks += 2) {
+          umma_f16(dst, al + ks, b + ks, idesc, ks > 0);
+          umma_f16(dst, a + ks, bl + ks, idesc, 1u);
+        }
+        umma_f16(dst, a, b, idesc, 1u);
+        umma_f16(dst + 128, a, b1, idesc, 0u);
+        if (r.ls == 0) {
+#pragma unroll
+          for (int ks = 2; ks < 8; ks += 2) umma_f16(dst, a + ks, b + ks, umma_idesc_f16(128, 256), 1u);
+        } else {
+#pragma unroll
+          for (int ks = 2; ks < 8; ks += 2) {
+            umma_f16(dst, a + ks, b + ks, idesc, 1u);
+            umma_f16(dst + 128, a + ks, b1 + ks, idesc, 1u);
+          }
+        }
+        umma_commit(&full[d]);
+      }
+      // nothing in flight when the CTA gives up its memory
+      for (uint32_t k = it > 2 ? it - 2 : 0; k < it; ++k) ok = mbar_wait(&full[k & 1], (k >> 1) & 1, kTcWaitPolls) && ok;
+    } else if (w == 17 && lane == 0) {
+      // --- steps of this CTA: those whose place in the cost prefix lies in [c0, c1) ---
+      const long long W = p.cost[U];
+      const int c0 = (int)(W * blockIdx.x / p.G), c1 = (int)(W * (blockIdx.x + 1) / p.G);
+      int u = 0, hi = U - 1;
+      while (u < hi) {
+        const int mid = (u + hi + 1) / 2;
+        if (p.cost[mid] <= c0) u = mid;
+        else hi = mid - 1;
+      }
+      SepStep x{u / nb, u % nb, 0, p.strips[u], 0};
+      int pos = p.cost[u], c = sep_step_cost(x.ls);
+      x.s = (c0 - pos + c - 1) / c;
+      pos += x.s * c;
+      int ls1 = u + 1 < U ? p.strips[u + 1] : 0;   // of the next unit, fetched early
+      uint32_t it = 0;
+      for (;; ++it) {
+        if (x.s >> x.ls) {
+          ++u;
+          x.s = 0;
+          x.ls = ls1;
+          c = sep_step_cost(ls1);
+          if (++x.b == nb) {
+            x.b = 0;
+            ++x.tile;
+            x.bb ^= 1;
+          }
+          if (u + 1 < U) ls1 = p.strips[u + 1];
+        }
+        const bool more = pos < c1;
+        // slot it & 3 was step it - 4's
+        if (it >= 4) ok = ok && mbar_wait(&empty[it & 3], ((it >> 2) - 1) & 1, kTcWaitPolls);
+        steps[it & 3] = more ? x : SepStep{0, -1, 0, 0, 0};
+        if (!more) {
+          mbar_arrive(&listed[it & 3]);
+          break;
+        }
+        mbar_expect_tx(&listed[it & 3], kFSlot);
+        const float4* src = p.poly + (size_t)x.tile * 4 * npad + x.b * kSepSpots;
+        for (int k = 0; k < 4; ++k)
+          bulk_g2s(sm + kFwdSlots + (it & 3) * kFSlot + k * 2048, src + (size_t)k * npad, 2048, &listed[it & 3]);
+        pos += c;
+        ++x.s;
+      }
+      for (uint32_t k = it > 3 ? it - 3 : 0; k < it; ++k) ok = mbar_wait(&listed[k & 3], (k >> 2) & 1, kTcWaitPolls) && ok;
+    }
+    __syncwarp();
+  } else {
+    // --- generators: spot `row`, half of the columns ---
+    const int g = t - 256, half = g >> 7;
+    auto gen_sync = [&]() { asm volatile("bar.sync 1, 256;" ::: "memory"); };
+    // B of a tile; returns the tile's scale 2^e (the nearfield is divided by it)
+    auto build_b = [&](int tile, uint8_t* bh) -> float {
+      // thread: tile row j, 8 columns from 8 c, powers u^(2 kh), u^(2 kh + 1)
+      const int j = g >> 3, c = g & 3, kh = (g >> 2) & 1;
+      const float4* f = p.fimg + ((size_t)tile * kTcChunksPerTile + (j >> 1)) * 32 + (j & 1) * 16 + c * 4;
+      float4 v[4];
+      float mx = 0.0f;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        v[q] = __ldg(f + q);
+        mx = fmaxf(mx, fmaxf(fabsf(v[q].x), fabsf(v[q].y)));
+      }
+      const uint32_t wm = __reduce_max_sync(0xffffffffu, __float_as_uint(mx));
+      if (lane == 0) smax[g >> 5] = wm;
+      gen_sync();
+      uint32_t m = 0;
+#pragma unroll
+      for (int q = 0; q < 8; ++q) m = max(m, smax[q]);
+      // exponent e with max < 2^e, kept where 2^e and 2^-e are normal
+      const int e = min(max((int)(m >> 23), 27), 227) - 126;
+      const float inv = __uint_as_float((uint32_t)(127 - e) << 23);
+      constexpr uint32_t S = 0x80008000u;
+#pragma unroll
+      for (int k2 = 0; k2 < 2; ++k2) {
+        uint32_t rh[4], rl[4], ih[4], il[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const float2 u = make_float2((float)(8 * c + 2 * q - 16) * 0.0625f, (float)(8 * c + 2 * q - 15) * 0.0625f);
+          float2 cs, sn;
+          cis2(mul2(make_float2(v[q].z, v[q].w), dup2(6.283185307179586f)), cs, sn);
+          float2 a = mul2(make_float2(v[q].x, v[q].y), dup2(inv));
+          if (kh) a = mul2(a, mul2(u, u));
+          if (k2) a = mul2(a, u);
+          split_pack(mul2(a, cs), rh[q], rl[q]);
+          split_pack(mul2(a, sn), ih[q], il[q]);
+        }
+        const int r0 = kh * 128 + (j >> 1) * 8 + k2 * 4 + (j & 1);   // re row; im row is r0 + 2
+        put16(bh, r0, c, rh);
+        put16(bh, r0, 4 + c, ih, S);
+        put16(bh, r0 + 2, c, ih);
+        put16(bh, r0 + 2, 4 + c, rh);
+        if (kh == 0) {
+          put16(bh + kFB, r0, c, rl);
+          put16(bh + kFB, r0, 4 + c, il, S);
+          put16(bh + kFB, r0 + 2, c, il);
+          put16(bh + kFB, r0 + 2, 4 + c, rl);
+        }
+      }
+      return __uint_as_float((uint32_t)(127 + e) << 23);
+    };
+
+    // A: X(u) of this thread's spot for its 16 columns, about the strip's row
+    auto build_a = [&](const float4* sq, const SepStep& x, uint8_t* ah) {
+      const SepPoly q = sep_unpack(sq[0], sq[128], sq[256], sq[384]);
+      float ax = q.ax, axl = q.axl, x2 = q.x2, x3 = q.x3;
+      if (x.ls) {
+        const float ms = strip_mid(x.s, x.ls);
+        const float R1 = ms * (q.c11 + ms * (q.c12 + ms * q.c13)), R2 = ms * (q.c21 + ms * q.c22), n3 = ms * q.n31;
+        const float d = R1 * (0.15915494309189535f * 0.0625f);
+        const float s = __fadd_rn(ax, d), z = __fsub_rn(s, ax);
+        axl = fmaf(__fadd_rn(__fsub_rn(ax, __fsub_rn(s, z)), __fsub_rn(d, z)), 6.283185307179586f, axl);
+        ax = s;
+        x2 = fmaf(R2, 0.0625f * 0.0625f, x2);
+        x3 = fmaf(n3, -0.0625f * 0.0625f * 0.0625f, x3);
+      }
+      // X = exp(-i angle): the negated angle's cosine and sine
+#pragma unroll
+      for (int c8 = 0; c8 < 2; ++c8) {
+        uint32_t rh[4], rl[4], ih[4], il[4];
+#pragma unroll
+        for (int q2 = 0; q2 < 4; ++q2) {
+          const float m0 = (float)(16 * half - 16 + 8 * c8 + 2 * q2);
+          float2 cs, sn;
+          cis2(sep_angle(-ax, ax, -axl, -x2, -x3, -q.x4, make_float2(0.0f, 0.0f), make_float2(m0, m0 + 1.0f)), cs, sn);
+          split_pack(cs, rh[q2], rl[q2]);
+          split_pack(sn, ih[q2], il[q2]);
+        }
+        const int c = 2 * half + c8;
+        put16(ah, row, c, rh);
+        put16(ah, row, 4 + c, ih);
+        put16(ah + kFA, row, c, rl);
+        put16(ah + kFA, row, 4 + c, il);
+      }
+    };
+
+    float scale = 1.0f;
+    int tile = -1;
+    for (uint32_t it = 0;; ++it) {
+      const int d = it & 1;
+      ok = ok && mbar_wait(&listed[it & 3], (it >> 2) & 1, kTcWaitPolls);
+      // MMA(it - 2) done: its A, and B of an older tile, are free
+      if (it >= 2) ok = ok && mbar_wait(&full[d], ((it >> 1) - 1) & 1, kTcWaitPolls);
+      // every generator goes on or none (they meet at a barrier)
+      int stop;
+      asm volatile(
+          "{\n\t.reg .pred p, q;\n\tsetp.eq.s32 p, %1, 0;\n\tbarrier.red.or.pred q, 2, 256, p;\n\t"
+          "selp.s32 %0, 1, 0, q;\n\t}"
+          : "=r"(stop)
+          : "r"((int)ok)
+          : "memory");
+      if (stop) break;
+      const SepStep x = steps[it & 3];
+      if (x.b < 0) {
+        if (g == 0) mbar_arrive(&ready[it & 3]);
+        break;
+      }
+      if (x.tile != tile) {
+        tile = x.tile;
+        scale = build_b(tile, sm + kFwdB + (uint32_t)x.bb * kFwdBuf);
+      }
+      build_a(reinterpret_cast<const float4*>(sm + kFwdSlots + (it & 3) * kFSlot) + row, x,
+              sm + (uint32_t)d * 2 * kFA);
+      fence_async_smem();
+      if (g == 0) scales[it & 3] = scale;
+      gen_sync();
+      if (g == 0) mbar_arrive(&ready[it & 3]);
+    }
+  }
+  if (!ok) atomicOr(p.err, kErrTimeout);
+  tc_fence_before();
+  __syncthreads();
+  if (w == 0) tmem_dealloc(tmem, 512);
+}
+
+// E_n = the sum of the CTAs' partial rows, in a fixed order: row-lane k of the
+// 32 x 32 threads adds rows k, k + 32, ..., then a fixed-shape tree.
+__global__ void k_sep_forward_reduce(const float2* __restrict__ part, int rows, int npad, int N,
+                                     float2* __restrict__ E) {
+  __shared__ float2 acc[32][33];
+  const int n = blockIdx.x * 32 + threadIdx.x, k = threadIdx.y;
+  float2 v = make_float2(0.0f, 0.0f);
+#pragma unroll 10
+  for (int r = k; r < rows; r += 32) {
+    const float2 x = __ldg(part + (size_t)r * npad + n);
+    v.x += x.x;
+    v.y += x.y;
+  }
+  acc[k][threadIdx.x] = v;
+  __syncthreads();
+  for (int h = 16; h > 0; h >>= 1) {
+    if (k < h) {
+      acc[k][threadIdx.x].x += acc[k + h][threadIdx.x].x;
+      acc[k][threadIdx.x].y += acc[k + h][threadIdx.x].y;
+    }
+    __syncthreads();
+  }
+  if (k == 0 && n < N) E[n] = acc[0][threadIdx.x];
+}
+
+}  // namespace
+
+cudaError_t sep_build_table(const Geometry& g, const MonoTerm* terms, const int* term_off, float* tab,
+                            cudaStream_t s) {
+  const long long n = (long long)g.T * g.D;
+  k_sep_table<<<(unsigned)((n + 127) / 128), 128, 0, s>>>(g, terms, term_off, tab);
+  return cudaGetLastError();
+}
+
+cudaError_t sep_build_params(const Geometry& g, const float* tab, const float* coeff, float4* poly,
+                             unsigned char* strips, int* cost, cudaStream_t s) {
+  const int nb = sep_blocks(g.N);
+  k_sep_params<<<dim3(g.T, nb), kSepSpots, 0, s>>>(g, tab, coeff, poly, strips, nb * kSepSpots);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  k_sep_scan<<<1, 1024, 0, s>>>(strips, g.T * nb, cost);
+  return cudaGetLastError();
+}
+
+cudaError_t sep_prepare() {
+  cudaError_t e;
+  if ((e = cudaFuncSetAttribute(k_sep_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFwdSmem))) return e;
+  for (const void* k : {(const void*)k_sep_forward, (const void*)k_sep_forward_reduce, (const void*)k_sep_params})
+    if ((e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                  (int)cudaSharedmemCarveoutMaxShared)))
+      return e;
+  return cudaSuccess;
+}
+
+cudaError_t sep_launch_forward(const SepFwdParams& p, cudaStream_t s) {
+  k_sep_forward<<<p.G, kFwdThreads, kFwdSmem, s>>>(p);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  k_sep_forward_reduce<<<(p.g.N + 31) / 32, dim3(32, 32), 0, s>>>(p.part, kSepFwdRows * p.G, p.nb * kSepSpots, p.g.N, p.E);
+  return cudaGetLastError();
+}
+
+}  // namespace ash
