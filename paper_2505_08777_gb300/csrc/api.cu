@@ -173,17 +173,31 @@ bool use_tc_adj(const ash_hologram* h) {
 }
 // The separable transforms serve the automatic choice for polynomial bases of
 // degree <= 4. The mixed terms of a tile shrink with the square (third order:
-// the cube) of the grid's side; below these sides most tiles need 16 or more
-// row strips and the others are faster (forward, us before / after: 256^2
-// N = 200 D = 10 18 / 40, 384^2 N = 200 D = 11 29 / 35, 512^2 N = 300 D = 10
-// 62 / 40; degree 2, 256^2 N = 100: 15 / 14). A step costs the same however
-// few of its 128 spots are used: with fewer than 64 it pays only where most
-// tiles need one strip (742 x 486 N = 27: 26 / 34; 1024^2 N = 20: 52 / 36).
-constexpr int kSepMinSide = 400, kSepMinSide2 = 200, kSepFewSpots = 64, kSepFewSide = 900;
-bool sep_pays(int ord, int side, int N) {
-  return ord <= 2 ? side >= kSepMinSide2 : side >= (N < kSepFewSpots ? kSepFewSide : kSepMinSide);
+// the cube) of the grid's side; on small sides most tiles need many row strips
+// and the other kernels are faster, the adjoint's sooner (its products cover
+// all rows for every strip). Kernels, us, others / separable: forward, degree
+// 4: 384^2 N = 200 29 / 33, 450^2 N = 200 46 / 36, 512^2 N = 300 62 / 40;
+// adjoint: 450^2 N = 200 53 / 62, 512^2 N = 300 58 / 59, 600^2 N = 200
+// 82 / 49, 901 x 611 N = 230 90 / 85. A forward step and an adjoint tile cost
+// the same however few spots they have: with fewer than 64 they pay only where
+// most tiles need one strip (forward: 742 x 486 N = 27 25 / 33, 1024^2 N = 20
+// 52 / 36). Degree 2 (one mixed term): forward 220^2 N = 30 12.5 / 13.8,
+// 300^2 N = 200 28 / 17; adjoint 256^2 N = 100 13.5 / 16.4, 300^2 N = 200
+// 24 / 20.
+constexpr int kSepSideFwd = 400, kSepSideAdj = 560, kSepSide2 = 200, kSepFewSpots = 64, kSepFewSide = 900;
+constexpr long long kSepTerms2Fwd = 6LL << 20, kSepTerms2Adj = 10LL << 20;
+bool sep_pays(const ash_hologram* h, int side4, long long terms2) {
+  const Geometry& g = h->g;
+  const int side = g.nx < g.ny_full ? g.nx : g.ny_full;
+  if (h->sep_ord <= 2) return side >= kSepSide2 && (long long)g.nx * g.ny * g.N >= terms2;
+  return side >= side4 && (g.N >= kSepFewSpots || side >= kSepFewSide);
 }
-bool use_sep_fwd(const ash_hologram* h) { return h->sep_ok && h->variant == 0; }
+bool use_sep_fwd(const ash_hologram* h) {
+  return h->sep_ok && h->variant == 0 && sep_pays(h, kSepSideFwd, kSepTerms2Fwd);
+}
+bool use_sep_adj(const ash_hologram* h) {
+  return h->sep_ok && h->variant == 0 && sep_pays(h, kSepSideAdj, kSepTerms2Adj);
+}
 // The coefficient-gradient moments on the tensor cores need one K-atom,
 // D <= 12 and a polynomial basis of total degree <= 4 (the tile polynomials);
 // from N = 64, as the forward whose structure they share.
@@ -273,7 +287,8 @@ constexpr int kSrcImg = 2;
 cudaError_t enqueue_tc_coeff(ash_hologram* h, cudaStream_t s) {
   if (!h->tc_ok) return cudaSuccess;
   if (h->sep_ok) {
-    const cudaError_t e = sep_build_params(h->g, h->sep_tab, h->coeff, h->sep_poly, h->sep_strips, h->sep_cost, s);
+    const cudaError_t e = sep_build_params(h->g, h->sep_tab, h->coeff, h->sep_poly, h->sep_strips, h->sep_cost,
+                                           h->sep_acost, s);
     if (e != cudaSuccess) return e;
   }
   return tc_build_coeff(h->g, h->tc_layout, h->coeff, h->anchors, h->czs, h->rot, s);
@@ -310,6 +325,22 @@ SepFwdParams sep_fwd_params(const ash_hologram* h, float2* E) {
   p.E = E;
   p.G = h->sep_G;
   p.err = h->err_word;
+  return p;
+}
+
+TcAdjParams tc_adj_params(const ash_hologram* h, const float2* y, const AdjOut& out);
+SepAdjParams sep_adj_params(const ash_hologram* h, const float2* y, const AdjOut& out) {
+  SepAdjParams p{};
+  p.a = tc_adj_params(h, y, out);
+  p.nb = sep_blocks(h->g.N);
+  p.poly = h->sep_poly;
+  p.strips = h->sep_strips;
+  p.cost = h->sep_acost;
+  p.split = h->sep_split;
+  p.tickets = h->sep_tickets;
+  p.ys = h->sep_ys;
+  p.scale = h->sep_scale;
+  p.G = h->sep_G;
   return p;
 }
 
@@ -390,6 +421,11 @@ ash_status enqueue_adjoint(ash_hologram* h, const float2* y, float2* g_out, floa
   p.out.phase_in = phase_in;
   p.out.dphase = dphase;
   p.out.epilogue = epilogue;
+  if (use_sep_adj(h)) {
+    cudaError_t e = sep_launch_scale(y, h->g.N, h->sep_ys, h->sep_scale, s);
+    if (e == cudaSuccess) e = sep_launch_adjoint(sep_adj_params(h, y, p.out), s);
+    return e == cudaSuccess ? ASH_OK : cuda_fail(e, "separable adjoint launch");
+  }
   if (use_tc_adj(h)) {
     const TcAdjParams tp = tc_adj_params(h, y, p.out);
     cudaError_t e = tc_launch_adjoint(h->tc_na, tp, h->tadj.G, s);
@@ -417,7 +453,7 @@ ash_status enqueue_adjoint(ash_hologram* h, const float2* y, float2* g_out, floa
 // metrics. When both transforms run on the tensor cores the adjoint also
 // writes the next forward's nearfield (kEpiFimg), so only the first forward
 // converts a phase.
-bool wgs_fused_field(const ash_hologram* h) { return (use_sep_fwd(h) || use_tc_fwd(h)) && use_tc_adj(h); }
+bool wgs_fused_field(const ash_hologram* h) { return (use_sep_fwd(h) || use_tc_fwd(h)) && (use_sep_adj(h) || use_tc_adj(h)); }
 
 ash_status enqueue_wgs_body(ash_hologram* h, int iters, cudaStream_t s) {
   const bool tc = wgs_fused_field(h);
@@ -808,9 +844,10 @@ ash_status create_impl(ash_hologram** out, int nx, int ny, int row0, int ny_full
   if (h->tc_ok && spec) {
     int ord = 0;
     for (const MonoTerm& m : spec->terms) ord = m.px + m.py > ord ? m.px + m.py : ord;
-    const int side = nx < ny_full ? nx : ny_full;
-    if (ord <= kSepMaxOrd && sep_pays(ord, side, N)) {
+    h->sep_ord = ord;
+    if (ord <= kSepMaxOrd && (sep_pays(h, kSepSideFwd, kSepTerms2Fwd) || sep_pays(h, kSepSideAdj, kSepTerms2Adj))) {
       ce = sep_prepare();
+      if (ce == cudaSuccess) ce = sep_adjoint_prepare();
       if (ce != cudaSuccess) return fail(cuda_fail(ce, "separable kernel preparation"));
       h->sep_ok = true;
       h->sep_G = sms;
@@ -853,6 +890,11 @@ ash_status create_impl(ash_hologram** out, int nx, int ny, int row0, int ny_full
     if ((st = ws(h, &h->sep_poly, (size_t)g.T * 4 * npad)) != ASH_OK) return fail(st);
     if ((st = ws(h, &h->sep_strips, (size_t)g.T * sep_blocks(N))) != ASH_OK) return fail(st);
     if ((st = ws(h, &h->sep_cost, (size_t)g.T * sep_blocks(N) + 1)) != ASH_OK) return fail(st);
+    if ((st = ws(h, &h->sep_acost, (size_t)g.T * sep_blocks(N) + 2)) != ASH_OK) return fail(st);
+    if ((st = ws(h, &h->sep_split, 2 * (size_t)h->sep_G * kTilePix)) != ASH_OK) return fail(st);
+    if ((st = ws(h, &h->sep_ys, npad)) != ASH_OK) return fail(st);
+    if ((st = ws(h, &h->sep_scale, npad / kSepChunk)) != ASH_OK) return fail(st);
+    if ((st = ws(h, &h->sep_tickets, (size_t)g.T)) != ASH_OK) return fail(st);
     if ((st = ws(h, &h->sep_part, (size_t)kSepFwdRows * h->sep_G * npad)) != ASH_OK) return fail(st);
   }
   if (h->tgrad_ok) {
@@ -939,7 +981,10 @@ ash_status create_impl(ash_hologram** out, int nx, int ny, int row0, int ny_full
     // pixels outside the grid stay 0 in every nearfield image
     CREATE_CUDA(cudaMemsetAsync(h->fimg, 0, tc_fimg_float4s(g) * sizeof(float4), s));
   }
-  if (h->sep_ok) CREATE_CUDA(sep_build_table(g, h->terms, h->term_off, h->sep_tab, s));
+  if (h->sep_ok) {
+    CREATE_CUDA(sep_build_table(g, h->terms, h->term_off, h->sep_tab, s));
+    CREATE_CUDA(cudaMemsetAsync(h->sep_tickets, 0, (size_t)g.T * sizeof(int), s));
+  }
   CREATE_CUDA(enqueue_tc_coeff(h, s));
   k_amp_image<<<g.T, g.NT, 0, s>>>(g, amp, h->amp_img);
   CREATE_CUDA(cudaGetLastError());
@@ -1259,10 +1304,9 @@ int ash_wgs_launches(const ash_hologram* h, int iters) {
   // forward: tensor-core (nearfield image unless fused, kernel, reduce if
   // split) or FMA (kernel, reduction); adjoint: kernel (+ fix-up)
   const bool fused = wgs_fused_field(h);
-  const bool sep = use_sep_fwd(h);
-  const int fwd_first = sep ? 3 : use_tc_fwd(h) ? 2 + (h->tfwd_split ? 1 : 0) : 2;
-  const int fwd = sep ? (fused ? 2 : 3) : use_tc_fwd(h) ? (fused ? 1 : 2) + (h->tfwd_split ? 1 : 0) : 2;
-  const int adj = use_tc_adj(h) ? 1 + (h->tadj_split ? 1 : 0) : 1 + (h->split_tiles ? 1 : 0);
+  const int fwd_first = use_sep_fwd(h) ? 3 : use_tc_fwd(h) ? 2 + (h->tfwd_split ? 1 : 0) : 2;
+  const int fwd = use_sep_fwd(h) ? (fused ? 2 : 3) : use_tc_fwd(h) ? (fused ? 1 : 2) + (h->tfwd_split ? 1 : 0) : 2;
+  const int adj = use_sep_adj(h) ? 2 : use_tc_adj(h) ? 1 + (h->tadj_split ? 1 : 0) : 1 + (h->split_tiles ? 1 : 0);
   return fwd_first + iters * (1 + adj + fwd) + 1;   // + metrics
 }
 

@@ -64,11 +64,17 @@ struct ash_hologram {
   float* tpoly = nullptr;       // tile polynomials of the basis
   // separable tile transforms (polynomial bases of total degree <= 4)
   bool sep_ok = false;
+  int sep_ord = 0;              // total degree of the basis
   int sep_G = 0;                // forward CTAs
   float* sep_tab = nullptr;     // basis polynomials per tile
   float4* sep_poly = nullptr;   // phase polynomials per (tile, spot)
   unsigned char* sep_strips = nullptr;   // per (tile, spot block): log2 of its row strips
-  int* sep_cost = nullptr;      // prefix of its steps' cost
+  int* sep_cost = nullptr;      // prefix of its forward steps' cost
+  int* sep_acost = nullptr;     // prefix of its adjoint chunks' cost
+  float2* sep_split = nullptr;  // [sep_G][2][kTilePix] adjoint sums of tiles split between CTAs
+  int* sep_tickets = nullptr;   // [T]
+  float2* sep_ys = nullptr;     // [128 nb] y of an adjoint, scaled, and the scale per 32 spots
+  float* sep_scale = nullptr;
   float2* sep_part = nullptr;   // [kSepFwdRows sep_G][128 nb]
   float2* split = nullptr;
   float* gradc_partial = nullptr;

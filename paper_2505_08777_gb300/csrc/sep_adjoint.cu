@@ -1,0 +1,450 @@
+// Separable adjoint transform (see sep_common.cuh): over a tile
+//
+//   g(u, v) = sum_k u^k sum_n [y_n Y_n(v) Q_k,n(v)] X_n(u),
+//
+// the inner sum a matrix product over the spots. W = y Y Q_k and X are
+// written by the warps as split-f16 operands; the tensor core contracts 32
+// spots per step, and the partial products are added up in fp32 registers.
+#include "sep_common.cuh"
+#include "tc_epilogue.cuh"
+
+namespace ash {
+
+namespace {
+
+// One CTA per SM, 28 warps. Warps 0-7 (adders): lane = tile row, warp w adds
+// up half of the columns of the plane u^(w % 4); warp 8 issues the MMAs, warp
+// 9 lists the steps and fetches their spots; warps 12-19 and 20-27
+// (generators, taking turns step by step): lane = spot, four tile rows and
+// four tile columns each. A step is 32 spots of a tile and one strip of its
+// rows (the strips of a chunk share W). A: rows (k, tile row), (Re W, Im W) of
+// the 32 spots; low parts for k = 0, 1 only (|Q_2|, |Q_3| < 0.01). B: rows
+// (column, re / im), (Re X, -Im X) and (Im X, Re X), high then low parts.
+// D[128][128]: products with the high and with the low parts of X.
+constexpr int kAdjThreads = 896;
+// Registers: launched with 72 a thread; the adders keep 72, warps 8-11 drop
+// to 40, the generators take 80.
+static_assert(2 * 72 + 40 + 4 * 80 <= 7 * 72);
+constexpr int kAdjBufs = 3, kAdjSlots = 8;
+constexpr uint32_t kAA = 32768, kAB = 16384, kASlot = 2048 + 256;
+constexpr uint32_t kAdjB = kAdjBufs * kAA, kAdjSum = kAdjB + kAdjBufs * kAB;   // sums of the planes: [4][32][33] float2
+constexpr uint32_t kAdjSlot0 = kAdjSum + 4 * 32 * 33 * 8, kAdjTail = kAdjSlot0 + kAdjSlots * kASlot;
+constexpr size_t kAdjSmem = 1024 + kAdjTail + 512;
+static_assert(28 * 8 + 16 + kAdjSlots * 24 <= 512);
+static_assert(kAdjSum % 16 == 0 && kAdjSlot0 % 16 == 0 && kAdjTail % 8 == 0);
+
+struct AdjStep {
+  int tile;      // -1: no more steps
+  int s, ls;     // strip s of 2^ls
+  int a;         // buffer of W
+  int end;       // bits: 1 the CTA's last step of this tile, 2 other CTAs have part of it, 4 it starts here
+  float scale;   // 2^e: y is divided by it
+};
+
+// (see kTruncation of the forward: here -1.5e-7)
+constexpr float kAdjTruncation = 1.0f + 1.2e-7f;
+
+template <int V>
+struct IntTag {
+  static constexpr int value = V;
+};
+template <int OFF>
+__device__ __forceinline__ void sts32(uint32_t addr, uint32_t v) {
+  asm volatile("st.shared.u32 [%0 + %1], %2;" ::"r"(addr), "n"(OFF), "r"(v) : "memory");
+}
+
+// CTA whose range [W g / G, W (g + 1) / G) holds position c.
+__device__ __forceinline__ int adj_owner(long long W, int G, int c) {
+  int g = (int)((long long)c * G / W);
+  while (g + 1 < G && W * (g + 1) / G <= c) ++g;
+  while (g > 0 && W * g / G > c) --g;
+  return g;
+}
+
+__global__ void __launch_bounds__(kAdjThreads, 1) k_sep_adjoint(const SepAdjParams p) {
+  extern __shared__ uint8_t raw[];
+  uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(raw) + 1023) & ~(uintptr_t)1023);
+  uint64_t* full = reinterpret_cast<uint64_t*>(sm + kAdjTail);   // [4] MMAs of a step done
+  uint64_t* empty = full + 4;                                    // [8] its D and record read
+  uint64_t* ready = full + 12;                                   // [8] its operands written
+  uint64_t* listed = full + 20;                                  // [8] its record and spots written
+  uint32_t* slot = reinterpret_cast<uint32_t*>(full + 28);
+  AdjStep* steps = reinterpret_cast<AdjStep*>(slot + 4);         // [8]
+  const int t = threadIdx.x, w = t >> 5, lane = t & 31;
+  const int N = p.a.g.N, nb = p.nb, npad = nb * kSepSpots, U = p.a.g.T * nb;
+  // rows k = 2, 3 of W's low parts stay zero
+  for (int k = t; k < kAdjBufs * 512; k += kAdjThreads)
+    reinterpret_cast<uint4*>(sm + (k >> 9) * kAA + 16384 + 8192)[k & 511] = make_uint4(0, 0, 0, 0);
+  if (w == 0) tmem_alloc(slot, 512);
+  if (t == 0) {
+    for (int k = 0; k < 28; ++k) mbar_init(full + k, k >= 4 && k < 12 ? 8 : 1);
+    fence_mbar_init();
+  }
+  fence_async_smem();
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *slot;
+  bool ok = true;
+  const long long W = p.cost[U];
+  // ranges no shorter than a chunk, so that every CTA of a split tile has one
+  const int G = (int)max(1LL, min((long long)p.G, W / p.cost[U + 1]));
+
+  if (w < 8) {
+    // --- adders: plane u^pl of tile row `lane`, columns 16 hc .. 16 hc + 15 ---
+    const int pl = w & 3, hc = w >> 2;
+    const uint32_t ta = tmem + ((uint32_t)(pl * 32) << 16) + 32u * hc;
+    float2* sums = reinterpret_cast<float2*>(sm + kAdjSum);
+    auto add_sync = [&]() { asm volatile("bar.sync 1, 256;" ::: "memory"); };
+    float2 acc[16];
+#pragma unroll
+    for (int i = 0; i < 16; ++i) acc[i] = make_float2(0.0f, 0.0f);
+    for (uint32_t it = 0;; ++it) {
+      const int sl = it & 7, d = it & 3;
+      ok = ok && mbar_wait(&listed[sl], (it >> 3) & 1, kTcWaitPolls);
+      AdjStep x{-1, 0, 0, 0, 0, 0.0f};
+      if (ok) x = steps[sl];
+      if (x.tile >= 0) ok = mbar_wait(&full[d], (it >> 2) & 1, kTcWaitPolls) && ok;
+      // the eight warps go on or stop together
+      int stop;
+      asm volatile(
+          "{\n\t.reg .pred p, q;\n\tsetp.lt.s32 p, %1, 0;\n\tbarrier.red.or.pred q, 1, 256, p;\n\t"
+          "selp.s32 %0, 1, 0, q;\n\t}"
+          : "=r"(stop)
+          : "r"(ok ? x.tile : -1)
+          : "memory");
+      if (stop) break;
+      tc_fence_after();
+      const int n = 32 >> x.ls;
+      const float f = (lane >= x.s * n && lane < (x.s + 1) * n) ? x.scale : 0.0f;
+#pragma unroll
+      for (int h = 0; h < 4; ++h) {
+        uint32_t a[8], b[8];
+        tmem_ld8_nowait(ta + (uint32_t)(128 * d + 8 * h), a);
+        tmem_ld8_nowait(ta + (uint32_t)(128 * d + 64 + 8 * h), b);
+        tmem_wait();
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const float2 v = add2(make_float2(__uint_as_float(a[2 * i]), __uint_as_float(a[2 * i + 1])),
+                                make_float2(__uint_as_float(b[2 * i]), __uint_as_float(b[2 * i + 1])));
+          acc[4 * h + i] = fma2(v, dup2(f), acc[4 * h + i]);
+        }
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&empty[sl]);
+      if (!x.end) continue;
+      // sum of the planes; then thread: pixels (row q * 8 + w, column lane)
+      float2* mine = sums + (size_t)(pl * 32 + lane) * 33 + 16 * hc;
+#pragma unroll
+      for (int i = 0; i < 16; ++i) {
+        const float u = (float)(16 * hc + i - 16) * 0.0625f;
+        const float c = (pl & 1 ? u : 1.0f) * (pl & 2 ? u * u : 1.0f) * kAdjTruncation;
+        mine[i] = mul2(acc[i], dup2(c));
+        acc[i] = make_float2(0.0f, 0.0f);
+      }
+      add_sync();
+      const TcAdjParams& o = p.a;
+      const Geometry& g = o.g;
+      const int tx = x.tile % g.tiles_x, ty = x.tile / g.tiles_x;
+      const int pi = tx * kTileX + lane, pj = ty * kTileY + w;   // pixel of q = 0; rows 8 apart
+      float2 v[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const float2* s = sums + (size_t)(8 * q + w) * 33 + lane;
+        v[q] = add2(add2(s[0], s[32 * 33]), add2(s[2 * 32 * 33], s[3 * 32 * 33]));
+      }
+      bool out = true;
+      if (x.end & 2) {
+        // a split tile: the last of its CTAs adds up the partial sums (a
+        // CTA's second buffer is that of the tile that starts in it)
+        float2* dst = p.split + ((size_t)blockIdx.x * 2 + (x.end & 4 ? 1 : 0)) * kTilePix + w * 32 + lane;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) dst[q * 256] = v[q];
+        __threadfence();
+        add_sync();
+        int* flag = reinterpret_cast<int*>(slot + 1);   // [2]: the tile's first CTA if this is the last to come, its last CTA
+        if (t == 0) {
+          const int u0 = x.tile * nb, u1 = u0 + nb;
+          const int g_lo = adj_owner(W, G, p.cost[u0]);
+          const int g_hi = adj_owner(W, G, p.cost[u1] - sep_chunk_cost(p.strips[u1 - 1]));
+          const bool last = atomicAdd(&p.tickets[x.tile], 1) == g_hi - g_lo;
+          if (last) p.tickets[x.tile] = 0;
+          flag[0] = last ? g_lo : -1;
+          flag[1] = g_hi;
+        }
+        add_sync();
+        const int g_lo = flag[0], g_hi = flag[1];
+        out = g_lo >= 0;
+        if (out) {
+          __threadfence();
+#pragma unroll
+          for (int q = 0; q < 4; ++q) v[q] = make_float2(0.0f, 0.0f);
+          for (int k = g_lo; k <= g_hi; ++k) {
+            const float2* src = p.split + ((size_t)k * 2 + (k == g_lo ? 1 : 0)) * kTilePix + w * 32 + lane;
+            float2 r[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) r[q] = __ldcg(src + q * 256);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) v[q] = add2(v[q], r[q]);
+          }
+        }
+      }
+      if (out && pi < g.nx) {
+        float amp[4] = {};
+        if (o.out.epilogue & (kEpiGradPhase | kEpiFimg)) {
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            amp[q] = __ldg(o.amp_img + tc_pixel(g, (long long)x.tile * kTcChunksPerTile + 4 * q + (w >> 1), (w & 1) * 32 + lane).img);
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int j = pj + 8 * q;
+          if (j >= g.ny) break;
+          adjoint_epilogue(o.out, (size_t)j * g.nx + pi, v[q].x, v[q].y, amp[q]);
+          if (o.out.epilogue & kEpiFimg) {
+            const float ph = (v[q].x == 0.0f && v[q].y == 0.0f) ? 0.0f : atan2f(v[q].y, v[q].x) * 0.15915494309189535f;
+            // row 8 q + w of the tile, column lane
+            float* f = reinterpret_cast<float*>(o.fimg + ((size_t)x.tile * kTcChunksPerTile + 4 * q + (w >> 1)) * 32 +
+                                                (w & 1) * 16 + (lane >> 1)) + (lane & 1);
+            f[0] = amp[q];
+            f[2] = ph;
+          }
+        }
+      }
+      add_sync();   // `sums` is rewritten at the next tile's end
+    }
+  } else if (w < 12) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
+    if (w == 8 && lane == 0) {
+      // --- MMA issue ---
+      uint32_t it = 0, bi = 0;
+      for (;; ++it, bi = bi == kAdjBufs - 1 ? 0 : bi + 1) {
+        const int sl = it & 7, d = it & 3;
+        ok = ok && mbar_wait(&listed[sl], (it >> 3) & 1, kTcWaitPolls);
+        if (!ok) break;
+        const AdjStep x = steps[sl];
+        if (x.tile < 0) break;
+        ok = ok && mbar_wait(&ready[sl], (it >> 3) & 1, kTcWaitPolls);
+        if (it >= 4) ok = ok && mbar_wait(&empty[(it - 4) & 7], ((it - 4) >> 3) & 1, kTcWaitPolls);
+        if (!ok) break;
+        tc_fence_after();
+        const uint32_t dst = tmem + 128u * d;
+        const uint64_t a = umma_desc(smem_u32(sm) + (uint32_t)x.a * kAA), al = a + (16384 >> 4);
+        const uint64_t b = umma_desc(smem_u32(sm + kAdjB) + bi * kAB);
+#pragma unroll
+        for (int ks = 0; ks < 8; ks += 2) umma_f16(dst, a + ks, b + ks, umma_idesc_f16(128, 128), ks > 0);
+#pragma unroll
+        for (int ks = 0; ks < 8; ks += 2) umma_f16(dst + 64, al + ks, b + ks, umma_idesc_f16(128, 64), 1u);
+        umma_commit(&full[d]);
+      }
+      // nothing in flight when the CTA gives up its memory
+      for (uint32_t k = it > 3 ? it - 3 : 0; k < it; ++k) ok = mbar_wait(&full[k & 3], (k >> 2) & 1, kTcWaitPolls) && ok;
+    } else if (w == 9 && lane == 0) {
+      // --- steps of this CTA: the chunks whose place in the cost prefix lies in [c0, c1) ---
+      const int c0 = blockIdx.x < G ? (int)(W * blockIdx.x / G) : 0;
+      const int c1 = blockIdx.x < G ? (int)(W * (blockIdx.x + 1) / G) : 0;
+      int u = 0, hi = U - 1;
+      while (u < hi) {
+        const int mid = (u + hi + 1) / 2;
+        if (p.cost[mid] <= c0) u = mid;
+        else hi = mid - 1;
+      }
+      int tile = u / nb, b = u % nb, ls = p.strips[u], pos = p.cost[u];
+      int cc = sep_chunk_cost(ls), c = (c0 - pos + cc - 1) / cc, s = 0, a = 0;
+      pos += c * cc;
+      int ls1 = u + 1 < U ? p.strips[u + 1] : 0;   // of the next unit, fetched early
+      uint32_t it = 0;
+      for (;; ++it) {
+        const int sl = it & 7;
+        if (s == 0 && c == sep_chunks(N, b)) {
+          c = 0;
+          ++u;
+          ls = ls1;
+          cc = sep_chunk_cost(ls);
+          if (++b == nb) {
+            b = 0;
+            ++tile;
+          }
+          if (u + 1 < U) ls1 = p.strips[u + 1];
+        }
+        const bool more = s > 0 || pos < c1;
+        const int chunk = b * (kSepSpots / kSepChunk) + c;
+        const float sc = more ? __ldg(p.scale + chunk) : 0.0f;
+        if (it >= 8) ok = ok && mbar_wait(&empty[sl], ((it >> 3) - 1) & 1, kTcWaitPolls);
+        if (!more) {
+          // an end for each of the two groups of generators
+          steps[sl] = AdjStep{-1, 0, 0, 0, 0, 0.0f};
+          mbar_arrive(&listed[sl]);
+          const int s2 = (it + 1) & 7;
+          if (it >= 7) ok = ok && mbar_wait(&empty[s2], (((it + 1) >> 3) - 1) & 1, kTcWaitPolls);
+          steps[s2] = AdjStep{-1, 0, 0, 0, 0, 0.0f};
+          mbar_arrive(&listed[s2]);
+          break;
+        }
+        uint8_t* dst = sm + kAdjSlot0 + sl * kASlot;
+        AdjStep x{tile, s, ls, a, 0, sc};
+        if (((s + 1) >> ls) && (pos + cc >= c1 || (c + 1 == sep_chunks(N, b) && b + 1 == nb))) {
+          const int t1 = p.cost[(tile + 1) * nb] - sep_chunk_cost(p.strips[(tile + 1) * nb - 1]);
+          const bool here = c0 <= p.cost[tile * nb];
+          x.end = 1 | (here && t1 < c1 ? 0 : 2) | (here ? 4 : 0);
+        }
+        steps[sl] = x;
+        mbar_expect_tx(&listed[sl], kASlot);
+        bulk_g2s(dst, p.poly + ((size_t)tile * (npad / kSepChunk) + chunk) * 128, 2048, &listed[sl]);
+        bulk_g2s(dst + 2048, p.ys + chunk * kSepChunk, 256, &listed[sl]);
+        if (++s >> ls) {
+          s = 0;
+          ++c;
+          pos += cc;
+          a = a == kAdjBufs - 1 ? 0 : a + 1;
+        }
+      }
+      for (uint32_t k = it > 6 ? it - 6 : 0; k < it; ++k) ok = mbar_wait(&listed[k & 7], (k >> 3) & 1, kTcWaitPolls) && ok;
+    }
+  } else {
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 80;");
+    // --- generators: spot `lane`, tile rows and columns 4 gw .. 4 gw + 3 ---
+    const int group = (w - 12) >> 3, gw = (w - 12) & 7;
+    // The spot's 4 bytes in a row r (r = 8 a + e) of a 128-byte-swizzled operand
+    // lie at row + (place ^ (e << 4)). W: rows k 32 + 4 gw + c, X: rows 8 gw + e.
+    const uint32_t place = (uint32_t)lane * 4;
+    const uint32_t w0 = smem_u32(sm) + (uint32_t)gw * 512 + (place ^ ((uint32_t)(gw & 1) << 6));
+    const uint32_t x0 = smem_u32(sm + kAdjB) + (uint32_t)gw * 1024 + place;
+    uint32_t bi = group;
+    for (uint32_t it = group;; it += 2, bi = bi == 0 ? 2 : bi - 1) {
+      const int sl = it & 7;
+      ok = ok && mbar_wait(&listed[sl], (it >> 3) & 1, kTcWaitPolls);
+      // the MMAs of step it - 3 are done: its X, and W of an older chunk, are free
+      if (it >= 3) ok = ok && mbar_wait(&full[(it - 3) & 3], ((it - 3) >> 2) & 1, kTcWaitPolls);
+      AdjStep x{-1, 0, 0, 0, 0, 0.0f};
+      if (ok) x = steps[sl];
+      if (x.tile >= 0) {
+        const float4* sq = reinterpret_cast<const float4*>(sm + kAdjSlot0 + sl * kASlot) + lane;
+        const SepPoly q = sep_unpack(sq[0], sq[32], sq[64], sq[96]);
+        if (x.s == 0) {
+          const float2 y = reinterpret_cast<const float2*>(sm + kAdjSlot0 + sl * kASlot + 2048)[lane];
+          const uint32_t ah = w0 + (uint32_t)x.a * kAA;
+#pragma unroll
+          for (int pr = 0; pr < 2; ++pr) {
+          const int j = 4 * gw + 2 * pr;
+          const float2 m = make_float2((float)(j - 16), (float)(j - 15));
+          // the rows' strip: its middle row carries the mixed terms of X
+          const int n = 32 >> x.ls;
+          const float ms = strip_mid(j / n, x.ls), ms1 = strip_mid((j + 1) / n, x.ls);
+          const float2 mid = make_float2(ms, ms1);
+          auto R1of = [&](float2 v) { return mul2(fma2(fma2(dup2(q.c13), v, dup2(q.c12)), v, dup2(q.c11)), v); };
+          auto R2of = [&](float2 v) { return mul2(fma2(dup2(q.c22), v, dup2(q.c21)), v); };
+          float2 R1 = R1of(m), R2 = R2of(m), n3 = mul2(dup2(q.n31), m);
+          if (x.ls) {
+            R1 = fma2(R1of(mid), dup2(-1.0f), R1);
+            R2 = fma2(R2of(mid), dup2(-1.0f), R2);
+            n3 = fma2(dup2(-q.n31), mid, n3);
+          }
+          // exp(+i r) = 1 + i R1 u + (q2r + i q2i) u^2 + (q3r + i q3i) u^3
+          const float2 s2 = mul2(R1, R1), n1 = mul2(R1, dup2(-1.0f));
+          const float2 q2r = fma2(s2, fma2(s2, dup2(1.0f / 24.0f), dup2(-0.5f)), mul2(R2, mul2(R2, dup2(-0.5f))));
+          const float2 q2i = mul2(R2, fma2(s2, dup2(-0.5f), dup2(1.0f)));
+          const float2 q3r = mul2(n1, R2), n3i = fma2(mul2(R1, s2), dup2(1.0f / 6.0f), n3);   // -q3i
+          float2 c, sn;
+          cis2(sep_angle(q.ay, -q.ay, q.ayl, q.y2, q.y3, q.y4, q.base, -q.base, m), c, sn);
+          // (a complex product: the phase of y, carried from iteration to iteration
+          // by a WGS loop, keeps its fp32 accuracy)
+          const float2 wr = fma2(sn, dup2(-y.y), mul2(c, dup2(y.x))), wi = fma2(c, dup2(y.y), mul2(sn, dup2(y.x)));
+          // rows c = 2 pr, 2 pr + 1 of the thread's four
+          const uint32_t r0 = ah ^ (uint32_t)(pr << 5), r1 = ah ^ (uint32_t)(pr << 5 | 16);
+          auto emit = [&](auto kk, float2 re, float2 im) {
+            constexpr int k = decltype(kk)::value;
+            constexpr int o0 = k * 4096, lo = 16384;
+            if constexpr (k < 2) {
+              const float2 hr = split_hi2(re), hi = split_hi2(im);
+              const float2 lr = fma2(hr, dup2(-1.0f), re), li = fma2(hi, dup2(-1.0f), im);
+              sts32<o0>(r0 + 256 * pr, pack_f16(hr.x, hi.x));
+              sts32<o0 + 128>(r1 + 256 * pr, pack_f16(hr.y, hi.y));
+              sts32<o0 + lo>(r0 + 256 * pr, pack_f16(lr.x, li.x));
+              sts32<o0 + lo + 128>(r1 + 256 * pr, pack_f16(lr.y, li.y));
+            } else {
+              sts32<o0>(r0 + 256 * pr, pack_f16(re.x, im.x));
+              sts32<o0 + 128>(r1 + 256 * pr, pack_f16(re.y, im.y));
+            }
+          };
+          emit(IntTag<0>{}, wr, wi);
+          emit(IntTag<1>{}, mul2(n1, wi), mul2(R1, wr));
+          const float2 nwi = mul2(wi, dup2(-1.0f));
+          emit(IntTag<2>{}, fma2(q2r, wr, mul2(q2i, nwi)), fma2(q2r, wi, mul2(q2i, wr)));
+          emit(IntTag<3>{}, fma2(q3r, wr, mul2(n3i, wi)), fma2(q3r, wi, mul2(n3i, mul2(wr, dup2(-1.0f)))));
+          }
+        }
+        const SepColumns o = sep_columns(q, x.s, x.ls);
+        const uint32_t bh = x0 + bi * kAB;
+        constexpr uint32_t S = 0x80000000u;   // the sign of the upper half
+#pragma unroll
+        for (int pr = 0; pr < 2; ++pr) {
+          const int i = 4 * gw + 2 * pr;
+          const float2 m = make_float2((float)(i - 16), (float)(i - 15));
+          float2 c, sn;
+          cis2(sep_angle(o.ax, -o.ax, o.axl, o.x2, o.x3, o.x4, m), c, sn);
+          const float2 hc = split_hi2(c), hs = split_hi2(sn);
+          const float2 lc = fma2(hc, dup2(-1.0f), c), ls = fma2(hs, dup2(-1.0f), sn);
+          // rows e = 4 pr .. 4 pr + 3: (re, im) of column i, then of i + 1
+          const uint32_t b0 = (bh ^ (uint32_t)(pr << 6)) + 512 * pr;
+          sts32<0>(b0, pack_f16(hc.x, hs.x) ^ S);
+          sts32<128>(b0 ^ 16u, pack_f16(hs.x, hc.x));
+          sts32<256>(b0 ^ 32u, pack_f16(hc.y, hs.y) ^ S);
+          sts32<384>(b0 ^ 48u, pack_f16(hs.y, hc.y));
+          sts32<8192>(b0, pack_f16(lc.x, ls.x) ^ S);
+          sts32<8192 + 128>(b0 ^ 16u, pack_f16(ls.x, lc.x));
+          sts32<8192 + 256>(b0 ^ 32u, pack_f16(lc.y, ls.y) ^ S);
+          sts32<8192 + 384>(b0 ^ 48u, pack_f16(ls.y, lc.y));
+        }
+        fence_async_smem();
+      }
+      // all generators go on or stop together
+      int stop;
+      asm volatile(
+          "{\n\t.reg .pred p, q;\n\tsetp.lt.s32 p, %1, 0;\n\tbarrier.red.or.pred q, %2, 256, p;\n\t"
+          "selp.s32 %0, 1, 0, q;\n\t}"
+          : "=r"(stop)
+          : "r"(x.tile), "r"(2 + group)
+          : "memory");
+      if (gw == 0 && lane == 0 && ok) mbar_arrive(&ready[sl]);
+      if (stop) break;
+    }
+  }
+  if (!ok) atomicOr(p.a.err, kErrTimeout);
+  tc_fence_before();
+  __syncthreads();
+  if (w == 0) tmem_dealloc(tmem, 512);
+}
+
+// One warp per chunk of 32 spots.
+__global__ void k_sep_scale(const float2* __restrict__ y, int N, int chunks, float2* __restrict__ ys,
+                            float* __restrict__ scale) {
+  const int c = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
+  if (c < chunks) sep_scale_chunk(y, N, c, ys, scale);
+}
+
+}  // namespace
+
+cudaError_t sep_launch_scale(const float2* y, int N, float2* ys, float* scale, cudaStream_t s) {
+  const int chunks = sep_blocks(N) * (kSepSpots / kSepChunk);
+  k_sep_scale<<<(chunks + 3) / 4, 128, 0, s>>>(y, N, chunks, ys, scale);
+  return cudaGetLastError();
+}
+
+cudaError_t sep_adjoint_prepare() {
+  cudaError_t e = cudaFuncSetAttribute(k_sep_adjoint, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kAdjSmem);
+  if (e != cudaSuccess) return e;
+  for (const void* k : {(const void*)k_sep_adjoint, (const void*)k_sep_scale})
+    if ((e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                  (int)cudaSharedmemCarveoutMaxShared)))
+      return e;
+  return cudaSuccess;
+}
+
+cudaError_t sep_launch_adjoint(const SepAdjParams& p, cudaStream_t s) {
+  k_sep_adjoint<<<p.G, kAdjThreads, kAdjSmem, s>>>(p);
+  return cudaGetLastError();
+}
+
+}  // namespace ash

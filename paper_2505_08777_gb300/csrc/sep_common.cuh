@@ -85,7 +85,7 @@ __device__ __forceinline__ uint32_t swz_chunk(int r, int c) { return (uint32_t)(
 // A (tile, spot)'s phase polynomial as stored by k_sep_params, in the pixel
 // offsets mx = col - 16, my = row - 16 from the tile's pixel (16, 16).
 struct SepPoly {
-  float base;                  // at that pixel, radians, about [-pi, pi]
+  float base;                  // at that pixel, turns, about [-1/2, 1/2]
   float ax, ay;                // turns per pixel along columns and rows,
   float axl, ayl;              // and what their rounding left, radians
   float x2, x3, x4;            // mx^2, mx^3, mx^4, radians
@@ -112,7 +112,9 @@ __device__ __forceinline__ SepPoly sep_unpack(float4 a, float4 b, float4 c, floa
   return p;
 }
 
-// sin and cos of two angles of at most about 2 pi through the MUFU.
+// sin and cos of two angles through the MUFU. Its error is a phase error of
+// -7.5e-8 of the angle (besides the random part), so the angles are kept to
+// [-pi, pi] and a little.
 __device__ __forceinline__ void cis2(float2 x, float2& c, float2& s) {
   s.x = __sinf(x.x);
   c.x = __cosf(x.x);
@@ -120,15 +122,72 @@ __device__ __forceinline__ void cis2(float2 x, float2& c, float2& s) {
   c.y = __cosf(x.y);
 }
 
-// The angles base + 2 pi a m + m (al + q2 m + q3 m^2 + q4 m^3), less a whole
-// number of turns of a m, for two offsets m; a - rint(a m) / m is exact. `na`
-// is -a (the packed operations take no sign).
-__device__ __forceinline__ float2 sep_angle(float a, float na, float al, float q2, float q3, float q4, float2 base,
-                                            float2 m) {
-  const float2 k = add2(fma2(dup2(na), m, dup2(12582912.0f)), dup2(-12582912.0f));   // -rint(a m)
+// The angles 2 pi (a m + b) + m (al + q2 m + q3 m^2 + q4 m^3), less whole turns
+// of a m + b, for two offsets m; a m less an integer is exact. `na`, `nb` are
+// -a, -b (the packed operations take no sign). b is in turns, |b| <= 1.
+__device__ __forceinline__ float2 sep_angle(float a, float na, float al, float q2, float q3, float q4, float b,
+                                            float nb, float2 m) {
+  const float2 k = add2(add2(fma2(dup2(na), m, dup2(nb)), dup2(12582912.0f)), dup2(-12582912.0f));   // -rint(a m + b)
+  const float2 r = add2(fma2(dup2(a), m, k), dup2(b));
+  const float2 q = fma2(fma2(fma2(dup2(q4), m, dup2(q3)), m, dup2(q2)), m, dup2(al));
+  return fma2(r, dup2(6.283185307179586f), mul2(q, m));
+}
+// The same with b = 0.
+__device__ __forceinline__ float2 sep_angle(float a, float na, float al, float q2, float q3, float q4, float2 m) {
+  const float2 k = add2(fma2(dup2(na), m, dup2(12582912.0f)), dup2(-12582912.0f));
   const float2 r = fma2(dup2(a), m, k);
   const float2 q = fma2(fma2(fma2(dup2(q4), m, dup2(q3)), m, dup2(q2)), m, dup2(al));
-  return fma2(r, dup2(6.283185307179586f), fma2(q, m, base));
+  return fma2(r, dup2(6.283185307179586f), mul2(q, m));
+}
+
+// Offset my of a strip's middle row (0 for the whole tile).
+__device__ __forceinline__ float strip_mid(int s, int ls) {
+  const int n = 32 >> ls;
+  return ls == 0 ? 0.0f : (float)(s * n - 16) + 0.5f * (float)(n - 1);
+}
+
+__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+
+// Two values split into f16 pairs (hi, lo).
+__device__ __forceinline__ void split_pack(float2 v, uint32_t& hi, uint32_t& lo) {
+  const float2 h = split_hi2(v), l = fma2(h, dup2(-1.0f), v);
+  hi = pack_f16(h.x, h.y);
+  lo = pack_f16(l.x, l.y);
+}
+
+// A spot's column polynomials about a strip's middle row (the mixed terms
+// there are phases of the column part).
+struct SepColumns {
+  float ax, axl, x2, x3, x4;
+};
+__device__ __forceinline__ SepColumns sep_columns(const SepPoly& q, int s, int ls) {
+  SepColumns o{q.ax, q.axl, q.x2, q.x3, q.x4};
+  if (ls) {
+    const float ms = strip_mid(s, ls);
+    const float R1 = ms * (q.c11 + ms * (q.c12 + ms * q.c13)), R2 = ms * (q.c21 + ms * q.c22), n3 = ms * q.n31;
+    const float d = R1 * (0.15915494309189535f * 0.0625f);
+    const float a = __fadd_rn(q.ax, d), z = __fsub_rn(a, q.ax);
+    o.axl = fmaf(__fadd_rn(__fsub_rn(q.ax, __fsub_rn(a, z)), __fsub_rn(d, z)), 6.283185307179586f, q.axl);
+    o.ax = a;
+    o.x2 = fmaf(R2, 0.0625f * 0.0625f, q.x2);
+    o.x3 = fmaf(n3, -0.0625f * 0.0625f * 0.0625f, q.x3);
+  }
+  return o;
+}
+
+// y of the 32 spots of a chunk divided by a power of two (scale), so that
+// |y| <= 1; by one warp.
+__device__ __forceinline__ void sep_scale_chunk(const float2* __restrict__ y, int N, int c, float2* __restrict__ ys,
+                                                float* __restrict__ scale) {
+  const int lane = threadIdx.x & 31, n = c * 32 + lane;
+  const float2 v = n < N ? __ldg(y + n) : make_float2(0.0f, 0.0f);
+  const uint32_t mx = __reduce_max_sync(0xffffffffu, __float_as_uint(hypotf(v.x, v.y)));
+  const int e = min(max((int)(mx >> 23), 27), 227) - 126;
+  const float inv = __uint_as_float((uint32_t)(127 - e) << 23);
+  ys[c * 32 + lane] = make_float2(v.x * inv, v.y * inv);
+  if (lane == 0) scale[c] = __uint_as_float((uint32_t)(127 + e) << 23);
 }
 
 }  // namespace ash

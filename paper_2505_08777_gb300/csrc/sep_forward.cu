@@ -105,14 +105,14 @@ __global__ void __launch_bounds__(kSepSpots) k_sep_params(const Geometry G, cons
     axh = x;
     ayh = y;
   }
-  // radians per pixel offset (u = mx / 16, v = my / 16)
+  // per pixel offset (u = mx / 16, v = my / 16); the powers in radians
   constexpr float tp = 6.283185307179586f, h = 0.0625f;
-  const size_t o = (size_t)tile * 4 * npad + n;
-  poly[o] = make_float4(tp * base, axh, ayh, __uint_as_float(pack_bf16_rz(tp * axl, tp * ayl)));
-  poly[o + npad] = make_float4(tp * q[0] * (h * h), tp * q[1] * (h * h * h), tp * q[2] * (h * h * h * h),
+  const size_t o = ((size_t)tile * (npad / 32) + (n >> 5)) * 128 + (n & 31);
+  poly[o] = make_float4(base, axh, ayh, __uint_as_float(pack_bf16_rz(tp * axl, tp * ayl)));
+  poly[o + 32] = make_float4(tp * q[0] * (h * h), tp * q[1] * (h * h * h), tp * q[2] * (h * h * h * h),
                                tp * q[3] * (h * h));
-  poly[o + 2 * (size_t)npad] = make_float4(tp * q[4] * (h * h * h), tp * q[5] * (h * h * h * h), q[6] * h, q[7] * h);
-  poly[o + 3 * (size_t)npad] = make_float4(q[8] * (h * h), q[9] * (h * h), -q[10] * h, q[11] * (h * h * h));
+  poly[o + 64] = make_float4(tp * q[4] * (h * h * h), tp * q[5] * (h * h * h * h), q[6] * h, q[7] * h);
+  poly[o + 96] = make_float4(q[8] * (h * h), q[9] * (h * h), -q[10] * h, q[11] * (h * h * h));
   // Row strips: the cubic in u takes u^4 R1^4 / 24 etc. as u^2 (off by at most
   // 1/4) and drops the rest; with 2^k strips R_k about a strip's middle row is
   // at most |dR_k/dv| / 2^k. The fewest strips that drop less than kSepTol.
@@ -137,20 +137,35 @@ __global__ void __launch_bounds__(kSepSpots) k_sep_params(const Geometry G, cons
   if (t == 0) strips[(size_t)tile * gridDim.y + b] = (unsigned char)max(max(sred[0], sred[1]), max(sred[2], sred[3]));
 }
 
-// Cost prefix of the (tile, spot block) units, cost[u] .. cost[u + 1]: unit u
-// runs 2^strips[u] steps of kSepStepCost. One CTA of 1024 threads.
-__global__ void k_sep_scan(const unsigned char* __restrict__ strips, int U, int* __restrict__ cost) {
-  __shared__ int wsum[32];
+// Cost prefixes of the (tile, spot block) units, cost[u] .. cost[u + 1]: unit
+// u runs 2^strips[u] forward steps (CTA 0), or the chunks of its spots in the
+// adjoint (CTA 1; acost[U + 1]: the largest chunk). CTAs of 1024 threads.
+__global__ void k_sep_scan(const unsigned char* __restrict__ strips, int U, int N, int nb, int* __restrict__ cost,
+                           int* __restrict__ acost) {
+  __shared__ int wsum[32], wmax[32];
+  const bool adj = blockIdx.x == 1;
+  int* out = adj ? acost : cost;
   const int t = threadIdx.x, per = (U + 1023) / 1024;
   const int a = min(U, t * per), b = min(U, a + per);
-  int sum = 0;
-  for (int u = a; u < b; ++u) sum += sep_step_cost(strips[u]) << strips[u];
+  auto of = [&](int u) {
+    const int ls = strips[u];
+    return adj ? sep_chunks(N, u % nb) * sep_chunk_cost(ls) : sep_step_cost(ls) << ls;
+  };
+  int sum = 0, most = 0;
+  for (int u = a; u < b; ++u) {
+    sum += of(u);
+    most = max(most, (int)strips[u]);
+  }
+  most = __reduce_max_sync(0xffffffffu, most);
   int inc = sum;
   for (int h = 1; h < 32; h <<= 1) {
     const int v = __shfl_up_sync(0xffffffffu, inc, h);
     if ((t & 31) >= h) inc += v;
   }
-  if ((t & 31) == 31) wsum[t >> 5] = inc;
+  if ((t & 31) == 31) {
+    wsum[t >> 5] = inc;
+    wmax[t >> 5] = most;
+  }
   __syncthreads();
   if (t < 32) {
     int v = wsum[t];
@@ -159,14 +174,16 @@ __global__ void k_sep_scan(const unsigned char* __restrict__ strips, int U, int*
       if (t >= h) v += x;
     }
     wsum[t] = v;
+    most = __reduce_max_sync(0xffffffffu, wmax[t]);
+    if (adj && t == 0) out[U + 1] = sep_chunk_cost(most);
   }
   __syncthreads();
   int acc = inc - sum + (t >= 32 ? wsum[(t >> 5) - 1] : 0);
   for (int u = a; u < b; ++u) {
-    cost[u] = acc;
-    acc += sep_step_cost(strips[u]) << strips[u];
+    out[u] = acc;
+    acc += of(u);
   }
-  if (t == 1023) cost[U] = acc;
+  if (t == 1023) out[U] = acc;
 }
 
 // --- forward --------------------------------------------------------------------
@@ -198,15 +215,6 @@ struct SepStep {
   int tile, b, s, ls, bb;
 };
 
-// Offset my of a strip's middle row (0 for the whole tile).
-__device__ __forceinline__ float strip_mid(int s, int ls) {
-  const int n = 32 >> ls;
-  return ls == 0 ? 0.0f : (float)(s * n - 16) + 0.5f * (float)(n - 1);
-}
-
-__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
 // The tensor core's fp32 accumulator truncates: measured over 256^2 to
 // 1920 x 1152 pixels, fields came out smaller by 2.8e-7 of themselves whatever
 // the input, and by 5e-8 at random. The scale makes up for the first.
@@ -238,7 +246,7 @@ __device__ __forceinline__ void sep_sum_pair(const SepPoly& q, float R1s, float 
   float2 Ti = fma2(q2r, D(z, 1), fma2(n1, D(x, 2), D(x, 1)));
   Ti = fma2(q3r, D(z, 3), fma2(q3i, D(z, 2), fma2(q2i, D(z, 0), Ti)));
   float2 c, sn;
-  cis2(sep_angle(q.ay, -q.ay, q.ayl, q.y2, q.y3, q.y4, dup2(q.base), m), c, sn);
+  cis2(sep_angle(q.ay, -q.ay, q.ayl, q.y2, q.y3, q.y4, q.base, -q.base, m), c, sn);
   if (one >= 0) {
     const float2 w = one ? make_float2(0.0f, 1.0f) : make_float2(1.0f, 0.0f);
     c = mul2(c, w);
@@ -273,13 +281,6 @@ __device__ __forceinline__ void sep_sum_rows(const SepPoly& q, float ms, uint32_
   }
 }
 
-// (c, s) split into f16 pairs (hi, lo); s negated by the caller's angle.
-__device__ __forceinline__ void split_pack(float2 v, uint32_t& hi, uint32_t& lo) {
-  const float2 h = split_hi2(v), l = fma2(h, dup2(-1.0f), v);
-  hi = pack_f16(h.x, h.y);
-  lo = pack_f16(l.x, l.y);
-}
-
 __device__ __forceinline__ void put16(uint8_t* base, int r, int c, const uint32_t (&v)[4], uint32_t flip = 0) {
   *reinterpret_cast<uint4*>(base + swz_chunk(r, c)) = make_uint4(v[0] ^ flip, v[1] ^ flip, v[2] ^ flip, v[3] ^ flip);
 }
@@ -296,7 +297,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) k_sep_forward(const SepFwdPara
   float* scales = reinterpret_cast<float*>(smax + 8);            // [4] 2^e of the steps' tiles
   SepStep* steps = reinterpret_cast<SepStep*>(scales + 4);       // [4]
   const int t = threadIdx.x, w = t >> 5, lane = t & 31;
-  const int row = t & 127;
+  const int row = t & 127, prow = (row >> 5) * 128 + (row & 31);   // the spot's place in a slot
   const int nb = p.nb, npad = nb * kSepSpots, U = p.g.T * nb;
   if (w == 0) tmem_alloc(slot, 512);
   if (t == 0) {
@@ -339,8 +340,8 @@ __global__ void __launch_bounds__(kFwdThreads, 1) k_sep_forward(const SepFwdPara
         psc = scale;
       }
       if (r.b < 0) break;
-      const float4* sq = reinterpret_cast<const float4*>(sm + kFwdSlots + (it & 3) * kFSlot) + row;
-      const SepPoly q = sep_unpack(sq[0], sq[128], sq[256], sq[384]);
+      const float4* sq = reinterpret_cast<const float4*>(sm + kFwdSlots + (it & 3) * kFSlot) + prow;
+      const SepPoly q = sep_unpack(sq[0], sq[32], sq[64], sq[96]);
       const int rows = 32 >> r.ls, pairs = rows >= 2 ? rows >> 1 : 1;
       const int np = pairs >= 2 ? pairs >> 1 : (half ? 0 : 1), p0 = ((r.s * rows) >> 1) + half * np;
       ok = ok && mbar_wait(&full[it & 1], (it >> 1) & 1, kTcWaitPolls);
@@ -434,9 +435,8 @@ __global__ void __launch_bounds__(kFwdThreads, 1) k_sep_forward(const SepFwdPara
           break;
         }
         mbar_expect_tx(&listed[it & 3], kFSlot);
-        const float4* src = p.poly + (size_t)x.tile * 4 * npad + x.b * kSepSpots;
-        for (int k = 0; k < 4; ++k)
-          bulk_g2s(sm + kFwdSlots + (it & 3) * kFSlot + k * 2048, src + (size_t)k * npad, 2048, &listed[it & 3]);
+        bulk_g2s(sm + kFwdSlots + (it & 3) * kFSlot, p.poly + ((size_t)x.tile * nb + x.b) * (4 * kSepSpots), kFSlot,
+                 &listed[it & 3]);
         pos += c;
         ++x.s;
       }
@@ -500,18 +500,8 @@ __global__ void __launch_bounds__(kFwdThreads, 1) k_sep_forward(const SepFwdPara
 
     // A: X(u) of this thread's spot for its 16 columns, about the strip's row
     auto build_a = [&](const float4* sq, const SepStep& x, uint8_t* ah) {
-      const SepPoly q = sep_unpack(sq[0], sq[128], sq[256], sq[384]);
-      float ax = q.ax, axl = q.axl, x2 = q.x2, x3 = q.x3;
-      if (x.ls) {
-        const float ms = strip_mid(x.s, x.ls);
-        const float R1 = ms * (q.c11 + ms * (q.c12 + ms * q.c13)), R2 = ms * (q.c21 + ms * q.c22), n3 = ms * q.n31;
-        const float d = R1 * (0.15915494309189535f * 0.0625f);
-        const float s = __fadd_rn(ax, d), z = __fsub_rn(s, ax);
-        axl = fmaf(__fadd_rn(__fsub_rn(ax, __fsub_rn(s, z)), __fsub_rn(d, z)), 6.283185307179586f, axl);
-        ax = s;
-        x2 = fmaf(R2, 0.0625f * 0.0625f, x2);
-        x3 = fmaf(n3, -0.0625f * 0.0625f * 0.0625f, x3);
-      }
+      const SepPoly q = sep_unpack(sq[0], sq[32], sq[64], sq[96]);
+      const SepColumns o = sep_columns(q, x.s, x.ls);
       // X = exp(-i angle): the negated angle's cosine and sine
 #pragma unroll
       for (int c8 = 0; c8 < 2; ++c8) {
@@ -520,7 +510,8 @@ __global__ void __launch_bounds__(kFwdThreads, 1) k_sep_forward(const SepFwdPara
         for (int q2 = 0; q2 < 4; ++q2) {
           const float m0 = (float)(16 * half - 16 + 8 * c8 + 2 * q2);
           float2 cs, sn;
-          cis2(sep_angle(-ax, ax, -axl, -x2, -x3, -q.x4, make_float2(0.0f, 0.0f), make_float2(m0, m0 + 1.0f)), cs, sn);
+          cis2(sep_angle(-o.ax, o.ax, -o.axl, -o.x2, -o.x3, -o.x4, make_float2(m0, m0 + 1.0f)), cs,
+               sn);
           split_pack(cs, rh[q2], rl[q2]);
           split_pack(sn, ih[q2], il[q2]);
         }
@@ -557,7 +548,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) k_sep_forward(const SepFwdPara
         tile = x.tile;
         scale = build_b(tile, sm + kFwdB + (uint32_t)x.bb * kFwdBuf);
       }
-      build_a(reinterpret_cast<const float4*>(sm + kFwdSlots + (it & 3) * kFSlot) + row, x,
+      build_a(reinterpret_cast<const float4*>(sm + kFwdSlots + (it & 3) * kFSlot) + prow, x,
               sm + (uint32_t)d * 2 * kFA);
       fence_async_smem();
       if (g == 0) scales[it & 3] = scale;
@@ -606,12 +597,12 @@ cudaError_t sep_build_table(const Geometry& g, const MonoTerm* terms, const int*
 }
 
 cudaError_t sep_build_params(const Geometry& g, const float* tab, const float* coeff, float4* poly,
-                             unsigned char* strips, int* cost, cudaStream_t s) {
+                             unsigned char* strips, int* cost, int* acost, cudaStream_t s) {
   const int nb = sep_blocks(g.N);
   k_sep_params<<<dim3(g.T, nb), kSepSpots, 0, s>>>(g, tab, coeff, poly, strips, nb * kSepSpots);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  k_sep_scan<<<1, 1024, 0, s>>>(strips, g.T * nb, cost);
+  k_sep_scan<<<2, 1024, 0, s>>>(strips, g.T * nb, g.N, nb, cost, acost);
   return cudaGetLastError();
 }
 

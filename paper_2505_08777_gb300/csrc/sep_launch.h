@@ -5,6 +5,7 @@
 
 #include "common.cuh"
 #include "mono.h"
+#include "tc_launch.h"
 
 namespace ash {
 
@@ -18,6 +19,13 @@ constexpr float kSepTol = 1e-6f;   // largest part of exp(-i r) the cubic in u m
 // tile: 20): preparing X and the MMAs' latency stay, the sums shrink.
 __host__ __device__ constexpr int sep_step_cost(int ls) { return ls == 0 ? 20 : ls == 1 ? 13 : ls == 2 ? 10 : 8; }
 
+// The same of one chunk (32 spots of a tile) of the adjoint, all its strips.
+constexpr int kSepChunk = 32;
+__host__ __device__ constexpr int sep_chunk_cost(int ls) { return 20 + 14 * ((1 << ls) - 1); }
+__host__ __device__ constexpr int sep_chunks(int N, int b) {
+  return (N - b * kSepSpots >= kSepSpots) ? kSepSpots / kSepChunk : (N - b * kSepSpots + kSepChunk - 1) / kSepChunk;
+}
+
 inline int sep_blocks(int N) { return (N + kSepSpots - 1) / kSepSpots; }
 
 // Basis polynomials over each tile about its pixel (16, 16), in turns:
@@ -25,11 +33,14 @@ inline int sep_blocks(int N) { return (N + kSepSpots - 1) / kSepSpots; }
 // c20 c30 c40 c02 c03 c04 c11 c21 c12 c22 c31 c13 per u^k v^l.
 cudaError_t sep_build_table(const Geometry& g, const MonoTerm* terms, const int* term_off, float* tab, cudaStream_t s);
 
-// Phase polynomials of every (tile, spot), [T][4][npad] float4 (SepPoly), and
+// Phase polynomials of every (tile, spot), [T][chunk of 32 spots][4][32]
+// float4 (SepPoly), and
 // per (tile, spot block) the log2 of the row strips its mixed terms need and
-// the prefix of its steps' cost [T nb + 1].
+// the prefixes of their forward steps' cost
+// [T nb + 1] and of their adjoint chunks' cost [T nb + 1], then the largest
+// chunk cost.
 cudaError_t sep_build_params(const Geometry& g, const float* tab, const float* coeff, float4* poly,
-                             unsigned char* strips, int* cost, cudaStream_t s);
+                             unsigned char* strips, int* cost, int* acost, cudaStream_t s);
 
 struct SepFwdParams {
   Geometry g;
@@ -43,7 +54,23 @@ struct SepFwdParams {
   int G;
   unsigned* err;
 };
+struct SepAdjParams {
+  TcAdjParams a;                 // geometry, amplitude, y, outputs
+  int nb;
+  const float4* poly;
+  const unsigned char* strips;
+  const int* cost;               // adjoint prefix
+  const float2* ys;              // [128 nb] y / scale
+  const float* scale;            // [4 nb] power of two per chunk of 32 spots
+  float2* split;                 // [G][2][kTilePix] partial sums of tiles split between CTAs
+  int* tickets;                  // [T] CTAs done with a split tile (left at 0)
+  int G;
+};
 cudaError_t sep_prepare();
+cudaError_t sep_adjoint_prepare();
+// y divided by a power of two (scale) per chunk of 32 spots.
+cudaError_t sep_launch_scale(const float2* y, int N, float2* ys, float* scale, cudaStream_t s);
+cudaError_t sep_launch_adjoint(const SepAdjParams& p, cudaStream_t s);
 cudaError_t sep_launch_forward(const SepFwdParams& p, cudaStream_t s);   // kernel and reduction
 
 }  // namespace ash

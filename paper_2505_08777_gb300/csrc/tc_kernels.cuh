@@ -35,6 +35,7 @@
 
 #include "common.cuh"
 #include "tc_common.cuh"
+#include "tc_epilogue.cuh"
 #include "tc_launch.h"
 
 namespace ash {
@@ -289,23 +290,6 @@ __device__ __forceinline__ void tc_range_end(uint64_t* bars, const uint32_t* arm
     if (threadIdx.x == 0) tc_drain(bars, armed, nbars);
   }
   __syncthreads();
-}
-
-// Adjoint output of row r of chunk qc (in the pixel's user-layout slot and,
-// for kEpiFimg, in the tc-layout nearfield f = A exp(i arg g) as (A, arg g / 2 pi)).
-__device__ __forceinline__ void tc_adjoint_epilogue(const TcAdjParams& p, long long qc, int r, float gr, float gi) {
-  const Geometry& G = p.g;
-  const TcPixel px = tc_pixel(G, qc, r);
-  if (px.i >= G.nx || px.j >= G.ny) return;
-  const bool need_a = (p.out.epilogue & (kEpiGradPhase | kEpiFimg)) != 0;
-  const float a = need_a ? __ldg(p.amp_img + px.img) : 0.0f;
-  adjoint_epilogue(p.out, (size_t)px.j * G.nx + px.i, gr, gi, a);
-  if (p.out.epilogue & kEpiFimg) {
-    const float ph = (gr == 0.0f && gi == 0.0f) ? 0.0f : atan2f(gi, gr) * 0.15915494309189535f;
-    float* q = reinterpret_cast<float*>(p.fimg + (size_t)qc * 32 + (r >> 1));
-    q[r & 1] = a;
-    q[2 + (r & 1)] = ph;
-  }
 }
 
 // --- adjoint ------------------------------------------------------------------
