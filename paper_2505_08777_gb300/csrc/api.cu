@@ -185,6 +185,7 @@ bool use_tc_adj(const ash_hologram* h) {
 // 300^2 N = 200 28 / 17; adjoint 256^2 N = 100 13.5 / 16.4, 300^2 N = 200
 // 24 / 20.
 constexpr int kSepSideFwd = 400, kSepSideAdj = 560, kSepSide2 = 200, kSepFewSpots = 64, kSepFewSide = 900;
+constexpr size_t kSepMaxBytes = (size_t)8 << 30;   // of phase polynomials, and of partial dL/dC an eighth
 constexpr long long kSepTerms2Fwd = 6LL << 20, kSepTerms2Adj = 10LL << 20;
 bool sep_pays(const ash_hologram* h, int side4, long long terms2) {
   const Geometry& g = h->g;
@@ -206,9 +207,25 @@ bool use_tc_grad(const ash_hologram* h) {
   return h->variant == 2 || h->g.N >= kTcFwdMinSpots;
 }
 
+// The moments take u^4 as u^2 - 1/8 over a tile: with degree 4 the dropped part
+// of dL/dC, (16 / R)^4 of a quartic mode's scale, is below 1e-6 from this side
+// (2.5e-6 at 700).
+constexpr int kSepSideGrad4 = 900;
+bool use_sep_grad(const ash_hologram* h) {
+  const int side = h->g.nx < h->g.ny_full ? h->g.nx : h->g.ny_full;
+  return use_sep_adj(h) && h->sep_dpart && (h->sep_ord < 4 || side >= kSepSideGrad4);
+}
+
+// Whether any kernel but the separable ones may read czs and rot.
+bool needs_tc_images(const ash_hologram* h) {
+  return h->tc_ok && (h->tc_pinned || !(use_sep_fwd(h) && use_sep_adj(h) && use_sep_grad(h)));
+}
+
 // Whether the handle's current kernel choice runs any FMA-pipe kernel (they
 // read the register-image basis dz; the tensor-core kernels do not).
-bool needs_fma_image(const ash_hologram* h) { return !(use_tc_fwd(h) && use_tc_adj(h) && use_tc_grad(h)); }
+bool needs_fma_image(const ash_hologram* h) {
+  return !((use_sep_fwd(h) || use_tc_fwd(h)) && (use_sep_adj(h) || use_tc_adj(h)) && (use_sep_grad(h) || use_tc_grad(h)));
+}
 
 // CTA range starts that give every CTA the same estimated time rather than
 // the same number of units: prefix(u) is the summed cost of units [0, u)
@@ -291,6 +308,9 @@ cudaError_t enqueue_tc_coeff(ash_hologram* h, cudaStream_t s) {
                                            h->sep_acost, s);
     if (e != cudaSuccess) return e;
   }
+  // the other tensor-core kernels' images only where one of them is in use
+  h->tc_stale = !needs_tc_images(h);
+  if (h->tc_stale) return cudaSuccess;
   return tc_build_coeff(h->g, h->tc_layout, h->coeff, h->anchors, h->czs, h->rot, s);
 }
 
@@ -325,6 +345,15 @@ SepFwdParams sep_fwd_params(const ash_hologram* h, float2* E) {
   p.E = E;
   p.G = h->sep_G;
   p.err = h->err_word;
+  return p;
+}
+
+SepFwdParams sep_grad_params(const ash_hologram* h, const float2* gE, float* dC) {
+  SepFwdParams p = sep_fwd_params(h, nullptr);
+  p.gE = gE;
+  p.tab = h->sep_tab;
+  p.dpart = h->sep_dpart;
+  p.dC = dC;
   return p;
 }
 
@@ -382,7 +411,9 @@ ash_status enqueue_forward(ash_hologram* h, int source, const float* phase, cons
       if (e != cudaSuccess) return cuda_fail(e, "nearfield image launch");
     }
     if (use_sep_fwd(h)) {
-      e = sep_launch_forward(sep_fwd_params(h, E), s);
+      const SepFwdParams sp = sep_fwd_params(h, E);
+      e = sep_launch_forward(sp, s);
+      if (e == cudaSuccess) e = sep_launch_forward_reduce(sp, s);
       return e == cudaSuccess ? ASH_OK : cuda_fail(e, "separable forward launch");
     }
     const TcFwdParams tp = tc_fwd_params(h, E);
@@ -498,6 +529,15 @@ ash_status ensure_fma_image(ash_hologram* h) {
   k_basis<<<h->g.T, h->g.NT, 0, h->home>>>(bp);
   ASH_CUDA(cudaGetLastError());
   ASH_CUDA(cudaStreamSynchronize(h->home));
+  return ASH_OK;
+}
+
+ash_status ensure_tc_images(ash_hologram* h) {
+  if (!h->tc_ok || !h->tc_stale) return ASH_OK;
+  ASH_CUDA(cudaDeviceSynchronize());
+  ASH_CUDA(tc_build_coeff(h->g, h->tc_layout, h->coeff, h->anchors, h->czs, h->rot, h->home));
+  ASH_CUDA(cudaStreamSynchronize(h->home));
+  h->tc_stale = false;
   return ASH_OK;
 }
 
@@ -845,7 +885,8 @@ ash_status create_impl(ash_hologram** out, int nx, int ny, int row0, int ny_full
     int ord = 0;
     for (const MonoTerm& m : spec->terms) ord = m.px + m.py > ord ? m.px + m.py : ord;
     h->sep_ord = ord;
-    if (ord <= kSepMaxOrd && (sep_pays(h, kSepSideFwd, kSepTerms2Fwd) || sep_pays(h, kSepSideAdj, kSepTerms2Adj))) {
+    const size_t poly = (size_t)g.T * sep_blocks(N) * kSepSpots * 64;   // bytes of the phase polynomials
+    if (ord <= kSepMaxOrd && poly <= kSepMaxBytes && (sep_pays(h, kSepSideFwd, kSepTerms2Fwd) || sep_pays(h, kSepSideAdj, kSepTerms2Adj))) {
       ce = sep_prepare();
       if (ce == cudaSuccess) ce = sep_adjoint_prepare();
       if (ce != cudaSuccess) return fail(cuda_fail(ce, "separable kernel preparation"));
@@ -894,6 +935,8 @@ ash_status create_impl(ash_hologram** out, int nx, int ny, int row0, int ny_full
     if ((st = ws(h, &h->sep_split, 2 * (size_t)h->sep_G * kTilePix)) != ASH_OK) return fail(st);
     if ((st = ws(h, &h->sep_ys, npad)) != ASH_OK) return fail(st);
     if ((st = ws(h, &h->sep_scale, npad / kSepChunk)) != ASH_OK) return fail(st);
+    const size_t dp = (size_t)kSepFwdRows * h->sep_G * D * npad;
+    if (dp * sizeof(float) <= kSepMaxBytes / 8 && (st = ws(h, &h->sep_dpart, dp)) != ASH_OK) return fail(st);
     if ((st = ws(h, &h->sep_tickets, (size_t)g.T)) != ASH_OK) return fail(st);
     if ((st = ws(h, &h->sep_part, (size_t)kSepFwdRows * h->sep_G * npad)) != ASH_OK) return fail(st);
   }
@@ -1241,7 +1284,12 @@ ash_status ash_grad(ash_hologram* h, const float* phase, const float* grad_E, fl
     ash_status st = enqueue_adjoint(h, gE, nullptr, nullptr, phase, dphase, kEpiGradPhase, s);
     if (st != ASH_OK) return st;
   }
-  if (dcoeff && use_tc_grad(h)) {
+  if (dcoeff && use_sep_grad(h)) {
+    ASH_CUDA(tc_field_img(h->g, h->amp_img, phase, nullptr, h->fimg, s));
+    const SepFwdParams sp = sep_grad_params(h, gE, dcoeff);
+    ASH_CUDA(sep_launch_gradc(sp, s));
+    ASH_CUDA(sep_launch_gradc_reduce(sp, s));
+  } else if (dcoeff && use_tc_grad(h)) {
     ASH_CUDA(enqueue_tc_gradc(h, phase, gE, dcoeff, s));
   } else if (dcoeff) {
     if (!h->dz) return set_error(ASH_ERR_DEVICE, "FMA-pipe moments without their basis image");
@@ -1279,6 +1327,10 @@ ash_status ash_set_kernel_variant(ash_hologram* h, int variant) {
     return set_error(ASH_ERR_UNSUPPORTED, "tensor-core kernels need D <= %d (D = %d)", kTcMaxModes, h->g.D);
   h->variant = variant;
   clear_graphs(h);
+  if (needs_tc_images(h)) {
+    const ash_status st = ensure_tc_images(h);
+    if (st != ASH_OK) return st;
+  }
   if (needs_fma_image(h)) return ensure_fma_image(h);
   return ASH_OK;
 }
@@ -1329,15 +1381,18 @@ ash_status ash_profile(ash_hologram* h, const float* phase, const float* y, floa
   fp.source = kSrcPhase;
   fp.partial = h->partial;
   const int cols = 2 * h->g.N;
-  const bool tc = use_tc_fwd(h), tca = use_tc_adj(h);
+  const bool tc = use_tc_fwd(h), tca = use_tc_adj(h), sf = use_sep_fwd(h), sa = use_sep_adj(h), sg = use_sep_grad(h);
   const TcFwdParams tf = tc_fwd_params(h, h->E);
-  if (tc) e = tc_field_img(h->g, h->amp_img, phase, nullptr, h->fimg, s);
+  const SepFwdParams spf = sep_fwd_params(h, h->E);
+  if (sf || tc) e = tc_field_img(h->g, h->amp_img, phase, nullptr, h->fimg, s);
   cudaEventRecord(ev[0], s);
-  if (e == cudaSuccess) e = tc ? tc_launch_forward(h->tc_na, tf, h->tfwd.G, s) : launch_forward(h->g.D, fp, h->sched.G, s);
+  if (e == cudaSuccess) e = sf ? sep_launch_forward(spf, s) : tc ? tc_launch_forward(h->tc_na, tf, h->tfwd.G, s) : launch_forward(h->g.D, fp, h->sched.G, s);
   cudaEventRecord(ev[1], s);
   if (e == cudaSuccess) {
     cudaEventRecord(ev[2], s);
-    if (!tc) {
+    if (sf) {
+      e = sep_launch_forward_reduce(spf, s);
+    } else if (!tc) {
       k_col_reduce<<<(cols + 31) / 32, dim3(32, 32), 0, s>>>(h->partial, h->fwd_rows, cols, reinterpret_cast<float*>(h->E));
       e = cudaGetLastError();
     } else if (h->tfwd_split) {
@@ -1354,14 +1409,18 @@ ash_status ash_profile(ash_hologram* h, const float* phase, const float* y, floa
   ap.out.phase_out = h->wgs_phase;
   ap.out.epilogue = kEpiPhase;
   const TcAdjParams tp = tc_adj_params(h, y2, ap.out);
+  const SepAdjParams spa = sep_adj_params(h, y2, ap.out);
+  if (e == cudaSuccess && sa) e = sep_launch_scale(y2, h->g.N, h->sep_ys, h->sep_scale, s);
   if (e == cudaSuccess) {
     cudaEventRecord(ev[4], s);
-    e = tca ? tc_launch_adjoint(h->tc_na, tp, h->tadj.G, s) : launch_adjoint(h->g.D, ap, h->sched.G, s);
+    e = sa ? sep_launch_adjoint(spa, s) : tca ? tc_launch_adjoint(h->tc_na, tp, h->tadj.G, s) : launch_adjoint(h->g.D, ap, h->sched.G, s);
     cudaEventRecord(ev[5], s);
   }
   if (e == cudaSuccess) {
     cudaEventRecord(ev[6], s);
-    if (tca && h->tadj_split) {
+    if (sa) {
+      // no fix-up: the last CTA of a split tile finishes it
+    } else if (tca && h->tadj_split) {
       e = tc_launch_adjoint_fixup(tp, h->tadj_nsplit, s);
     } else if (!tca && h->split_tiles) {
       k_adjoint_fixup<<<h->g.T, h->g.NT, 0, s>>>(ap);
@@ -1383,7 +1442,8 @@ ash_status ash_profile(ash_hologram* h, const float* phase, const float* y, floa
     gp.gradE = y2;
     gp.partial = h->gradc_partial;
     cudaEventRecord(ev[10], s);
-    e = use_tc_grad(h) ? tc_launch_gradc(tc_grad_params(h, y2, h->gradc_partial), h->tgrad_split, s)
+    e = sg ? sep_launch_gradc(sep_grad_params(h, y2, h->gradc_partial), s)
+        : use_tc_grad(h) ? tc_launch_gradc(tc_grad_params(h, y2, h->gradc_partial), h->tgrad_split, s)
                        : launch_gradc(h->g.D, gp, dim3(h->gradc_gx, h->gradc_gy), s);
     cudaEventRecord(ev[11], s);
   }

@@ -580,8 +580,12 @@ ash_status build_group(ash_batch* b, long long solo_terms, cudaStream_t s) {
     }
     b->group_idx.push_back(i);
     b->holos.push_back(h);
-    // the persistent FMA-pipe kernels read the register-image basis
-    ash_status st = ensure_fma_image(h);
+    // the persistent kernels read the register-image basis or the
+    // tensor-core spot images
+    h->tc_pinned = true;
+    ash_status st = ensure_tc_images(h);
+    if (st != ASH_OK) return st;
+    st = ensure_fma_image(h);
     if (st != ASH_OK) return st;
     BatchHolo bh{};
     bh.v = view_of(h);

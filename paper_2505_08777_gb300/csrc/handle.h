@@ -41,6 +41,8 @@ struct ash_hologram {
   bool tadj_split = false;      // some group's spots span two CTA ranges
   ash::TcFwdSched tfwd{};       // forward units (spot block, pixel chunk)
   bool tfwd_split = false;      // some spot block's pixels span two CTA ranges
+  bool tc_stale = false;        // czs and rot are older than the coefficients (no kernel in use reads them)
+  bool tc_pinned = false;       // a batch's persistent kernels read them
   float* zs = nullptr;
   float* czs = nullptr;
   float4* fimg = nullptr;
@@ -69,6 +71,7 @@ struct ash_hologram {
   float* sep_tab = nullptr;     // basis polynomials per tile
   float4* sep_poly = nullptr;   // phase polynomials per (tile, spot)
   unsigned char* sep_strips = nullptr;   // per (tile, spot block): log2 of its row strips
+  float* sep_dpart = nullptr;   // [kSepFwdRows sep_G][D][128 nb] partial dL/dC
   int* sep_cost = nullptr;      // prefix of its forward steps' cost
   int* sep_acost = nullptr;     // prefix of its adjoint chunks' cost
   float2* sep_split = nullptr;  // [sep_G][2][kTilePix] adjoint sums of tiles split between CTAs
@@ -130,6 +133,9 @@ int graph_kernel_nodes(cudaGraph_t g);
 // The FMA-pipe kernels' register-image basis: rebuilt from the monomial
 // tables if it was released (synchronises the device).
 ash_status ensure_fma_image(ash_hologram* h);
+// The tensor-core spot images (czs, rot), if they are older than the
+// coefficients (synchronises the device).
+ash_status ensure_tc_images(ash_hologram* h);
 // Record a message for ash_last_error() (any translation unit).
 void record_error(const char* msg);
 // Map a CUDA error to ASH_ERR_CUDA with a message.

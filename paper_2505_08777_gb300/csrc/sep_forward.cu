@@ -1,5 +1,7 @@
 // Separable forward transform (see sep_common.cuh): the tables it works from,
 // the kernel and the sum of its CTAs' partial fields.
+#include <type_traits>
+
 #include "sep_common.cuh"
 
 namespace ash {
@@ -258,6 +260,99 @@ __device__ __forceinline__ void sep_sum_pair(const SepPoly& q, float R1s, float 
   acc.sr = fma2(sn, Tr, acc.sr);
 }
 
+// Moments of a tile over its pixels, Im(conj(gE) f K) mx^k my^l summed: m0[l]
+// (k = 0), m1, m2, m3.
+struct SepMoments {
+  float2 m0[5], m1[4], m2[3], m3[2];
+  __device__ __forceinline__ void zero() {
+    for (float2& v : m0) v = make_float2(0.0f, 0.0f);
+    for (float2& v : m1) v = make_float2(0.0f, 0.0f);
+    for (float2& v : m2) v = make_float2(0.0f, 0.0f);
+    for (float2& v : m3) v = make_float2(0.0f, 0.0f);
+  }
+};
+
+// The moments' share of one pair of rows (arguments as sep_sum_pair; g is
+// dL/dE). u^k exp(-i r) keeps powers up to 3: u^4 counts as u^2 - 1/8, and
+// what lies beyond is dropped (its factors b_dk Q_m are below 4e-6 of the
+// largest basis values at the sides this serves).
+__device__ __forceinline__ void sep_moment_pair(const SepPoly& q, float R1s, float R2s, float n3s, const uint32_t* x,
+                                                const uint32_t* z, float2 m, int one, float2 g, SepMoments& acc) {
+  auto D = [](const uint32_t* a, int i) { return make_float2(__uint_as_float(a[2 * i]), __uint_as_float(a[2 * i + 1])); };
+  const float2 R1 = fma2(fma2(fma2(dup2(q.c13), m, dup2(q.c12)), m, dup2(q.c11)), m, dup2(-R1s));
+  const float2 R2 = fma2(fma2(dup2(q.c22), m, dup2(q.c21)), m, dup2(-R2s));
+  const float2 n3 = fma2(dup2(q.n31), m, dup2(-n3s));   // -R3
+  const float2 n1 = mul2(R1, dup2(-1.0f)), s = mul2(R1, R1);
+  const float2 q2r = fma2(s, fma2(s, dup2(1.0f / 24.0f), dup2(-0.5f)), mul2(R2, mul2(R2, dup2(-0.5f))));
+  const float2 q2i = mul2(R2, fma2(s, dup2(0.5f), dup2(-1.0f))), p2i = mul2(q2i, dup2(-1.0f));
+  const float2 q3r = mul2(n1, R2), q3i = fma2(mul2(R1, s), dup2(1.0f / 6.0f), n3), p3i = mul2(q3i, dup2(-1.0f));
+  const float2 d4r = fma2(D(x, 0), dup2(-0.125f), D(z, 0)), d4i = fma2(D(x, 1), dup2(-0.125f), D(z, 1));
+  // conj(gE) Y
+  float2 c, sn;
+  cis2(sep_angle(q.ay, -q.ay, q.ayl, q.y2, q.y3, q.y4, q.base, -q.base, m), c, sn);
+  if (one >= 0) {
+    const float2 w = one ? make_float2(0.0f, 1.0f) : make_float2(1.0f, 0.0f);
+    c = mul2(c, w);
+    sn = mul2(sn, w);
+  }
+  const float2 Gr = fma2(sn, dup2(-g.y), mul2(c, dup2(g.x))), Gi = fma2(sn, dup2(-g.x), mul2(c, dup2(-g.y)));
+  const float2 mm = mul2(m, m), m3 = mul2(mm, m), m4 = mul2(mm, mm);
+  {
+    float2 Sr = fma2(R1, D(x, 3), D(x, 0)), Si = fma2(n1, D(x, 2), D(x, 1));
+    Sr = fma2(q2r, D(z, 0), fma2(p2i, D(z, 1), Sr));
+    Si = fma2(q2r, D(z, 1), fma2(q2i, D(z, 0), Si));
+    Sr = fma2(q3r, D(z, 2), fma2(p3i, D(z, 3), Sr));
+    Si = fma2(q3r, D(z, 3), fma2(q3i, D(z, 2), Si));
+    const float2 P = fma2(Gr, Si, mul2(Gi, Sr));
+    acc.m0[0] = add2(acc.m0[0], P);
+    acc.m0[1] = fma2(P, m, acc.m0[1]);
+    acc.m0[2] = fma2(P, mm, acc.m0[2]);
+    acc.m0[3] = fma2(P, m3, acc.m0[3]);
+    acc.m0[4] = fma2(P, m4, acc.m0[4]);
+  }
+  {
+    float2 Sr = fma2(R1, D(z, 1), D(x, 2)), Si = fma2(n1, D(z, 0), D(x, 3));
+    Sr = fma2(q2r, D(z, 2), fma2(p2i, D(z, 3), Sr));
+    Si = fma2(q2r, D(z, 3), fma2(q2i, D(z, 2), Si));
+    Sr = fma2(q3r, d4r, fma2(p3i, d4i, Sr));
+    Si = fma2(q3r, d4i, fma2(q3i, d4r, Si));
+    const float2 P = fma2(Gr, Si, mul2(Gi, Sr));
+    acc.m1[0] = add2(acc.m1[0], P);
+    acc.m1[1] = fma2(P, m, acc.m1[1]);
+    acc.m1[2] = fma2(P, mm, acc.m1[2]);
+    acc.m1[3] = fma2(P, m3, acc.m1[3]);
+  }
+  {
+    float2 Sr = fma2(R1, D(z, 3), D(z, 0)), Si = fma2(n1, D(z, 2), D(z, 1));
+    Sr = fma2(q2r, d4r, fma2(p2i, d4i, Sr));
+    Si = fma2(q2r, d4i, fma2(q2i, d4r, Si));
+    const float2 P = fma2(Gr, Si, mul2(Gi, Sr));
+    acc.m2[0] = add2(acc.m2[0], P);
+    acc.m2[1] = fma2(P, m, acc.m2[1]);
+    acc.m2[2] = fma2(P, mm, acc.m2[2]);
+  }
+  {
+    const float2 Sr = fma2(R1, d4i, D(z, 2)), Si = fma2(n1, d4r, D(z, 3));
+    const float2 P = fma2(Gr, Si, mul2(Gi, Sr));
+    acc.m3[0] = add2(acc.m3[0], P);
+    acc.m3[1] = fma2(P, m, acc.m3[1]);
+  }
+}
+
+// The row pairs [p0, p0 + np) of D at TMEM address ta.
+__device__ __forceinline__ void sep_moment_rows(const SepPoly& q, float ms, uint32_t ta, int p0, int np, int one,
+                                                float2 g, SepMoments& acc) {
+  const float R1s = ms * (q.c11 + ms * (q.c12 + ms * q.c13)), R2s = ms * (q.c21 + ms * q.c22), n3s = ms * q.n31;
+  for (int k = 0; k < np; ++k) {
+    uint32_t x[8], z[8];
+    tmem_ld8_nowait(ta + (uint32_t)((p0 + k) * 8), x);
+    tmem_ld8_nowait(ta + (uint32_t)(128 + (p0 + k) * 8), z);
+    tmem_wait();
+    const float m0 = (float)(2 * (p0 + k) - 16);
+    sep_moment_pair(q, R1s, R2s, n3s, x, z, make_float2(m0, m0 + 1.0f), one, g, acc);
+  }
+}
+
 // The row pairs [p0, p0 + np) of D at TMEM address ta (np 1 or even).
 __device__ __forceinline__ void sep_sum_rows(const SepPoly& q, float ms, uint32_t ta, int p0, int np, int one,
                                              SepSum& acc) {
@@ -285,6 +380,10 @@ __device__ __forceinline__ void put16(uint8_t* base, int r, int c, const uint32_
   *reinterpret_cast<uint4*>(base + swz_chunk(r, c)) = make_uint4(v[0] ^ flip, v[1] ^ flip, v[2] ^ flip, v[3] ^ flip);
 }
 
+// GRAD: the moment pass dL/dC = Im(conj(gE_n) sum_m Z_dm f_m K_nm): the summers
+// take moments of the same row sums over mx, my per tile and contract them with
+// the tile's basis polynomials.
+template <bool GRAD>
 __global__ void __launch_bounds__(kFwdThreads, 1) k_sep_forward(const SepFwdParams p) {
   extern __shared__ uint8_t raw[];
   uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(raw) + 1023) & ~(uintptr_t)1023);
@@ -315,27 +414,61 @@ __global__ void __launch_bounds__(kFwdThreads, 1) k_sep_forward(const SepFwdPara
     // --- summers: spot `row`, half of a step's row pairs ---
     const int half = t >> 7;
     float2* part = p.part + (size_t)(kSepFwdRows * blockIdx.x + half) * npad + row;
+    const int D = p.g.D;
+    float* dpart = p.dpart + (size_t)(kSepFwdRows * blockIdx.x + half) * D * npad + row;
     // no other thread touches these partial sums
-    for (int b = 0; b < nb; ++b) part[b * kSepSpots] = make_float2(0.0f, 0.0f);
+    if constexpr (GRAD) {
+      for (int k = 0; k < D * nb; ++k) dpart[(size_t)k * kSepSpots] = 0.0f;
+    } else {
+      for (int b = 0; b < nb; ++b) part[b * kSepSpots] = make_float2(0.0f, 0.0f);
+    }
     const uint32_t tlane = tmem + ((uint32_t)((w & 3) * 32) << 16);
-    SepSum acc;
+    std::conditional_t<GRAD, SepMoments, SepSum> acc;
     acc.zero();
-    int pb = -1;          // block and scale of the sums held
+    int pb = -1, pt = -1;   // block, tile and scale of the sums held
     float psc = 1.0f, pscale = 1.0f;
+    float2 g = make_float2(0.0f, 0.0f);
+    auto flush = [&]() {
+      if constexpr (GRAD) {
+        constexpr float tp = 6.283185307179586f, h = 0.0625f;
+        auto S = [&](float2 v, float f) { return (v.x + v.y) * (f * pscale); };
+        // in the table's units: turns for the pure powers, per pixel for the slopes
+        const float a00 = S(acc.m0[0], tp), a01 = S(acc.m0[1], tp), a02 = S(acc.m0[2], tp * h * h),
+                    a03 = S(acc.m0[3], tp * h * h * h), a04 = S(acc.m0[4], tp * h * h * h * h);
+        const float a10 = S(acc.m1[0], tp * 16.0f), a20 = S(acc.m2[0], tp), a30 = S(acc.m3[0], tp);
+        const float a40 = fmaf(a00, -0.125f, a20);
+        const float a11 = S(acc.m1[1], h), a21 = S(acc.m2[1], h), a12 = S(acc.m1[2], h * h), a22 = S(acc.m2[2], h * h),
+                    a31 = S(acc.m3[1], h), a13 = S(acc.m1[3], h * h * h);
+        const float2* tb = reinterpret_cast<const float2*>(p.tab + (size_t)pt * D * kSepTab);
+        for (int d = 0; d < D; ++d, tb += kSepTab / 2) {
+          const float2 t0 = __ldg(tb), t1 = __ldg(tb + 1), t2 = __ldg(tb + 2), t3 = __ldg(tb + 3), t4 = __ldg(tb + 4),
+                       t5 = __ldg(tb + 5), t6 = __ldg(tb + 6), t7 = __ldg(tb + 7), t8 = __ldg(tb + 8);
+          float v = fmaf(t0.x, a00, fmaf(t0.y, a00, fmaf(t1.x, a10, t2.x * a01)));
+          v = fmaf(t3.x, a20, fmaf(t3.y, a30, fmaf(t4.x, a40, fmaf(t4.y, a02, fmaf(t5.x, a03, fmaf(t5.y, a04, v))))));
+          v = fmaf(t6.x, a11, fmaf(t6.y, a21, fmaf(t7.x, a12, fmaf(t7.y, a22, fmaf(t8.x, a31, fmaf(t8.y, a13, v))))));
+          atomicAdd(dpart + (size_t)d * npad + pb * kSepSpots, v);
+        }
+      } else {
+        float2* o = part + pb * kSepSpots;
+        atomicAdd(&o->x, ((acc.cr.x + acc.cr.y) + (acc.si.x + acc.si.y)) * pscale);
+        atomicAdd(&o->y, ((acc.ci.x + acc.ci.y) - (acc.sr.x + acc.sr.y)) * pscale);
+      }
+    };
     for (uint32_t it = 0;; ++it) {
       ok = ok && mbar_wait(&ready[it & 3], (it >> 2) & 1, kTcWaitPolls);
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
       const SepStep r = steps[it & 3];
       const float scale = scales[it & 3];
-      if (r.b != pb || scale != psc) {
-        if (pb >= 0) {
-          float2* o = part + pb * kSepSpots;
-          atomicAdd(&o->x, ((acc.cr.x + acc.cr.y) + (acc.si.x + acc.si.y)) * pscale);
-          atomicAdd(&o->y, ((acc.ci.x + acc.ci.y) - (acc.sr.x + acc.sr.y)) * pscale);
-        }
+      if (r.b != pb || scale != psc || (GRAD && r.tile != pt)) {
+        if (pb >= 0) flush();
         acc.zero();
+        if (GRAD && r.b >= 0 && r.b != pb) {
+          const int n = r.b * kSepSpots + row;
+          g = n < p.g.N ? __ldg(p.gE + n) : make_float2(0.0f, 0.0f);
+        }
         pb = r.b;
+        pt = r.tile;
         pscale = scale * kTruncation;
         psc = scale;
       }
@@ -348,8 +481,12 @@ __global__ void __launch_bounds__(kFwdThreads, 1) k_sep_forward(const SepFwdPara
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
       tc_fence_after();
-      if (np > 0)
-        sep_sum_rows(q, strip_mid(r.s, r.ls), tlane + 256u * (it & 1), p0, np, rows == 1 ? (r.s & 1) : -1, acc);
+      const int one = rows == 1 ? (r.s & 1) : -1;
+      if constexpr (GRAD) {
+        sep_moment_rows(q, strip_mid(r.s, r.ls), tlane + 256u * (it & 1), p0, np, one, g, acc);
+      } else {
+        if (np > 0) sep_sum_rows(q, strip_mid(r.s, r.ls), tlane + 256u * (it & 1), p0, np, one, acc);
+      }
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&empty[it & 3]);
@@ -562,6 +699,23 @@ __global__ void __launch_bounds__(kFwdThreads, 1) k_sep_forward(const SepFwdPara
   if (w == 0) tmem_dealloc(tmem, 512);
 }
 
+// dL/dC_nd = the sum of the CTAs' partial rows (as k_sep_forward_reduce).
+__global__ void k_sep_gradc_reduce(const float* __restrict__ part, int rows, int npad, int N, int D,
+                                   float* __restrict__ dC) {
+  __shared__ float acc[16][33];
+  const int n = blockIdx.x * 32 + threadIdx.x, d = blockIdx.y, k = threadIdx.y;
+  float v = 0.0f;
+#pragma unroll 10
+  for (int r = k; r < rows; r += 16) v += __ldg(part + ((size_t)r * D + d) * npad + n);
+  acc[k][threadIdx.x] = v;
+  __syncthreads();
+  for (int h = 8; h > 0; h >>= 1) {
+    if (k < h) acc[k][threadIdx.x] += acc[k + h][threadIdx.x];
+    __syncthreads();
+  }
+  if (k == 0 && n < N) dC[(size_t)n * D + d] = acc[0][threadIdx.x];
+}
+
 // E_n = the sum of the CTAs' partial rows, in a fixed order: row-lane k of the
 // 32 x 32 threads adds rows k, k + 32, ..., then a fixed-shape tree.
 __global__ void k_sep_forward_reduce(const float2* __restrict__ part, int rows, int npad, int N,
@@ -608,8 +762,11 @@ cudaError_t sep_build_params(const Geometry& g, const float* tab, const float* c
 
 cudaError_t sep_prepare() {
   cudaError_t e;
-  if ((e = cudaFuncSetAttribute(k_sep_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFwdSmem))) return e;
-  for (const void* k : {(const void*)k_sep_forward, (const void*)k_sep_forward_reduce, (const void*)k_sep_params})
+  for (const void* k : {(const void*)k_sep_forward<false>, (const void*)k_sep_forward<true>})
+    if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFwdSmem))) return e;
+  for (const void* k : {(const void*)k_sep_forward<false>, (const void*)k_sep_forward<true>,
+                        (const void*)k_sep_forward_reduce, (const void*)k_sep_gradc_reduce, (const void*)k_sep_params,
+                        (const void*)k_sep_scan})
     if ((e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout,
                                   (int)cudaSharedmemCarveoutMaxShared)))
       return e;
@@ -617,10 +774,24 @@ cudaError_t sep_prepare() {
 }
 
 cudaError_t sep_launch_forward(const SepFwdParams& p, cudaStream_t s) {
-  k_sep_forward<<<p.G, kFwdThreads, kFwdSmem, s>>>(p);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  k_sep_forward_reduce<<<(p.g.N + 31) / 32, dim3(32, 32), 0, s>>>(p.part, kSepFwdRows * p.G, p.nb * kSepSpots, p.g.N, p.E);
+  k_sep_forward<false><<<p.G, kFwdThreads, kFwdSmem, s>>>(p);
+  return cudaGetLastError();
+}
+
+cudaError_t sep_launch_forward_reduce(const SepFwdParams& p, cudaStream_t s) {
+  k_sep_forward_reduce<<<(p.g.N + 31) / 32, dim3(32, 32), 0, s>>>(p.part, kSepFwdRows * p.G, p.nb * kSepSpots, p.g.N,
+                                                                  p.E);
+  return cudaGetLastError();
+}
+
+cudaError_t sep_launch_gradc(const SepFwdParams& p, cudaStream_t s) {
+  k_sep_forward<true><<<p.G, kFwdThreads, kFwdSmem, s>>>(p);
+  return cudaGetLastError();
+}
+
+cudaError_t sep_launch_gradc_reduce(const SepFwdParams& p, cudaStream_t s) {
+  k_sep_gradc_reduce<<<dim3((p.g.N + 31) / 32, p.g.D), dim3(32, 16), 0, s>>>(
+      p.dpart, kSepFwdRows * p.G, p.nb * kSepSpots, p.g.N, p.g.D, p.dC);
   return cudaGetLastError();
 }
 

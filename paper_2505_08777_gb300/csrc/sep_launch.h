@@ -53,7 +53,14 @@ struct SepFwdParams {
   float2* E;                     // [N]
   int G;
   unsigned* err;
+  // the moment pass (dL/dC) instead of E
+  const float2* gE;              // [N] dL/dE
+  const float* tab;              // basis polynomials per tile
+  float* dpart;                  // [kSepFwdRows G][D][128 nb] partial sums
+  float* dC;                     // [N][D]
 };
+cudaError_t sep_launch_gradc(const SepFwdParams& p, cudaStream_t s);            // partial sums
+cudaError_t sep_launch_gradc_reduce(const SepFwdParams& p, cudaStream_t s);     // dL/dC from them
 struct SepAdjParams {
   TcAdjParams a;                 // geometry, amplitude, y, outputs
   int nb;
@@ -71,6 +78,7 @@ cudaError_t sep_adjoint_prepare();
 // y divided by a power of two (scale) per chunk of 32 spots.
 cudaError_t sep_launch_scale(const float2* y, int N, float2* ys, float* scale, cudaStream_t s);
 cudaError_t sep_launch_adjoint(const SepAdjParams& p, cudaStream_t s);
-cudaError_t sep_launch_forward(const SepFwdParams& p, cudaStream_t s);   // kernel and reduction
+cudaError_t sep_launch_forward(const SepFwdParams& p, cudaStream_t s);          // partial sums
+cudaError_t sep_launch_forward_reduce(const SepFwdParams& p, cudaStream_t s);   // E from them
 
 }  // namespace ash
