@@ -1031,7 +1031,8 @@ ash_status create_impl(ash_hologram** out, int nx, int ny, int row0, int ny_full
   CREATE_CUDA(enqueue_tc_coeff(h, s));
   k_amp_image<<<g.T, g.NT, 0, s>>>(g, amp, h->amp_img);
   CREATE_CUDA(cudaGetLastError());
-  k_sum_sq<<<1, 1024, 0, s>>>(amp, M, h->sum_a2);
+  k_sum_sq_part<<<kCgRedBlocks, 256, 0, s>>>(amp, M, h->cg_part);
+  k_sum_sq<<<1, kCgRedBlocks, 0, s>>>(h->cg_part, h->sum_a2);
   CREATE_CUDA(cudaGetLastError());
   // stream-ordered allocations and set-up must be complete before the handle
   // is used from another stream (the graph capture stream, or the caller's)
@@ -1191,7 +1192,8 @@ ash_status ash_set_amplitude(ash_hologram* h, const float* amp, void* stream) {
   cudaStream_t s = as_stream(stream);
   k_amp_image<<<h->g.T, h->g.NT, 0, s>>>(h->g, amp, h->amp_img);
   ASH_CUDA(cudaGetLastError());
-  k_sum_sq<<<1, 1024, 0, s>>>(amp, (size_t)h->g.nx * h->g.ny, h->sum_a2);
+  k_sum_sq_part<<<kCgRedBlocks, 256, 0, s>>>(amp, (size_t)h->g.nx * h->g.ny, h->cg_part);
+  k_sum_sq<<<1, kCgRedBlocks, 0, s>>>(h->cg_part, h->sum_a2);
   ASH_CUDA(cudaGetLastError());
   return ASH_OK;
 }

@@ -111,17 +111,32 @@ __device__ __forceinline__ double block_sum(double v, double* red) {
   __syncthreads();
   if (lane == 0) red[w] = v;
   __syncthreads();
-  double s = 0.0;
-  for (int q = 0; q < NTH / 32; ++q) s += red[q];
-  return s;
+  // the warps' sums by the first warp (fp64 is slow here: 2 results per clock
+  // and SM, so 1024 threads do not all add 32 values)
+  if (w == 0) {
+    double s = lane < NTH / 32 ? red[lane] : 0.0;
+    for (int o = 16; o >= 1; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    __syncwarp();
+    if (lane == 0) red[0] = s;
+  }
+  __syncthreads();
+  return red[0];
 }
 
-// sum_m A_m^2 in fp64 (one block).
-static __global__ void k_sum_sq(const float* __restrict__ a, size_t M, double* out) {
+// sum_m A_m^2 in fp64: partial sums of gridDim.x blocks, then their sum (one
+// block of as many threads). With one block over all pixels 1024^2 took 0.8 ms.
+static __global__ void __launch_bounds__(256) k_sum_sq_part(const float* __restrict__ a, size_t M,
+                                                            double* __restrict__ part) {
   __shared__ double red[32];
   double s = 0.0;
-  for (size_t m = threadIdx.x; m < M; m += blockDim.x) s += (double)a[m] * (double)a[m];
-  s = block_sum<1024>(s, red);
+  for (size_t m = (size_t)blockIdx.x * 256 + threadIdx.x; m < M; m += (size_t)gridDim.x * 256)
+    s += (double)a[m] * (double)a[m];
+  s = block_sum<256>(s, red);
+  if (threadIdx.x == 0) part[blockIdx.x] = s;
+}
+static __global__ void __launch_bounds__(512) k_sum_sq(const double* __restrict__ part, double* __restrict__ out) {
+  __shared__ double red[32];
+  const double s = block_sum<512>(part[threadIdx.x], red);
   if (threadIdx.x == 0) *out = s;
 }
 
@@ -288,26 +303,25 @@ __device__ __forceinline__ void spot_loss_body(const float2* __restrict__ E, con
     sI += (double)e.x * e.x + (double)e.y * e.y;
   }
   sI = block_sum<1024>(sI, red);
-  const double mu = sI / N;
+  const double mu = sI / N, inv = mu > 0.0 ? 1.0 / mu : 0.0;
   double sL = 0.0, sR = 0.0;
   for (int n = threadIdx.x; n < N; n += 1024) {
     const float2 e = E[n];
-    const double I = (double)e.x * e.x + (double)e.y * e.y;
-    const double r = (mu > 0.0 ? I / mu : 0.0) - (double)t[n];
+    const double x = ((double)e.x * e.x + (double)e.y * e.y) * inv;
+    const double r = x - (double)t[n];
     sL += r * r;
-    sR += mu > 0.0 ? r * I / mu : 0.0;
+    sR += r * x;
   }
   sL = block_sum<1024>(sL, red);
   sR = block_sum<1024>(sR, red);
   if (threadIdx.x == 0 && loss) *loss = (float)sL;
   if (!gE) return;
-  const double c = sR / N;
+  const double c = sR / N, f = 4.0 * inv;
   for (int n = threadIdx.x; n < N; n += 1024) {
     const float2 e = E[n];
-    const double I = (double)e.x * e.x + (double)e.y * e.y;
-    const double r = (mu > 0.0 ? I / mu : 0.0) - (double)t[n];
-    const double G = mu > 0.0 ? (2.0 / mu) * (r - c) : 0.0;
-    gE[n] = make_float2((float)(2.0 * G * e.x), (float)(2.0 * G * e.y));
+    const double x = ((double)e.x * e.x + (double)e.y * e.y) * inv;
+    const double G = f * ((x - (double)t[n]) - c);
+    gE[n] = make_float2((float)(G * e.x), (float)(G * e.y));
   }
 }
 
