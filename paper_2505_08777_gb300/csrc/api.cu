@@ -928,12 +928,12 @@ ash_status create_impl(ash_hologram** out, int nx, int ny, int row0, int ny_full
   if (h->sep_ok) {
     const size_t npad = (size_t)sep_blocks(N) * kSepSpots;
     if ((st = ws(h, &h->sep_tab, (size_t)g.T * D * kSepTab)) != ASH_OK) return fail(st);
-    if ((st = ws(h, &h->sep_poly, (size_t)g.T * 4 * npad)) != ASH_OK) return fail(st);
+    if ((st = ws(h, &h->sep_poly, (size_t)g.T * 16 * npad)) != ASH_OK) return fail(st);
     if ((st = ws(h, &h->sep_strips, (size_t)g.T * sep_blocks(N))) != ASH_OK) return fail(st);
     if ((st = ws(h, &h->sep_cost, (size_t)g.T * sep_blocks(N) + 1)) != ASH_OK) return fail(st);
     if ((st = ws(h, &h->sep_acost, (size_t)g.T * sep_blocks(N) + 2)) != ASH_OK) return fail(st);
     if ((st = ws(h, &h->sep_split, 2 * (size_t)h->sep_G * kTilePix)) != ASH_OK) return fail(st);
-    if ((st = ws(h, &h->sep_ys, npad)) != ASH_OK) return fail(st);
+    if ((st = ws(h, &h->sep_ys, 2 * npad)) != ASH_OK) return fail(st);
     if ((st = ws(h, &h->sep_scale, npad / kSepChunk)) != ASH_OK) return fail(st);
     const size_t dp = (size_t)kSepFwdRows * h->sep_G * D * npad;
     if (dp * sizeof(float) <= kSepMaxBytes / 8 && (st = ws(h, &h->sep_dpart, dp)) != ASH_OK) return fail(st);

@@ -69,14 +69,14 @@ struct ash_hologram {
   int sep_ord = 0;              // total degree of the basis
   int sep_G = 0;                // forward CTAs
   float* sep_tab = nullptr;     // basis polynomials per tile
-  float4* sep_poly = nullptr;   // phase polynomials per (tile, spot)
+  float* sep_poly = nullptr;    // phase polynomials per (tile, spot)
   unsigned char* sep_strips = nullptr;   // per (tile, spot block): log2 of its row strips
   float* sep_dpart = nullptr;   // [kSepFwdRows sep_G][D][128 nb] partial dL/dC
   int* sep_cost = nullptr;      // prefix of its forward steps' cost
   int* sep_acost = nullptr;     // prefix of its adjoint chunks' cost
   float2* sep_split = nullptr;  // [sep_G][2][kTilePix] adjoint sums of tiles split between CTAs
   int* sep_tickets = nullptr;   // [T]
-  float2* sep_ys = nullptr;     // [128 nb] y of an adjoint, scaled, and the scale per 32 spots
+  float* sep_ys = nullptr;      // [128 nb] y of an adjoint, scaled, and the scale per 32 spots
   float* sep_scale = nullptr;
   float2* sep_part = nullptr;   // [kSepFwdRows sep_G][128 nb]
   float2* split = nullptr;

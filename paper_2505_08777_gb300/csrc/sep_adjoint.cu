@@ -13,10 +13,12 @@ namespace ash {
 namespace {
 
 // One CTA per SM, 28 warps. Warps 0-7 (adders): lane = tile row, warp w adds
-// up half of the columns of the plane u^(w % 4); warp 8 issues the MMAs, warp
-// 9 lists the steps and fetches their spots; warps 12-19 and 20-27
-// (generators, taking turns step by step): lane = spot, four tile rows and
-// four tile columns each. A step is 32 spots of a tile and one strip of its
+// up half of the columns of the plane u^(w % 4); warp 8 lists the steps and
+// fetches their spots, warps 9-11 issue the MMAs of every third step each (one
+// issuer spent 2400 clocks a step, mostly on its waits: operands were always
+// ready); warps 12-19 and 20-27
+// (generators, taking turns step by step): two spots (in the halves of the
+// packed operations), two tile rows and two tile columns each. A step is 32 spots of a tile and one strip of its
 // rows (the strips of a chunk share W). A: rows (k, tile row), (Re W, Im W) of
 // the 32 spots; low parts for k = 0, 1 only (|Q_2|, |Q_3| < 0.01). B: rows
 // (column, re / im), (Re X, -Im X) and (Im X, Re X), high then low parts.
@@ -30,16 +32,29 @@ constexpr uint32_t kAA = 32768, kAB = 16384, kASlot = 2048 + 256;
 constexpr uint32_t kAdjB = kAdjBufs * kAA, kAdjSum = kAdjB + kAdjBufs * kAB;   // sums of the planes: [4][32][33] float2
 constexpr uint32_t kAdjSlot0 = kAdjSum + 4 * 32 * 33 * 8, kAdjTail = kAdjSlot0 + kAdjSlots * kASlot;
 constexpr size_t kAdjSmem = 1024 + kAdjTail + 512;
-static_assert(28 * 8 + 16 + kAdjSlots * 24 <= 512);
+static_assert(30 * 8 + 16 + kAdjSlots * 16 <= 512 && kAdjTail % 16 == 0);
 static_assert(kAdjSum % 16 == 0 && kAdjSlot0 % 16 == 0 && kAdjTail % 8 == 0);
 
-struct AdjStep {
-  int tile;      // -1: no more steps
-  int s, ls;     // strip s of 2^ls
-  int a;         // buffer of W
-  int end;       // bits: 1 the CTA's last step of this tile, 2 other CTAs have part of it, 4 it starts here
-  float scale;   // 2^e: y is divided by it
+// A step's record, read as one 16-byte word.
+struct __align__(16) AdjStep {
+  int tile;        // negative: no more steps
+  uint32_t bits;   // s | ls << 8 | a << 16 | end << 18: strip s of 2^ls, buffer of W
+  int used;        // the last step that used that buffer before this chunk (negative: none)
+  float scale;     // 2^e: y is divided by it
+  __device__ int s() const { return (int)(bits & 255u); }
+  __device__ int ls() const { return (int)(bits >> 8 & 255u); }
+  __device__ uint32_t a() const { return bits >> 16 & 3u; }
+  // bits: 1 the CTA's last step of this tile, 2 other CTAs have part of it, 4
+  // it starts here, 8 the CTA's last step
+  __device__ int end() const { return (int)(bits >> 18); }
 };
+__device__ __forceinline__ AdjStep adj_step(const AdjStep* p) {
+  const int4 v = *reinterpret_cast<const int4*>(p);
+  return AdjStep{v.x, (uint32_t)v.y, v.z, __int_as_float(v.w)};
+}
+__device__ __forceinline__ void put_step(AdjStep* p, int tile, uint32_t bits, int used, float scale) {
+  *reinterpret_cast<int4*>(p) = make_int4(tile, (int)bits, used, __float_as_int(scale));
+}
 
 // (see kTruncation of the forward: here -1.5e-7)
 constexpr float kAdjTruncation = 1.0f + 1.2e-7f;
@@ -49,8 +64,8 @@ struct IntTag {
   static constexpr int value = V;
 };
 template <int OFF>
-__device__ __forceinline__ void sts32(uint32_t addr, uint32_t v) {
-  asm volatile("st.shared.u32 [%0 + %1], %2;" ::"r"(addr), "n"(OFF), "r"(v) : "memory");
+__device__ __forceinline__ void sts64(uint32_t addr, uint32_t a, uint32_t b) {
+  asm volatile("st.shared.v2.u32 [%0 + %1], {%2, %3};" ::"r"(addr), "n"(OFF), "r"(a), "r"(b) : "memory");
 }
 
 // CTA whose range [W g / G, W (g + 1) / G) holds position c.
@@ -68,7 +83,8 @@ __global__ void __launch_bounds__(kAdjThreads, 1) k_sep_adjoint(const SepAdjPara
   uint64_t* empty = full + 4;                                    // [8] its D and record read
   uint64_t* ready = full + 12;                                   // [8] its operands written
   uint64_t* listed = full + 20;                                  // [8] its record and spots written
-  uint32_t* slot = reinterpret_cast<uint32_t*>(full + 28);
+  uint64_t* summed = full + 28;                                  // the adders' meeting point at a tile's end
+  uint32_t* slot = reinterpret_cast<uint32_t*>(full + 30);
   AdjStep* steps = reinterpret_cast<AdjStep*>(slot + 4);         // [8]
   const int t = threadIdx.x, w = t >> 5, lane = t & 31;
   const int N = p.a.g.N, nb = p.nb, npad = nb * kSepSpots, U = p.a.g.T * nb;
@@ -77,7 +93,7 @@ __global__ void __launch_bounds__(kAdjThreads, 1) k_sep_adjoint(const SepAdjPara
     reinterpret_cast<uint4*>(sm + (k >> 9) * kAA + 16384 + 8192)[k & 511] = make_uint4(0, 0, 0, 0);
   if (w == 0) tmem_alloc(slot, 512);
   if (t == 0) {
-    for (int k = 0; k < 28; ++k) mbar_init(full + k, k >= 4 && k < 12 ? 8 : 1);
+    for (int k = 0; k < 29; ++k) mbar_init(full + k, (k >= 4 && k < 12) || k == 28 ? 8 : 1);
     fence_mbar_init();
   }
   fence_async_smem();
@@ -95,28 +111,26 @@ __global__ void __launch_bounds__(kAdjThreads, 1) k_sep_adjoint(const SepAdjPara
     const int pl = w & 3, hc = w >> 2;
     const uint32_t ta = tmem + ((uint32_t)(pl * 32) << 16) + 32u * hc;
     float2* sums = reinterpret_cast<float2*>(sm + kAdjSum);
-    auto add_sync = [&]() { asm volatile("bar.sync 1, 256;" ::: "memory"); };
+    // (an mbarrier, not a named one: a warp whose wait runs out leaves alone)
+    uint32_t meets = 0;
+    auto add_sync = [&]() {
+      __syncwarp();
+      if (lane == 0) mbar_arrive(summed);
+      ok = ok && sep_wait(summed, meets & 1);
+      ++meets;
+    };
     float2 acc[16];
 #pragma unroll
     for (int i = 0; i < 16; ++i) acc[i] = make_float2(0.0f, 0.0f);
-    for (uint32_t it = 0;; ++it) {
+    for (uint32_t it = 0; blockIdx.x < G; ++it) {
       const int sl = it & 7, d = it & 3;
-      ok = ok && mbar_wait(&listed[sl], (it >> 3) & 1, kTcWaitPolls);
-      AdjStep x{-1, 0, 0, 0, 0, 0.0f};
-      if (ok) x = steps[sl];
-      if (x.tile >= 0) ok = mbar_wait(&full[d], (it >> 2) & 1, kTcWaitPolls) && ok;
-      // the eight warps go on or stop together
-      int stop;
-      asm volatile(
-          "{\n\t.reg .pred p, q;\n\tsetp.lt.s32 p, %1, 0;\n\tbarrier.red.or.pred q, 1, 256, p;\n\t"
-          "selp.s32 %0, 1, 0, q;\n\t}"
-          : "=r"(stop)
-          : "r"(ok ? x.tile : -1)
-          : "memory");
-      if (stop) break;
+      ok = ok && sep_wait(&full[d], (it >> 2) & 1);
+      ok = __all_sync(0xffffffffu, ok);
+      if (!ok) break;
+      const AdjStep x = adj_step(steps + sl);
       tc_fence_after();
-      const int n = 32 >> x.ls;
-      const float f = (lane >= x.s * n && lane < (x.s + 1) * n) ? x.scale : 0.0f;
+      const int n = 32 >> x.ls();
+      const float f = (lane >= x.s() * n && lane < (x.s() + 1) * n) ? x.scale : 0.0f;
 #pragma unroll
       for (int h = 0; h < 4; ++h) {
         uint32_t a[8], b[8];
@@ -133,7 +147,7 @@ __global__ void __launch_bounds__(kAdjThreads, 1) k_sep_adjoint(const SepAdjPara
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&empty[sl]);
-      if (!x.end) continue;
+      if (!x.end()) continue;
       // sum of the planes; then thread: pixels (row q * 8 + w, column lane)
       float2* mine = sums + (size_t)(pl * 32 + lane) * 33 + 16 * hc;
 #pragma unroll
@@ -155,10 +169,10 @@ __global__ void __launch_bounds__(kAdjThreads, 1) k_sep_adjoint(const SepAdjPara
         v[q] = add2(add2(s[0], s[32 * 33]), add2(s[2 * 32 * 33], s[3 * 32 * 33]));
       }
       bool out = true;
-      if (x.end & 2) {
+      if (x.end() & 2) {
         // a split tile: the last of its CTAs adds up the partial sums (a
         // CTA's second buffer is that of the tile that starts in it)
-        float2* dst = p.split + ((size_t)blockIdx.x * 2 + (x.end & 4 ? 1 : 0)) * kTilePix + w * 32 + lane;
+        float2* dst = p.split + ((size_t)blockIdx.x * 2 + (x.end() & 4 ? 1 : 0)) * kTilePix + w * 32 + lane;
 #pragma unroll
         for (int q = 0; q < 4; ++q) dst[q * 256] = v[q];
         __threadfence();
@@ -212,26 +226,31 @@ __global__ void __launch_bounds__(kAdjThreads, 1) k_sep_adjoint(const SepAdjPara
           }
         }
       }
+      if (x.end() & 8) break;
       add_sync();   // `sums` is rewritten at the next tile's end
     }
   } else if (w < 12) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
-    if (w == 8 && lane == 0) {
-      // --- MMA issue ---
-      uint32_t it = 0, bi = 0;
-      for (;; ++it, bi = bi == kAdjBufs - 1 ? 0 : bi + 1) {
+    if (w > 8 && lane == 0) {
+      // --- MMA issue: steps w - 9, w - 6, .. (their X is in buffer w - 9) ---
+      static_assert(kAdjBufs == 3);
+      uint32_t it = (uint32_t)(w - 9);
+      for (;; it += 3) {
         const int sl = it & 7, d = it & 3;
-        ok = ok && mbar_wait(&listed[sl], (it >> 3) & 1, kTcWaitPolls);
+        ok = ok && sep_wait(&ready[sl], (it >> 3) & 1);
         if (!ok) break;
-        const AdjStep x = steps[sl];
+        const AdjStep x = adj_step(steps + sl);
         if (x.tile < 0) break;
-        ok = ok && mbar_wait(&ready[sl], (it >> 3) & 1, kTcWaitPolls);
-        if (it >= 4) ok = ok && mbar_wait(&empty[(it - 4) & 7], ((it - 4) >> 3) & 1, kTcWaitPolls);
+        // W came with the chunk's first step (for s > 3 this thread's own last
+        // step, it - 3, has waited for it)
+        if (x.s() >= 1 && x.s() <= 3)
+          ok = ok && sep_wait(&ready[(it - x.s()) & 7], ((it - x.s()) >> 3) & 1);
+        if (it >= 4) ok = ok && sep_wait(&empty[(it - 4) & 7], ((it - 4) >> 3) & 1);
         if (!ok) break;
         tc_fence_after();
         const uint32_t dst = tmem + 128u * d;
-        const uint64_t a = umma_desc(smem_u32(sm) + (uint32_t)x.a * kAA), al = a + (16384 >> 4);
-        const uint64_t b = umma_desc(smem_u32(sm + kAdjB) + bi * kAB);
+        const uint64_t a = umma_desc(smem_u32(sm) + x.a() * kAA), al = a + (16384 >> 4);
+        const uint64_t b = umma_desc(smem_u32(sm + kAdjB) + (uint32_t)(w - 9) * kAB);
 #pragma unroll
         for (int ks = 0; ks < 8; ks += 2) umma_f16(dst, a + ks, b + ks, umma_idesc_f16(128, 128), ks > 0);
 #pragma unroll
@@ -239,8 +258,8 @@ __global__ void __launch_bounds__(kAdjThreads, 1) k_sep_adjoint(const SepAdjPara
         umma_commit(&full[d]);
       }
       // nothing in flight when the CTA gives up its memory
-      for (uint32_t k = it > 3 ? it - 3 : 0; k < it; ++k) ok = mbar_wait(&full[k & 3], (k >> 2) & 1, kTcWaitPolls) && ok;
-    } else if (w == 9 && lane == 0) {
+      if (it >= 3) ok = sep_wait(&full[(it - 3) & 3], ((it - 3) >> 2) & 1) && ok;
+    } else if (w == 8 && lane == 0) {
       // --- steps of this CTA: the chunks whose place in the cost prefix lies in [c0, c1) ---
       const int c0 = blockIdx.x < G ? (int)(W * blockIdx.x / G) : 0;
       const int c1 = blockIdx.x < G ? (int)(W * (blockIdx.x + 1) / G) : 0;
@@ -254,6 +273,7 @@ __global__ void __launch_bounds__(kAdjThreads, 1) k_sep_adjoint(const SepAdjPara
       int cc = sep_chunk_cost(ls), c = (c0 - pos + cc - 1) / cc, s = 0, a = 0;
       pos += c * cc;
       int ls1 = u + 1 < U ? p.strips[u + 1] : 0;   // of the next unit, fetched early
+      int used[kAdjBufs] = {-1, -1, -1};   // last steps of the last three chunks
       uint32_t it = 0;
       for (;; ++it) {
         const int sl = it & 7;
@@ -271,131 +291,145 @@ __global__ void __launch_bounds__(kAdjThreads, 1) k_sep_adjoint(const SepAdjPara
         const bool more = s > 0 || pos < c1;
         const int chunk = b * (kSepSpots / kSepChunk) + c;
         const float sc = more ? __ldg(p.scale + chunk) : 0.0f;
-        if (it >= 8) ok = ok && mbar_wait(&empty[sl], ((it >> 3) - 1) & 1, kTcWaitPolls);
         if (!more) {
-          // an end for each of the two groups of generators
-          steps[sl] = AdjStep{-1, 0, 0, 0, 0, 0.0f};
-          mbar_arrive(&listed[sl]);
-          const int s2 = (it + 1) & 7;
-          if (it >= 7) ok = ok && mbar_wait(&empty[s2], (((it + 1) >> 3) - 1) & 1, kTcWaitPolls);
-          steps[s2] = AdjStep{-1, 0, 0, 0, 0, 0.0f};
-          mbar_arrive(&listed[s2]);
+          // an end for each group of generators (-1, -2) and each issuer
+          for (uint32_t k = it; k < it + 3; ++k)
+            if (k >= 8) ok = ok && sep_wait(&empty[k & 7], ((k >> 3) - 1) & 1);
+          for (uint32_t k = it; k < it + 3; ++k) put_step(steps + (k & 7), -1 - (int)(k - it), 0, -1, 0.0f);
+          mbar_arrive(&listed[it & 7]);
+          mbar_arrive(&listed[(it + 1) & 7]);
           break;
         }
+        if (it >= 8) ok = ok && sep_wait(&empty[sl], ((it >> 3) - 1) & 1);
         uint8_t* dst = sm + kAdjSlot0 + sl * kASlot;
-        AdjStep x{tile, s, ls, a, 0, sc};
+        uint32_t end = 0;
         if (((s + 1) >> ls) && (pos + cc >= c1 || (c + 1 == sep_chunks(N, b) && b + 1 == nb))) {
           const int t1 = p.cost[(tile + 1) * nb] - sep_chunk_cost(p.strips[(tile + 1) * nb - 1]);
           const bool here = c0 <= p.cost[tile * nb];
-          x.end = 1 | (here && t1 < c1 ? 0 : 2) | (here ? 4 : 0);
+          end = 1u | (here && t1 < c1 ? 0u : 2u) | (here ? 4u : 0u) | (pos + cc >= c1 ? 8u : 0u);
         }
-        steps[sl] = x;
+        put_step(steps + sl, tile, (uint32_t)s | (uint32_t)ls << 8 | (uint32_t)a << 16 | end << 18, used[0], sc);
         mbar_expect_tx(&listed[sl], kASlot);
-        bulk_g2s(dst, p.poly + ((size_t)tile * (npad / kSepChunk) + chunk) * 128, 2048, &listed[sl]);
-        bulk_g2s(dst + 2048, p.ys + chunk * kSepChunk, 256, &listed[sl]);
+        bulk_g2s(dst, p.poly + ((size_t)tile * (npad / kSepChunk) + chunk) * 512, 2048, &listed[sl]);
+        bulk_g2s(dst + 2048, p.ys + chunk * 64, 256, &listed[sl]);
         if (++s >> ls) {
           s = 0;
           ++c;
           pos += cc;
           a = a == kAdjBufs - 1 ? 0 : a + 1;
+          used[0] = used[1];
+          used[1] = used[2];
+          used[2] = (int)it;
         }
       }
-      for (uint32_t k = it > 6 ? it - 6 : 0; k < it; ++k) ok = mbar_wait(&listed[k & 7], (k >> 3) & 1, kTcWaitPolls) && ok;
+      for (uint32_t k = it > 5 ? it - 5 : 0; k < it; ++k) ok = sep_wait(&listed[k & 7], (k >> 3) & 1) && ok;
     }
   } else {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 80;");
-    // --- generators: spot `lane`, tile rows and columns 4 gw .. 4 gw + 3 ---
-    const int group = (w - 12) >> 3, gw = (w - 12) & 7;
-    // The spot's 4 bytes in a row r (r = 8 a + e) of a 128-byte-swizzled operand
-    // lie at row + (place ^ (e << 4)). W: rows k 32 + 4 gw + c, X: rows 8 gw + e.
-    const uint32_t place = (uint32_t)lane * 4;
-    const uint32_t w0 = smem_u32(sm) + (uint32_t)gw * 512 + (place ^ ((uint32_t)(gw & 1) << 6));
-    const uint32_t x0 = smem_u32(sm + kAdjB) + (uint32_t)gw * 1024 + place;
+    // --- generators: spots 2 sp, 2 sp + 1 (as pairs), tile rows and columns j0, j0 + 1 ---
+    const int group = (w - 12) >> 3, gw = (w - 12) & 7, sp = lane & 15, hr = lane >> 4, j0 = 4 * gw + 2 * hr;
+    // The spots' 8 bytes in a row r (r = 8 a + e) of a 128-byte-swizzled operand
+    // lie at row + (place ^ (e << 4)). W: rows k 32 + j0 + c, X: rows 2 j0 + e.
+    const uint32_t place = (uint32_t)sp * 8;
+    const uint32_t w0 = smem_u32(sm) + (uint32_t)j0 * 128 + (place ^ ((uint32_t)(j0 & 7) << 4));
+    const uint32_t x0 = smem_u32(sm + kAdjB) + (uint32_t)j0 * 256 + (place ^ ((uint32_t)(j0 & 2) << 5));
     uint32_t bi = group;
     for (uint32_t it = group;; it += 2, bi = bi == 0 ? 2 : bi - 1) {
       const int sl = it & 7;
-      ok = ok && mbar_wait(&listed[sl], (it >> 3) & 1, kTcWaitPolls);
-      // the MMAs of step it - 3 are done: its X, and W of an older chunk, are free
-      if (it >= 3) ok = ok && mbar_wait(&full[(it - 3) & 3], ((it - 3) >> 2) & 1, kTcWaitPolls);
-      AdjStep x{-1, 0, 0, 0, 0, 0.0f};
-      if (ok) x = steps[sl];
+      ok = ok && sep_wait(&listed[sl], (it >> 3) & 1);
+      // the MMAs of step it - 3 are done: its X is free
+      if (it >= 3) ok = ok && sep_wait(&full[(it - 3) & 3], ((it - 3) >> 2) & 1);
+      AdjStep x{-4, 0u, -1, 0.0f};
+      if (ok) x = adj_step(steps + sl);
       if (x.tile >= 0) {
-        const float4* sq = reinterpret_cast<const float4*>(sm + kAdjSlot0 + sl * kASlot) + lane;
-        const SepPoly q = sep_unpack(sq[0], sq[32], sq[64], sq[96]);
-        if (x.s == 0) {
-          const float2 y = reinterpret_cast<const float2*>(sm + kAdjSlot0 + sl * kASlot + 2048)[lane];
-          const uint32_t ah = w0 + (uint32_t)x.a * kAA;
+        const int xs = x.s(), xl = x.ls();
+        const uint8_t* sd = sm + kAdjSlot0 + sl * kASlot;
+        auto word = [&](int k) { return *reinterpret_cast<const float2*>(sd + 128 * k + 8 * sp); };
+        const float2 lo = word(kWLow);
+        const float2 c11 = word(kWC11), c21 = word(kWC21), c12 = word(kWC12), c22 = word(kWC22), n31 = word(kWN31),
+                     c13 = word(kWC13);
+        if (xs == 0) {
+          // W's buffer: the MMAs of its last user are done (step it - 3: above;
+          // more than 7 steps ago: the record's slot was free; they are issued by
+          // three threads, so a later step's say nothing)
+          if (x.used >= 0 && (int)it - x.used > 3 && (int)it - x.used < 8)
+            ok = ok && sep_wait(&empty[x.used & 7], (x.used >> 3) & 1);
+          const float2 yr = word(16), yi = word(17), nyi = sub2(make_float2(0.0f, 0.0f), yi);
+          const float2 base = word(kWBase), ay = word(kWAy), y2 = word(kWY2), y3 = word(kWY3), y4 = word(kWY4);
+          const float2 ayl = make_float2(__uint_as_float(__float_as_uint(lo.x) & 0xffff0000u),
+                                         __uint_as_float(__float_as_uint(lo.y) & 0xffff0000u));
+          const uint32_t ah = w0 + x.a() * kAA;
 #pragma unroll
-          for (int pr = 0; pr < 2; ++pr) {
-          const int j = 4 * gw + 2 * pr;
-          const float2 m = make_float2((float)(j - 16), (float)(j - 15));
-          // the rows' strip: its middle row carries the mixed terms of X
-          const int n = 32 >> x.ls;
-          const float ms = strip_mid(j / n, x.ls), ms1 = strip_mid((j + 1) / n, x.ls);
-          const float2 mid = make_float2(ms, ms1);
-          auto R1of = [&](float2 v) { return mul2(fma2(fma2(dup2(q.c13), v, dup2(q.c12)), v, dup2(q.c11)), v); };
-          auto R2of = [&](float2 v) { return mul2(fma2(dup2(q.c22), v, dup2(q.c21)), v); };
-          float2 R1 = R1of(m), R2 = R2of(m), n3 = mul2(dup2(q.n31), m);
-          if (x.ls) {
-            R1 = fma2(R1of(mid), dup2(-1.0f), R1);
-            R2 = fma2(R2of(mid), dup2(-1.0f), R2);
-            n3 = fma2(dup2(-q.n31), mid, n3);
-          }
-          // exp(+i r) = 1 + i R1 u + (q2r + i q2i) u^2 + (q3r + i q3i) u^3
-          const float2 s2 = mul2(R1, R1), n1 = mul2(R1, dup2(-1.0f));
-          const float2 q2r = fma2(s2, fma2(s2, dup2(1.0f / 24.0f), dup2(-0.5f)), mul2(R2, mul2(R2, dup2(-0.5f))));
-          const float2 q2i = mul2(R2, fma2(s2, dup2(-0.5f), dup2(1.0f)));
-          const float2 q3r = mul2(n1, R2), n3i = fma2(mul2(R1, s2), dup2(1.0f / 6.0f), n3);   // -q3i
-          float2 c, sn;
-          cis2(sep_angle(q.ay, -q.ay, q.ayl, q.y2, q.y3, q.y4, q.base, -q.base, m), c, sn);
-          // (a complex product: the phase of y, carried from iteration to iteration
-          // by a WGS loop, keeps its fp32 accuracy)
-          const float2 wr = fma2(sn, dup2(-y.y), mul2(c, dup2(y.x))), wi = fma2(c, dup2(y.y), mul2(sn, dup2(y.x)));
-          // rows c = 2 pr, 2 pr + 1 of the thread's four
-          const uint32_t r0 = ah ^ (uint32_t)(pr << 5), r1 = ah ^ (uint32_t)(pr << 5 | 16);
-          auto emit = [&](auto kk, float2 re, float2 im) {
-            constexpr int k = decltype(kk)::value;
-            constexpr int o0 = k * 4096, lo = 16384;
-            if constexpr (k < 2) {
-              const float2 hr = split_hi2(re), hi = split_hi2(im);
-              const float2 lr = fma2(hr, dup2(-1.0f), re), li = fma2(hi, dup2(-1.0f), im);
-              sts32<o0>(r0 + 256 * pr, pack_f16(hr.x, hi.x));
-              sts32<o0 + 128>(r1 + 256 * pr, pack_f16(hr.y, hi.y));
-              sts32<o0 + lo>(r0 + 256 * pr, pack_f16(lr.x, li.x));
-              sts32<o0 + lo + 128>(r1 + 256 * pr, pack_f16(lr.y, li.y));
-            } else {
-              sts32<o0>(r0 + 256 * pr, pack_f16(re.x, im.x));
-              sts32<o0 + 128>(r1 + 256 * pr, pack_f16(re.y, im.y));
+          for (int c = 0; c < 2; ++c) {
+            const float2 m = dup2((float)(j0 + c - 16));
+            float2 R1 = mul2(fma2(fma2(c13, m, c12), m, c11), m);
+            float2 R2 = mul2(fma2(c22, m, c21), m);
+            float2 n3 = mul2(n31, m);
+            if (xl) {
+              // about the middle row of the row's strip: the rest is in X
+              const float2 v = dup2(strip_mid((j0 + c) / (32 >> xl), xl)), nv = sub2(make_float2(0.0f, 0.0f), v);
+              R1 = fma2(fma2(fma2(c13, v, c12), v, c11), nv, R1);
+              R2 = fma2(fma2(c22, v, c21), nv, R2);
+              n3 = fma2(n31, nv, n3);
             }
-          };
-          emit(IntTag<0>{}, wr, wi);
-          emit(IntTag<1>{}, mul2(n1, wi), mul2(R1, wr));
-          const float2 nwi = mul2(wi, dup2(-1.0f));
-          emit(IntTag<2>{}, fma2(q2r, wr, mul2(q2i, nwi)), fma2(q2r, wi, mul2(q2i, wr)));
-          emit(IntTag<3>{}, fma2(q3r, wr, mul2(n3i, wi)), fma2(q3r, wi, mul2(n3i, mul2(wr, dup2(-1.0f)))));
+            // exp(+i r) = 1 + i R1 u + (q2r + i q2i) u^2 + (q3r + i q3i) u^3
+            const float2 s2 = mul2(R1, R1), n1 = sub2(make_float2(0.0f, 0.0f), R1);
+            const float2 q2r = fma2(s2, fma2(s2, dup2(1.0f / 24.0f), dup2(-0.5f)), mul2(R2, mul2(R2, dup2(-0.5f))));
+            const float2 q2i = mul2(R2, fma2(s2, dup2(-0.5f), dup2(1.0f)));
+            const float2 q3r = mul2(n1, R2), n3i = fma2(mul2(R1, s2), dup2(1.0f / 6.0f), n3);   // -q3i
+            float2 cs, sn;
+            cis2(sep_angle(ay, ayl, y2, y3, y4, base, m), cs, sn);
+            // (a complex product: the phase of y, carried from iteration to
+            // iteration by a WGS loop, keeps its fp32 accuracy)
+            const float2 wr = fma2(sn, nyi, mul2(cs, yr)), wi = fma2(cs, yi, mul2(sn, yr));
+            const uint32_t at = (ah ^ (uint32_t)(c << 4)) + 128 * c;
+            auto emit = [&](auto kk, float2 re, float2 im) {
+              constexpr int k = decltype(kk)::value, o = k * 4096;
+              if constexpr (k < 2) {
+                const float2 hr2 = split_hi2(re), hi2 = split_hi2(im);
+                const float2 lr2 = sub2(re, hr2), li2 = sub2(im, hi2);
+                sts64<o>(at, pack_f16(hr2.x, hi2.x), pack_f16(hr2.y, hi2.y));
+                sts64<o + 16384>(at, pack_f16(lr2.x, li2.x), pack_f16(lr2.y, li2.y));
+              } else {
+                sts64<o>(at, pack_f16(re.x, im.x), pack_f16(re.y, im.y));
+              }
+            };
+            const float2 nwi = sub2(make_float2(0.0f, 0.0f), wi), nwr = sub2(make_float2(0.0f, 0.0f), wr);
+            emit(IntTag<0>{}, wr, wi);
+            emit(IntTag<1>{}, mul2(R1, nwi), mul2(R1, wr));
+            emit(IntTag<2>{}, fma2(q2r, wr, mul2(q2i, nwi)), fma2(q2r, wi, mul2(q2i, wr)));
+            emit(IntTag<3>{}, fma2(q3r, wr, mul2(n3i, wi)), fma2(q3r, wi, mul2(n3i, nwr)));
           }
         }
-        const SepColumns o = sep_columns(q, x.s, x.ls);
+        float2 ax = word(kWAx), x2 = word(kWX2), x3 = word(kWX3);
+        float2 axl = make_float2(__uint_as_float(__float_as_uint(lo.x) << 16), __uint_as_float(__float_as_uint(lo.y) << 16));
+        if (xl) {
+          // about the strip's middle row (sep_columns)
+          const float2 v = dup2(strip_mid(xs, xl));
+          const float2 R1 = mul2(fma2(fma2(c13, v, c12), v, c11), v), R2 = mul2(fma2(c22, v, c21), v);
+          const float2 d = mul2(R1, dup2(0.15915494309189535f * 0.0625f));
+          const float2 a = add2(ax, d), z = sub2(a, ax);
+          const float2 e = add2(fma2(sub2(a, z), dup2(-1.0f), ax), sub2(d, z));
+          axl = fma2(e, dup2(6.283185307179586f), axl);
+          ax = a;
+          x2 = fma2(R2, dup2(0.0625f * 0.0625f), x2);
+          x3 = fma2(mul2(n31, v), dup2(-0.0625f * 0.0625f * 0.0625f), x3);
+        }
+        const float2 x4 = word(kWX4);
         const uint32_t bh = x0 + bi * kAB;
         constexpr uint32_t S = 0x80000000u;   // the sign of the upper half
 #pragma unroll
-        for (int pr = 0; pr < 2; ++pr) {
-          const int i = 4 * gw + 2 * pr;
-          const float2 m = make_float2((float)(i - 16), (float)(i - 15));
-          float2 c, sn;
-          cis2(sep_angle(o.ax, -o.ax, o.axl, o.x2, o.x3, o.x4, m), c, sn);
-          const float2 hc = split_hi2(c), hs = split_hi2(sn);
-          const float2 lc = fma2(hc, dup2(-1.0f), c), ls = fma2(hs, dup2(-1.0f), sn);
-          // rows e = 4 pr .. 4 pr + 3: (re, im) of column i, then of i + 1
-          const uint32_t b0 = (bh ^ (uint32_t)(pr << 6)) + 512 * pr;
-          sts32<0>(b0, pack_f16(hc.x, hs.x) ^ S);
-          sts32<128>(b0 ^ 16u, pack_f16(hs.x, hc.x));
-          sts32<256>(b0 ^ 32u, pack_f16(hc.y, hs.y) ^ S);
-          sts32<384>(b0 ^ 48u, pack_f16(hs.y, hc.y));
-          sts32<8192>(b0, pack_f16(lc.x, ls.x) ^ S);
-          sts32<8192 + 128>(b0 ^ 16u, pack_f16(ls.x, lc.x));
-          sts32<8192 + 256>(b0 ^ 32u, pack_f16(lc.y, ls.y) ^ S);
-          sts32<8192 + 384>(b0 ^ 48u, pack_f16(ls.y, lc.y));
+        for (int c = 0; c < 2; ++c) {
+          float2 cs, sn;
+          cis2(sep_angle(ax, axl, x2, x3, x4, dup2((float)(j0 + c - 16))), cs, sn);
+          const float2 hc = split_hi2(cs), hs = split_hi2(sn);
+          const float2 lc = sub2(cs, hc), lsn = sub2(sn, hs);
+          // rows 2 (j0 + c): (re, -im), and the next: (im, re)
+          const uint32_t b0 = (bh ^ (uint32_t)(c << 5)) + 256 * c, b1 = (bh ^ (uint32_t)(c << 5 | 16)) + 256 * c;
+          sts64<0>(b0, pack_f16(hc.x, hs.x) ^ S, pack_f16(hc.y, hs.y) ^ S);
+          sts64<128>(b1, pack_f16(hs.x, hc.x), pack_f16(hs.y, hc.y));
+          sts64<8192>(b0, pack_f16(lc.x, lsn.x) ^ S, pack_f16(lc.y, lsn.y) ^ S);
+          sts64<8192 + 128>(b1, pack_f16(lsn.x, lc.x), pack_f16(lsn.y, lc.y));
         }
         fence_async_smem();
       }
@@ -407,7 +441,10 @@ __global__ void __launch_bounds__(kAdjThreads, 1) k_sep_adjoint(const SepAdjPara
           : "=r"(stop)
           : "r"(x.tile), "r"(2 + group)
           : "memory");
-      if (gw == 0 && lane == 0 && ok) mbar_arrive(&ready[sl]);
+      if (gw == 0 && lane == 0 && ok) {
+        mbar_arrive(&ready[sl]);
+        if (x.tile == -1) mbar_arrive(&ready[(it + 2) & 7]);   // the third issuer's end
+      }
       if (stop) break;
     }
   }
@@ -418,7 +455,7 @@ __global__ void __launch_bounds__(kAdjThreads, 1) k_sep_adjoint(const SepAdjPara
 }
 
 // One warp per chunk of 32 spots.
-__global__ void k_sep_scale(const float2* __restrict__ y, int N, int chunks, float2* __restrict__ ys,
+__global__ void k_sep_scale(const float2* __restrict__ y, int N, int chunks, float* __restrict__ ys,
                             float* __restrict__ scale) {
   const int c = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
   if (c < chunks) sep_scale_chunk(y, N, c, ys, scale);
@@ -426,7 +463,7 @@ __global__ void k_sep_scale(const float2* __restrict__ y, int N, int chunks, flo
 
 }  // namespace
 
-cudaError_t sep_launch_scale(const float2* y, int N, float2* ys, float* scale, cudaStream_t s) {
+cudaError_t sep_launch_scale(const float2* y, int N, float* ys, float* scale, cudaStream_t s) {
   const int chunks = sep_blocks(N) * (kSepSpots / kSepChunk);
   k_sep_scale<<<(chunks + 3) / 4, 128, 0, s>>>(y, N, chunks, ys, scale);
   return cudaGetLastError();

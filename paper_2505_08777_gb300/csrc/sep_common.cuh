@@ -43,19 +43,46 @@ __device__ __forceinline__ float2 add2(float2 a, float2 b) {
       : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
   return d;
 }
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) {
+  float2 d;
+  asm("{\n\t.reg .b64 ra, rb, rd;\n\t"
+      "mov.b64 ra, {%2, %3};\n\t"
+      "mov.b64 rb, {%4, %5};\n\t"
+      "sub.rn.f32x2 rd, ra, rb;\n\t"
+      "mov.b64 {%0, %1}, rd;\n\t}"
+      : "=f"(d.x), "=f"(d.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return d;
+}
 __device__ __forceinline__ float2 dup2(float a) { return make_float2(a, a); }
 __device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
 
 // hi of the split: x rounded to the grid 2^-11 (adding 1.5 * 2^12 leaves no
 // finer bits), for |x| <= 1.
 __device__ __forceinline__ float2 split_hi2(float2 x) {
-  return add2(add2(x, dup2(6144.0f)), dup2(-6144.0f));
+  return sub2(add2(x, dup2(6144.0f)), dup2(6144.0f));
 }
 // (a, b) as a pair of f16, a in the low half.
 __device__ __forceinline__ uint32_t pack_f16(float a, float b) {
   uint32_t d;
   asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(b), "f"(a));
   return d;
+}
+
+// mbar_wait with a suspend time (ns) for each poll, so that waiting warps leave
+// the issue slots to the others; at most about a second in all.
+constexpr uint32_t kSepWaitPolls = 1u << 20, kSepWaitNs = 1000;
+__device__ __forceinline__ bool sep_wait(uint64_t* bar, uint32_t parity) {
+  uint32_t done = 0;
+  for (uint32_t it = 0; it < kSepWaitPolls; ++it) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(done)
+        : "r"(smem_u32(bar)), "r"(parity), "r"(kSepWaitNs)
+        : "memory");
+    if (done) return true;
+  }
+  return false;
 }
 
 // Instruction descriptor of kind::f16 with f16 operands and an fp32
@@ -98,17 +125,30 @@ __device__ __forceinline__ uint32_t pack_bf16_rz(float lo, float hi) {
   return (__float_as_uint(lo) >> 16) | (__float_as_uint(hi) & 0xffff0000u);
 }
 
-__device__ __forceinline__ SepPoly sep_unpack(float4 a, float4 b, float4 c, float4 d) {
+// Words of a spot's polynomial: word k of the 32 spots of a chunk are 32
+// consecutive floats.
+enum SepWord : int { kWBase, kWAx, kWAy, kWLow, kWX2, kWX3, kWX4, kWY2, kWY3, kWY4, kWC11, kWC21, kWC12, kWC22, kWN31,
+                     kWC13 };
+__device__ __forceinline__ SepPoly sep_unpack(const float* w) {
   SepPoly p;
-  p.base = a.x;
-  p.ax = a.y;
-  p.ay = a.z;
-  const uint32_t lo = __float_as_uint(a.w);
+  p.base = w[32 * kWBase];
+  p.ax = w[32 * kWAx];
+  p.ay = w[32 * kWAy];
+  const uint32_t lo = __float_as_uint(w[32 * kWLow]);
   p.axl = __uint_as_float(lo << 16);
   p.ayl = __uint_as_float(lo & 0xffff0000u);
-  p.x2 = b.x; p.x3 = b.y; p.x4 = b.z; p.y2 = b.w;
-  p.y3 = c.x; p.y4 = c.y; p.c11 = c.z; p.c21 = c.w;
-  p.c12 = d.x; p.c22 = d.y; p.n31 = d.z; p.c13 = d.w;
+  p.x2 = w[32 * kWX2];
+  p.x3 = w[32 * kWX3];
+  p.x4 = w[32 * kWX4];
+  p.y2 = w[32 * kWY2];
+  p.y3 = w[32 * kWY3];
+  p.y4 = w[32 * kWY4];
+  p.c11 = w[32 * kWC11];
+  p.c21 = w[32 * kWC21];
+  p.c12 = w[32 * kWC12];
+  p.c22 = w[32 * kWC22];
+  p.n31 = w[32 * kWN31];
+  p.c13 = w[32 * kWC13];
   return p;
 }
 
@@ -123,20 +163,19 @@ __device__ __forceinline__ void cis2(float2 x, float2& c, float2& s) {
 }
 
 // The angles 2 pi (a m + b) + m (al + q2 m + q3 m^2 + q4 m^3), less whole turns
-// of a m + b, for two offsets m; a m less an integer is exact. `na`, `nb` are
-// -a, -b (the packed operations take no sign). b is in turns, |b| <= 1.
-__device__ __forceinline__ float2 sep_angle(float a, float na, float al, float q2, float q3, float q4, float b,
-                                            float nb, float2 m) {
-  const float2 k = add2(add2(fma2(dup2(na), m, dup2(nb)), dup2(12582912.0f)), dup2(-12582912.0f));   // -rint(a m + b)
-  const float2 r = add2(fma2(dup2(a), m, k), dup2(b));
-  const float2 q = fma2(fma2(fma2(dup2(q4), m, dup2(q3)), m, dup2(q2)), m, dup2(al));
+// of a m + b, for two values each; a m less an integer is exact. b is in
+// turns, |b| <= 1.
+__device__ __forceinline__ float2 sep_angle(float2 a, float2 al, float2 q2, float2 q3, float2 q4, float2 b, float2 m) {
+  const float2 k = sub2(dup2(12582912.0f), add2(fma2(a, m, b), dup2(12582912.0f)));   // -rint(a m + b)
+  const float2 r = add2(fma2(a, m, k), b);
+  const float2 q = fma2(fma2(fma2(q4, m, q3), m, q2), m, al);
   return fma2(r, dup2(6.283185307179586f), mul2(q, m));
 }
 // The same with b = 0.
-__device__ __forceinline__ float2 sep_angle(float a, float na, float al, float q2, float q3, float q4, float2 m) {
-  const float2 k = add2(fma2(dup2(na), m, dup2(12582912.0f)), dup2(-12582912.0f));
-  const float2 r = fma2(dup2(a), m, k);
-  const float2 q = fma2(fma2(fma2(dup2(q4), m, dup2(q3)), m, dup2(q2)), m, dup2(al));
+__device__ __forceinline__ float2 sep_angle(float2 a, float2 al, float2 q2, float2 q3, float2 q4, float2 m) {
+  const float2 k = sub2(dup2(12582912.0f), fma2(a, m, dup2(12582912.0f)));
+  const float2 r = fma2(a, m, k);
+  const float2 q = fma2(fma2(fma2(q4, m, q3), m, q2), m, al);
   return fma2(r, dup2(6.283185307179586f), mul2(q, m));
 }
 
@@ -152,7 +191,7 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
 
 // Two values split into f16 pairs (hi, lo).
 __device__ __forceinline__ void split_pack(float2 v, uint32_t& hi, uint32_t& lo) {
-  const float2 h = split_hi2(v), l = fma2(h, dup2(-1.0f), v);
+  const float2 h = split_hi2(v), l = sub2(v, h);
   hi = pack_f16(h.x, h.y);
   lo = pack_f16(l.x, l.y);
 }
@@ -178,15 +217,16 @@ __device__ __forceinline__ SepColumns sep_columns(const SepPoly& q, int s, int l
 }
 
 // y of the 32 spots of a chunk divided by a power of two (scale), so that
-// |y| <= 1; by one warp.
-__device__ __forceinline__ void sep_scale_chunk(const float2* __restrict__ y, int N, int c, float2* __restrict__ ys,
+// |y| <= 1: the 32 real, then the 32 imaginary parts; by one warp.
+__device__ __forceinline__ void sep_scale_chunk(const float2* __restrict__ y, int N, int c, float* __restrict__ ys,
                                                 float* __restrict__ scale) {
   const int lane = threadIdx.x & 31, n = c * 32 + lane;
   const float2 v = n < N ? __ldg(y + n) : make_float2(0.0f, 0.0f);
   const uint32_t mx = __reduce_max_sync(0xffffffffu, __float_as_uint(hypotf(v.x, v.y)));
   const int e = min(max((int)(mx >> 23), 27), 227) - 126;
   const float inv = __uint_as_float((uint32_t)(127 - e) << 23);
-  ys[c * 32 + lane] = make_float2(v.x * inv, v.y * inv);
+  ys[c * 64 + lane] = v.x * inv;
+  ys[c * 64 + 32 + lane] = v.y * inv;
   if (lane == 0) scale[c] = __uint_as_float((uint32_t)(127 + e) << 23);
 }
 

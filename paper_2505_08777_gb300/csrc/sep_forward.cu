@@ -76,7 +76,7 @@ __device__ __forceinline__ void acc_hl(float& hi, float& lo, float c, float bh, 
 // CTA (tile, block): thread = spot. Bound: the table is read once per CTA
 // from shared memory and 64 B per (tile, spot) are written.
 __global__ void __launch_bounds__(kSepSpots) k_sep_params(const Geometry G, const float* __restrict__ tab,
-                                                          const float* __restrict__ coeff, float4* __restrict__ poly,
+                                                          const float* __restrict__ coeff, float* __restrict__ poly,
                                                           unsigned char* __restrict__ strips, int npad) {
   __shared__ float st[kMaxModes * kSepTab];
   __shared__ int sred[4];
@@ -109,12 +109,23 @@ __global__ void __launch_bounds__(kSepSpots) k_sep_params(const Geometry G, cons
   }
   // per pixel offset (u = mx / 16, v = my / 16); the powers in radians
   constexpr float tp = 6.283185307179586f, h = 0.0625f;
-  const size_t o = ((size_t)tile * (npad / 32) + (n >> 5)) * 128 + (n & 31);
-  poly[o] = make_float4(base, axh, ayh, __uint_as_float(pack_bf16_rz(tp * axl, tp * ayl)));
-  poly[o + 32] = make_float4(tp * q[0] * (h * h), tp * q[1] * (h * h * h), tp * q[2] * (h * h * h * h),
-                               tp * q[3] * (h * h));
-  poly[o + 64] = make_float4(tp * q[4] * (h * h * h), tp * q[5] * (h * h * h * h), q[6] * h, q[7] * h);
-  poly[o + 96] = make_float4(q[8] * (h * h), q[9] * (h * h), -q[10] * h, q[11] * (h * h * h));
+  float* o = poly + ((size_t)tile * (npad / 32) + (n >> 5)) * 512 + (n & 31);
+  o[32 * kWBase] = base;
+  o[32 * kWAx] = axh;
+  o[32 * kWAy] = ayh;
+  o[32 * kWLow] = __uint_as_float(pack_bf16_rz(tp * axl, tp * ayl));
+  o[32 * kWX2] = tp * q[0] * (h * h);
+  o[32 * kWX3] = tp * q[1] * (h * h * h);
+  o[32 * kWX4] = tp * q[2] * (h * h * h * h);
+  o[32 * kWY2] = tp * q[3] * (h * h);
+  o[32 * kWY3] = tp * q[4] * (h * h * h);
+  o[32 * kWY4] = tp * q[5] * (h * h * h * h);
+  o[32 * kWC11] = q[6] * h;
+  o[32 * kWC21] = q[7] * h;
+  o[32 * kWC12] = q[8] * (h * h);
+  o[32 * kWC22] = q[9] * (h * h);
+  o[32 * kWN31] = -q[10] * h;
+  o[32 * kWC13] = q[11] * (h * h * h);
   // Row strips: the cubic in u takes u^4 R1^4 / 24 etc. as u^2 (off by at most
   // 1/4) and drops the rest; with 2^k strips R_k about a strip's middle row is
   // at most |dR_k/dv| / 2^k. The fewest strips that drop less than kSepTol.
@@ -193,8 +204,8 @@ __global__ void k_sep_scan(const unsigned char* __restrict__ strips, int U, int 
 // One CTA per SM, 20 warps in three roles. The generators (warps 8-15)
 // prepare the steps' operands, the summers (warps 0-7) read the results, one
 // thread (warp 17) lists the steps and fetches their phase polynomials, and
-// one (warp 16) issues the MMAs (issuing blocks while the tensor core is
-// busy, so no generator does it). A step: A = X(u) of 128 spots, rows [Re X(0..31) | Im X(0..31)];
+// two (warps 16, 18) issue the MMAs of every second step each (issuing and its
+// waits take longer than the MMAs themselves). A step: A = X(u) of 128 spots, rows [Re X(0..31) | Im X(0..31)];
 // B = the tile's nearfield times u^k, k = 0..3, rows (k / 2, row pair, k % 2,
 // re / im, row of the pair), [Re f | -Im f] and [Im f | Re f]. D[spot][256]
 // then holds the four complex sums of every tile row, to which the summers
@@ -238,17 +249,17 @@ __device__ __forceinline__ void sep_sum_pair(const SepPoly& q, float R1s, float 
   const float2 R2 = fma2(fma2(dup2(q.c22), m, dup2(q.c21)), m, dup2(-R2s));
   const float2 n3 = fma2(dup2(q.n31), m, dup2(-n3s));   // -R3
   // exp(-i r) = 1 - i R1 u + q2 u^2 + q3 u^3, with the u^4 term taken as u^2
-  const float2 n1 = mul2(R1, dup2(-1.0f)), s = mul2(R1, R1);
+  const float2 n1 = sub2(make_float2(0.0f, 0.0f), R1), s = mul2(R1, R1);
   const float2 q2r = fma2(s, fma2(s, dup2(1.0f / 24.0f), dup2(-0.5f)), mul2(R2, mul2(R2, dup2(-0.5f))));
   const float2 q2i = mul2(R2, fma2(s, dup2(0.5f), dup2(-1.0f)));
   const float2 q3r = mul2(n1, R2), q3i = fma2(mul2(R1, s), dup2(1.0f / 6.0f), n3);
   const float2 ur = fma2(q3i, D(z, 3), mul2(q2i, D(z, 1)));
   float2 Tr = fma2(q3r, D(z, 2), fma2(q2r, D(z, 0), fma2(R1, D(x, 3), D(x, 0))));
-  Tr = fma2(ur, dup2(-1.0f), Tr);
+  Tr = sub2(Tr, ur);
   float2 Ti = fma2(q2r, D(z, 1), fma2(n1, D(x, 2), D(x, 1)));
   Ti = fma2(q3r, D(z, 3), fma2(q3i, D(z, 2), fma2(q2i, D(z, 0), Ti)));
   float2 c, sn;
-  cis2(sep_angle(q.ay, -q.ay, q.ayl, q.y2, q.y3, q.y4, q.base, -q.base, m), c, sn);
+  cis2(sep_angle(dup2(q.ay), dup2(q.ayl), dup2(q.y2), dup2(q.y3), dup2(q.y4), dup2(q.base), m), c, sn);
   if (one >= 0) {
     const float2 w = one ? make_float2(0.0f, 1.0f) : make_float2(1.0f, 0.0f);
     c = mul2(c, w);
@@ -282,14 +293,14 @@ __device__ __forceinline__ void sep_moment_pair(const SepPoly& q, float R1s, flo
   const float2 R1 = fma2(fma2(fma2(dup2(q.c13), m, dup2(q.c12)), m, dup2(q.c11)), m, dup2(-R1s));
   const float2 R2 = fma2(fma2(dup2(q.c22), m, dup2(q.c21)), m, dup2(-R2s));
   const float2 n3 = fma2(dup2(q.n31), m, dup2(-n3s));   // -R3
-  const float2 n1 = mul2(R1, dup2(-1.0f)), s = mul2(R1, R1);
+  const float2 n1 = sub2(make_float2(0.0f, 0.0f), R1), s = mul2(R1, R1);
   const float2 q2r = fma2(s, fma2(s, dup2(1.0f / 24.0f), dup2(-0.5f)), mul2(R2, mul2(R2, dup2(-0.5f))));
-  const float2 q2i = mul2(R2, fma2(s, dup2(0.5f), dup2(-1.0f))), p2i = mul2(q2i, dup2(-1.0f));
-  const float2 q3r = mul2(n1, R2), q3i = fma2(mul2(R1, s), dup2(1.0f / 6.0f), n3), p3i = mul2(q3i, dup2(-1.0f));
+  const float2 q2i = mul2(R2, fma2(s, dup2(0.5f), dup2(-1.0f))), p2i = sub2(make_float2(0.0f, 0.0f), q2i);
+  const float2 q3r = mul2(n1, R2), q3i = fma2(mul2(R1, s), dup2(1.0f / 6.0f), n3), p3i = sub2(make_float2(0.0f, 0.0f), q3i);
   const float2 d4r = fma2(D(x, 0), dup2(-0.125f), D(z, 0)), d4i = fma2(D(x, 1), dup2(-0.125f), D(z, 1));
   // conj(gE) Y
   float2 c, sn;
-  cis2(sep_angle(q.ay, -q.ay, q.ayl, q.y2, q.y3, q.y4, q.base, -q.base, m), c, sn);
+  cis2(sep_angle(dup2(q.ay), dup2(q.ayl), dup2(q.y2), dup2(q.y3), dup2(q.y4), dup2(q.base), m), c, sn);
   if (one >= 0) {
     const float2 w = one ? make_float2(0.0f, 1.0f) : make_float2(1.0f, 0.0f);
     c = mul2(c, w);
@@ -396,7 +407,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) k_sep_forward(const SepFwdPara
   float* scales = reinterpret_cast<float*>(smax + 8);            // [4] 2^e of the steps' tiles
   SepStep* steps = reinterpret_cast<SepStep*>(scales + 4);       // [4]
   const int t = threadIdx.x, w = t >> 5, lane = t & 31;
-  const int row = t & 127, prow = (row >> 5) * 128 + (row & 31);   // the spot's place in a slot
+  const int row = t & 127, prow = (row >> 5) * 512 + (row & 31);   // the spot's place in a slot
   const int nb = p.nb, npad = nb * kSepSpots, U = p.g.T * nb;
   if (w == 0) tmem_alloc(slot, 512);
   if (t == 0) {
@@ -455,7 +466,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) k_sep_forward(const SepFwdPara
       }
     };
     for (uint32_t it = 0;; ++it) {
-      ok = ok && mbar_wait(&ready[it & 3], (it >> 2) & 1, kTcWaitPolls);
+      ok = ok && sep_wait(&ready[it & 3], (it >> 2) & 1);
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
       const SepStep r = steps[it & 3];
@@ -473,11 +484,10 @@ __global__ void __launch_bounds__(kFwdThreads, 1) k_sep_forward(const SepFwdPara
         psc = scale;
       }
       if (r.b < 0) break;
-      const float4* sq = reinterpret_cast<const float4*>(sm + kFwdSlots + (it & 3) * kFSlot) + prow;
-      const SepPoly q = sep_unpack(sq[0], sq[32], sq[64], sq[96]);
+      const SepPoly q = sep_unpack(reinterpret_cast<const float*>(sm + kFwdSlots + (it & 3) * kFSlot) + prow);
       const int rows = 32 >> r.ls, pairs = rows >= 2 ? rows >> 1 : 1;
       const int np = pairs >= 2 ? pairs >> 1 : (half ? 0 : 1), p0 = ((r.s * rows) >> 1) + half * np;
-      ok = ok && mbar_wait(&full[it & 1], (it >> 1) & 1, kTcWaitPolls);
+      ok = ok && sep_wait(&full[it & 1], (it >> 1) & 1);
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
       tc_fence_after();
@@ -493,16 +503,18 @@ __global__ void __launch_bounds__(kFwdThreads, 1) k_sep_forward(const SepFwdPara
     }
   } else if (w >= 16) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
-    if (w == 16 && lane == 0) {
-      // --- MMA issue ---
-      uint32_t it = 0;
-      for (;; ++it) {
-        const int d = it & 1;
-        ok = ok && mbar_wait(&ready[it & 3], (it >> 2) & 1, kTcWaitPolls);
-        if (it >= 2) ok = ok && mbar_wait(&empty[(it - 2) & 3], ((it - 2) >> 2) & 1, kTcWaitPolls);
+    if ((w == 16 || w == 18) && lane == 0) {
+      // --- MMA issue: even or odd steps, into D buffer d ---
+      const int d = (w - 16) >> 1;
+      uint32_t it = (uint32_t)d;
+      for (;; it += 2) {
+        ok = ok && sep_wait(&listed[it & 3], (it >> 2) & 1);
         if (!ok) break;
         const SepStep r = steps[it & 3];
         if (r.b < 0) break;
+        ok = ok && sep_wait(&ready[it & 3], (it >> 2) & 1);
+        if (it >= 2) ok = ok && sep_wait(&empty[(it - 2) & 3], ((it - 2) >> 2) & 1);
+        if (!ok) break;
         tc_fence_after();
         // the columns of the step's rows in each half of D (N >= 16)
         const int rows = 32 >> r.ls, p0 = (r.s * rows) >> 1;
@@ -533,7 +545,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) k_sep_forward(const SepFwdPara
         umma_commit(&full[d]);
       }
       // nothing in flight when the CTA gives up its memory
-      for (uint32_t k = it > 2 ? it - 2 : 0; k < it; ++k) ok = mbar_wait(&full[k & 1], (k >> 1) & 1, kTcWaitPolls) && ok;
+      if (it >= 2) ok = sep_wait(&full[d], ((it - 2) >> 1) & 1) && ok;
     } else if (w == 17 && lane == 0) {
       // --- steps of this CTA: those whose place in the cost prefix lies in [c0, c1) ---
       const long long W = p.cost[U];
@@ -564,20 +576,25 @@ __global__ void __launch_bounds__(kFwdThreads, 1) k_sep_forward(const SepFwdPara
           if (u + 1 < U) ls1 = p.strips[u + 1];
         }
         const bool more = pos < c1;
-        // slot it & 3 was step it - 4's
-        if (it >= 4) ok = ok && mbar_wait(&empty[it & 3], ((it >> 2) - 1) & 1, kTcWaitPolls);
-        steps[it & 3] = more ? x : SepStep{0, -1, 0, 0, 0};
         if (!more) {
-          mbar_arrive(&listed[it & 3]);
+          // an end for each of the two issuers
+          for (uint32_t k = it; k < it + 2; ++k) {
+            if (k >= 4) ok = ok && sep_wait(&empty[k & 3], ((k >> 2) - 1) & 1);
+            steps[k & 3] = SepStep{0, -1, 0, 0, 0};
+            mbar_arrive(&listed[k & 3]);
+          }
           break;
         }
+        // slot it & 3 was step it - 4's
+        if (it >= 4) ok = ok && sep_wait(&empty[it & 3], ((it >> 2) - 1) & 1);
+        steps[it & 3] = x;
         mbar_expect_tx(&listed[it & 3], kFSlot);
-        bulk_g2s(sm + kFwdSlots + (it & 3) * kFSlot, p.poly + ((size_t)x.tile * nb + x.b) * (4 * kSepSpots), kFSlot,
+        bulk_g2s(sm + kFwdSlots + (it & 3) * kFSlot, p.poly + ((size_t)x.tile * nb + x.b) * (16 * kSepSpots), kFSlot,
                  &listed[it & 3]);
         pos += c;
         ++x.s;
       }
-      for (uint32_t k = it > 3 ? it - 3 : 0; k < it; ++k) ok = mbar_wait(&listed[k & 3], (k >> 2) & 1, kTcWaitPolls) && ok;
+      for (uint32_t k = it > 2 ? it - 2 : 0; k < it; ++k) ok = sep_wait(&listed[k & 3], (k >> 2) & 1) && ok;
     }
     __syncwarp();
   } else {
@@ -636,8 +653,8 @@ __global__ void __launch_bounds__(kFwdThreads, 1) k_sep_forward(const SepFwdPara
     };
 
     // A: X(u) of this thread's spot for its 16 columns, about the strip's row
-    auto build_a = [&](const float4* sq, const SepStep& x, uint8_t* ah) {
-      const SepPoly q = sep_unpack(sq[0], sq[32], sq[64], sq[96]);
+    auto build_a = [&](const float* sq, const SepStep& x, uint8_t* ah) {
+      const SepPoly q = sep_unpack(sq);
       const SepColumns o = sep_columns(q, x.s, x.ls);
       // X = exp(-i angle): the negated angle's cosine and sine
 #pragma unroll
@@ -647,8 +664,8 @@ __global__ void __launch_bounds__(kFwdThreads, 1) k_sep_forward(const SepFwdPara
         for (int q2 = 0; q2 < 4; ++q2) {
           const float m0 = (float)(16 * half - 16 + 8 * c8 + 2 * q2);
           float2 cs, sn;
-          cis2(sep_angle(-o.ax, o.ax, -o.axl, -o.x2, -o.x3, -o.x4, make_float2(m0, m0 + 1.0f)), cs,
-               sn);
+          cis2(sep_angle(dup2(-o.ax), dup2(-o.axl), dup2(-o.x2), dup2(-o.x3), dup2(-o.x4), make_float2(m0, m0 + 1.0f)),
+               cs, sn);
           split_pack(cs, rh[q2], rl[q2]);
           split_pack(sn, ih[q2], il[q2]);
         }
@@ -664,9 +681,9 @@ __global__ void __launch_bounds__(kFwdThreads, 1) k_sep_forward(const SepFwdPara
     int tile = -1;
     for (uint32_t it = 0;; ++it) {
       const int d = it & 1;
-      ok = ok && mbar_wait(&listed[it & 3], (it >> 2) & 1, kTcWaitPolls);
+      ok = ok && sep_wait(&listed[it & 3], (it >> 2) & 1);
       // MMA(it - 2) done: its A, and B of an older tile, are free
-      if (it >= 2) ok = ok && mbar_wait(&full[d], ((it >> 1) - 1) & 1, kTcWaitPolls);
+      if (it >= 2) ok = ok && sep_wait(&full[d], ((it >> 1) - 1) & 1);
       // every generator goes on or none (they meet at a barrier)
       int stop;
       asm volatile(
@@ -685,7 +702,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) k_sep_forward(const SepFwdPara
         tile = x.tile;
         scale = build_b(tile, sm + kFwdB + (uint32_t)x.bb * kFwdBuf);
       }
-      build_a(reinterpret_cast<const float4*>(sm + kFwdSlots + (it & 3) * kFSlot) + prow, x,
+      build_a(reinterpret_cast<const float*>(sm + kFwdSlots + (it & 3) * kFSlot) + prow, x,
               sm + (uint32_t)d * 2 * kFA);
       fence_async_smem();
       if (g == 0) scales[it & 3] = scale;
@@ -750,7 +767,7 @@ cudaError_t sep_build_table(const Geometry& g, const MonoTerm* terms, const int*
   return cudaGetLastError();
 }
 
-cudaError_t sep_build_params(const Geometry& g, const float* tab, const float* coeff, float4* poly,
+cudaError_t sep_build_params(const Geometry& g, const float* tab, const float* coeff, float* poly,
                              unsigned char* strips, int* cost, int* acost, cudaStream_t s) {
   const int nb = sep_blocks(g.N);
   k_sep_params<<<dim3(g.T, nb), kSepSpots, 0, s>>>(g, tab, coeff, poly, strips, nb * kSepSpots);

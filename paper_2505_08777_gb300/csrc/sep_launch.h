@@ -33,19 +33,19 @@ inline int sep_blocks(int N) { return (N + kSepSpots - 1) / kSepSpots; }
 // c20 c30 c40 c02 c03 c04 c11 c21 c12 c22 c31 c13 per u^k v^l.
 cudaError_t sep_build_table(const Geometry& g, const MonoTerm* terms, const int* term_off, float* tab, cudaStream_t s);
 
-// Phase polynomials of every (tile, spot), [T][chunk of 32 spots][4][32]
-// float4 (SepPoly), and
+// Phase polynomials of every (tile, spot), [T][chunk of 32 spots][16 words][32]
+// (SepPoly), and
 // per (tile, spot block) the log2 of the row strips its mixed terms need and
 // the prefixes of their forward steps' cost
 // [T nb + 1] and of their adjoint chunks' cost [T nb + 1], then the largest
 // chunk cost.
-cudaError_t sep_build_params(const Geometry& g, const float* tab, const float* coeff, float4* poly,
+cudaError_t sep_build_params(const Geometry& g, const float* tab, const float* coeff, float* poly,
                              unsigned char* strips, int* cost, int* acost, cudaStream_t s);
 
 struct SepFwdParams {
   Geometry g;
   int nb;                        // spot blocks
-  const float4* poly;
+  const float* poly;
   const unsigned char* strips;
   const int* cost;
   const float4* fimg;            // nearfield image (tc_launch.h)
@@ -64,10 +64,10 @@ cudaError_t sep_launch_gradc_reduce(const SepFwdParams& p, cudaStream_t s);     
 struct SepAdjParams {
   TcAdjParams a;                 // geometry, amplitude, y, outputs
   int nb;
-  const float4* poly;
+  const float* poly;
   const unsigned char* strips;
   const int* cost;               // adjoint prefix
-  const float2* ys;              // [128 nb] y / scale
+  const float* ys;               // [4 nb][re, im][32] y / scale
   const float* scale;            // [4 nb] power of two per chunk of 32 spots
   float2* split;                 // [G][2][kTilePix] partial sums of tiles split between CTAs
   int* tickets;                  // [T] CTAs done with a split tile (left at 0)
@@ -76,7 +76,7 @@ struct SepAdjParams {
 cudaError_t sep_prepare();
 cudaError_t sep_adjoint_prepare();
 // y divided by a power of two (scale) per chunk of 32 spots.
-cudaError_t sep_launch_scale(const float2* y, int N, float2* ys, float* scale, cudaStream_t s);
+cudaError_t sep_launch_scale(const float2* y, int N, float* ys, float* scale, cudaStream_t s);
 cudaError_t sep_launch_adjoint(const SepAdjParams& p, cudaStream_t s);
 cudaError_t sep_launch_forward(const SepFwdParams& p, cudaStream_t s);          // partial sums
 cudaError_t sep_launch_forward_reduce(const SepFwdParams& p, cudaStream_t s);   // E from them
