@@ -436,8 +436,8 @@ ash_status enqueue_forward(ash_hologram* h, int source, const float* phase, cons
   cudaError_t e = launch_forward(h->g.D, p, h->sched.G, s);
   if (e != cudaSuccess) return cuda_fail(e, "forward kernel launch");
   const int cols = 2 * h->g.N;
-  k_col_reduce<<<(cols + 31) / 32, dim3(32, 32), 0, s>>>(h->partial, h->fwd_rows, cols, reinterpret_cast<float*>(E));
-  e = cudaGetLastError();
+  e = launch_pdl(k_col_reduce, (cols + 31) / 32, dim3(32, 32), 0, s, h->partial, h->fwd_rows, cols,
+                 reinterpret_cast<float*>(E));
   if (e != cudaSuccess) return cuda_fail(e, "forward reduce launch");
   return ASH_OK;
 }
@@ -473,8 +473,7 @@ ash_status enqueue_adjoint(ash_hologram* h, const float2* y, float2* g_out, floa
   cudaError_t e = launch_adjoint(h->g.D, p, h->sched.G, s);
   if (e != cudaSuccess) return cuda_fail(e, "adjoint kernel launch");
   if (h->split_tiles) {
-    k_adjoint_fixup<<<h->g.T, h->g.NT, 0, s>>>(p);
-    e = cudaGetLastError();
+    e = launch_pdl(k_adjoint_fixup, h->g.T, h->g.NT, 0, s, p);
     if (e != cudaSuccess) return cuda_fail(e, "adjoint fix-up launch");
   }
   return ASH_OK;
@@ -492,17 +491,16 @@ ash_status enqueue_wgs_body(ash_hologram* h, int iters, cudaStream_t s) {
   ash_status st = enqueue_forward(h, kSrcPhase, h->wgs_phase, nullptr, h->wgs_E, s);
   if (st != ASH_OK) return st;
   for (int it = 0; it < iters; ++it) {
-    k_wgs_update<<<1, 1024, 0, s>>>(h->wgs_E, h->wgs_w, h->wgs_T, h->y, h->g.N, h->wgs_feedback,
-                                    h->wgs_fix ? h->wgs_u : nullptr, h->wgs_fix ? nullptr : h->wgs_u);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = launch_pdl(k_wgs_update, 1, 1024, 0, s, h->wgs_E, h->wgs_w, h->wgs_T, h->y, h->g.N,
+                               h->wgs_feedback, h->wgs_fix ? h->wgs_u : nullptr, h->wgs_fix ? nullptr : h->wgs_u);
     if (e != cudaSuccess) return cuda_fail(e, "wgs update launch");
     st = enqueue_adjoint(h, h->y, nullptr, h->wgs_phase, nullptr, nullptr, adj_epi, s);
     if (st != ASH_OK) return st;
     st = enqueue_forward(h, tc ? kSrcImg : kSrcPhase, h->wgs_phase, nullptr, h->wgs_E, s);
     if (st != ASH_OK) return st;
   }
-  k_metrics<<<1, 1024, 0, s>>>(h->wgs_E, h->wgs_T, h->g.N, h->sum_a2, (double)h->g.nx * h->g.ny, h->wgs_metrics);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = launch_pdl(k_metrics, 1, 1024, 0, s, h->wgs_E, h->wgs_T, h->g.N, h->sum_a2,
+                             (double)h->g.nx * h->g.ny, h->wgs_metrics);
   if (e != cudaSuccess) return cuda_fail(e, "metrics launch");
   return ASH_OK;
 }

@@ -329,6 +329,7 @@ __device__ __forceinline__ void spot_loss_body(const float2* __restrict__ E, con
 // Single-hologram wrappers.
 
 static __global__ void k_col_reduce(const float* __restrict__ in, int rows, int cols, float* __restrict__ out) {
+  pdl_begin();
   col_reduce_body(in, rows, cols, out, blockIdx.x);
 }
 
@@ -341,6 +342,7 @@ static __global__ void __launch_bounds__(1024) k_wgs_update(const float2* __rest
                                                             const float* __restrict__ T, float2* __restrict__ y,
                                                             int N, float feedback, const float2* __restrict__ u_fixed,
                                                             float2* __restrict__ u_store) {
+  pdl_begin();
   wgs_update_body(E, w, T, y, N, feedback, u_fixed, u_store);
 }
 
@@ -352,11 +354,13 @@ static __global__ void __launch_bounds__(1024) k_spot_loss(const float2* __restr
 static __global__ void __launch_bounds__(1024) k_metrics(const float2* __restrict__ E, const float* __restrict__ T,
                                                          int N, const double* __restrict__ sum_a2, double M,
                                                          float* __restrict__ metrics) {
+  pdl_begin();
   metrics_body(E, T, N, sum_a2, M, metrics);
 }
 
 // One CTA of G.NT threads per tile; tiles owned by a single CTA return at once.
 static __global__ void k_adjoint_fixup(const AdjParams p) {
+  pdl_begin();
   const long long u_lo = (long long)blockIdx.x * p.v.g.N, u_hi = u_lo + p.v.g.N - 1;
   const int b_lo = p.sched.owner(u_lo), b_hi = p.sched.owner(u_hi);
   if (b_lo == b_hi) return;

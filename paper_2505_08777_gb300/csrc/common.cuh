@@ -67,6 +67,14 @@ __host__ __device__ constexpr int pixels_per_thread(int D) { return D <= 12 ? AS
 #endif
 #define ASH_BOUNDS(P) __launch_bounds__(kTilePix / (P), ((P) == 8 ? ASH_MIN_BLOCKS : 1))
 
+// Start of a kernel launched with launch_pdl: waits until the kernels before it
+// are done and their writes visible, then lets the next one's blocks be
+// scheduled (they wait here in turn). Nothing global is touched before it.
+__device__ __forceinline__ void pdl_begin() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // ---------------------------------------------------------------------------
 // Packed fp32x2 arithmetic (Blackwell FFMA2): one instruction, two lanes of
 // work; used for pixel pairs so the phase contraction and complex MAC take

@@ -30,12 +30,10 @@ struct Inst {
     return e;
   }
   static cudaError_t forward(const FwdParams& p, int grid, cudaStream_t s) {
-    k_forward<D, P><<<grid, NT, fwd_smem_bytes(D), s>>>(p);
-    return cudaGetLastError();
+    return launch_pdl(k_forward<D, P>, grid, NT, fwd_smem_bytes(D), s, p);
   }
   static cudaError_t adjoint(const AdjParams& p, int grid, cudaStream_t s) {
-    k_adjoint<D, P><<<grid, NT, adj_smem_bytes(D), s>>>(p);
-    return cudaGetLastError();
+    return launch_pdl(k_adjoint<D, P>, grid, NT, adj_smem_bytes(D), s, p);
   }
   static cudaError_t gradc(const GradCParams& p, dim3 grid, cudaStream_t s) {
     k_gradc<D><<<grid, kGradThreads, gradc_smem_bytes(D), s>>>(p);

@@ -102,6 +102,7 @@ __global__ void __launch_bounds__(kAdjThreads, 1) k_sep_adjoint(const SepAdjPara
   tc_fence_after();
   const uint32_t tmem = *slot;
   bool ok = true;
+  pdl_begin();
   const long long W = p.cost[U];
   // ranges no shorter than a chunk, so that every CTA of a split tile has one
   const int G = (int)max(1LL, min((long long)p.G, W / p.cost[U + 1]));
@@ -457,6 +458,7 @@ __global__ void __launch_bounds__(kAdjThreads, 1) k_sep_adjoint(const SepAdjPara
 // One warp per chunk of 32 spots.
 __global__ void k_sep_scale(const float2* __restrict__ y, int N, int chunks, float* __restrict__ ys,
                             float* __restrict__ scale) {
+  pdl_begin();
   const int c = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
   if (c < chunks) sep_scale_chunk(y, N, c, ys, scale);
 }
@@ -465,8 +467,7 @@ __global__ void k_sep_scale(const float2* __restrict__ y, int N, int chunks, flo
 
 cudaError_t sep_launch_scale(const float2* y, int N, float* ys, float* scale, cudaStream_t s) {
   const int chunks = sep_blocks(N) * (kSepSpots / kSepChunk);
-  k_sep_scale<<<(chunks + 3) / 4, 128, 0, s>>>(y, N, chunks, ys, scale);
-  return cudaGetLastError();
+  return launch_pdl(k_sep_scale, (chunks + 3) / 4, 128, 0, s, y, N, chunks, ys, scale);
 }
 
 cudaError_t sep_adjoint_prepare() {
@@ -480,8 +481,7 @@ cudaError_t sep_adjoint_prepare() {
 }
 
 cudaError_t sep_launch_adjoint(const SepAdjParams& p, cudaStream_t s) {
-  k_sep_adjoint<<<p.G, kAdjThreads, kAdjSmem, s>>>(p);
-  return cudaGetLastError();
+  return launch_pdl(k_sep_adjoint, p.G, kAdjThreads, kAdjSmem, s, p);
 }
 
 }  // namespace ash

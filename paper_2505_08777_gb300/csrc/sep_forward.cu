@@ -419,6 +419,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) k_sep_forward(const SepFwdPara
   tc_fence_after();
   const uint32_t tmem = *slot;
   bool ok = true;
+  pdl_begin();
 
   if (w < 8) {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 120;");
@@ -720,10 +721,11 @@ __global__ void __launch_bounds__(kFwdThreads, 1) k_sep_forward(const SepFwdPara
 __global__ void k_sep_gradc_reduce(const float* __restrict__ part, int rows, int npad, int N, int D,
                                    float* __restrict__ dC) {
   __shared__ float acc[16][33];
+  pdl_begin();
   const int n = blockIdx.x * 32 + threadIdx.x, d = blockIdx.y, k = threadIdx.y;
   float v = 0.0f;
 #pragma unroll 10
-  for (int r = k; r < rows; r += 16) v += __ldg(part + ((size_t)r * D + d) * npad + n);
+  for (int r = k; r < rows; r += 16) v += part[((size_t)r * D + d) * npad + n];
   acc[k][threadIdx.x] = v;
   __syncthreads();
   for (int h = 8; h > 0; h >>= 1) {
@@ -738,11 +740,12 @@ __global__ void k_sep_gradc_reduce(const float* __restrict__ part, int rows, int
 __global__ void k_sep_forward_reduce(const float2* __restrict__ part, int rows, int npad, int N,
                                      float2* __restrict__ E) {
   __shared__ float2 acc[32][33];
+  pdl_begin();
   const int n = blockIdx.x * 32 + threadIdx.x, k = threadIdx.y;
   float2 v = make_float2(0.0f, 0.0f);
 #pragma unroll 10
   for (int r = k; r < rows; r += 32) {
-    const float2 x = __ldg(part + (size_t)r * npad + n);
+    const float2 x = part[(size_t)r * npad + n];
     v.x += x.x;
     v.y += x.y;
   }
@@ -791,25 +794,21 @@ cudaError_t sep_prepare() {
 }
 
 cudaError_t sep_launch_forward(const SepFwdParams& p, cudaStream_t s) {
-  k_sep_forward<false><<<p.G, kFwdThreads, kFwdSmem, s>>>(p);
-  return cudaGetLastError();
+  return launch_pdl(k_sep_forward<false>, p.G, kFwdThreads, kFwdSmem, s, p);
 }
 
 cudaError_t sep_launch_forward_reduce(const SepFwdParams& p, cudaStream_t s) {
-  k_sep_forward_reduce<<<(p.g.N + 31) / 32, dim3(32, 32), 0, s>>>(p.part, kSepFwdRows * p.G, p.nb * kSepSpots, p.g.N,
-                                                                  p.E);
-  return cudaGetLastError();
+  return launch_pdl(k_sep_forward_reduce, (p.g.N + 31) / 32, dim3(32, 32), 0, s, p.part, kSepFwdRows * p.G,
+                    p.nb * kSepSpots, p.g.N, p.E);
 }
 
 cudaError_t sep_launch_gradc(const SepFwdParams& p, cudaStream_t s) {
-  k_sep_forward<true><<<p.G, kFwdThreads, kFwdSmem, s>>>(p);
-  return cudaGetLastError();
+  return launch_pdl(k_sep_forward<true>, p.G, kFwdThreads, kFwdSmem, s, p);
 }
 
 cudaError_t sep_launch_gradc_reduce(const SepFwdParams& p, cudaStream_t s) {
-  k_sep_gradc_reduce<<<dim3((p.g.N + 31) / 32, p.g.D), dim3(32, 16), 0, s>>>(
-      p.dpart, kSepFwdRows * p.G, p.nb * kSepSpots, p.g.N, p.g.D, p.dC);
-  return cudaGetLastError();
+  return launch_pdl(k_sep_gradc_reduce, dim3((p.g.N + 31) / 32, p.g.D), dim3(32, 16), 0, s, p.dpart,
+                    kSepFwdRows * p.G, p.nb * kSepSpots, p.g.N, p.g.D, p.dC);
 }
 
 }  // namespace ash

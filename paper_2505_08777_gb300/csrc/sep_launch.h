@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 
 #include "common.cuh"
+#include "launch.h"
 #include "mono.h"
 #include "tc_launch.h"
 

@@ -1,5 +1,6 @@
 // Launchers of the tensor-core transform path (one instantiation per number
 // of K-atoms, NA = 1 for D <= 10 and NA = 2 for D <= 21).
+#include "launch.h"
 #include "tc_kernels.cuh"
 
 namespace ash {
@@ -186,8 +187,8 @@ cudaError_t tc_build_coeff(const Geometry& g, const TcLayout& L, const float* co
 cudaError_t tc_field_img(const Geometry& g, const float* amp_img, const float* phase, const float2* field,
                          float4* fimg, cudaStream_t s) {
   const long long px = (long long)g.T * kTilePix;
-  k_tc_field_img<<<blocks_for(px, 256), 256, 0, s>>>(g, amp_img, phase, field, reinterpret_cast<float*>(fimg));
-  return cudaGetLastError();
+  return launch_pdl(k_tc_field_img, blocks_for(px, 256), 256, 0, s, g, amp_img, phase, field,
+                    reinterpret_cast<float*>(fimg));
 }
 
 }  // namespace ash

@@ -155,6 +155,7 @@ __device__ __forceinline__ float turns_of_phase(float ph) {
 static __global__ void k_tc_field_img(const Geometry G, const float* __restrict__ amp_img,
                                       const float* __restrict__ phase, const float2* __restrict__ field,
                                       float* __restrict__ fimg) {
+  pdl_begin();
   const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= (long long)G.T * kTilePix) return;
   const long long qc = e / kTcChunk;

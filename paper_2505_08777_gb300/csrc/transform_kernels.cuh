@@ -319,6 +319,7 @@ __device__ __forceinline__ void adjoint_finish(const HoloView& hv, const AdjOut&
 // every entry is written exactly once per launch.
 template <int D, int P>
 __global__ void ASH_BOUNDS(P) k_forward(const FwdParams p) {
+  pdl_begin();
   constexpr int NW = kTilePix / P / 32;
   constexpr int CPS = cpair_stride(D);
   extern __shared__ float4 smem4[];
@@ -341,6 +342,7 @@ __global__ void ASH_BOUNDS(P) k_forward(const FwdParams p) {
 // for k_adjoint_fixup, which adds them in CTA order.
 template <int D, int P>
 __global__ void ASH_BOUNDS(P) k_adjoint(const AdjParams p) {
+  pdl_begin();
   constexpr int CPS = cpair_stride(D);
   extern __shared__ float4 smem4[];
   float* sC = reinterpret_cast<float*>(smem4);
