@@ -299,7 +299,7 @@ cudaError_t enqueue_tc_gradc(ash_hologram* h, const float* phase, const float2* 
 
 // Source of a forward: a phase or a complex field in user layout, or the
 // tc-layout nearfield the previous tensor-core adjoint wrote (kEpiFimg).
-constexpr int kSrcImg = 2;
+constexpr int kSrcImg = kSrcImage;
 
 cudaError_t enqueue_tc_coeff(ash_hologram* h, cudaStream_t s) {
   if (!h->tc_ok) return cudaSuccess;
@@ -602,6 +602,7 @@ ash_status adjoint_enqueue(ash_hologram* h, const float2* y, float2* g_out, floa
   return enqueue_adjoint(h, y, g_out, phase_out, phase_in, dphase, epilogue, s);
 }
 cudaError_t coeff_images_enqueue(ash_hologram* h, cudaStream_t s) { return enqueue_tc_coeff(h, s); }
+bool forward_reads_image(const ash_hologram* h) { return use_sep_fwd(h) || use_tc_fwd(h); }
 }  // namespace ash
 
 // A bounded wait that is never released: one thread waits on a fresh

@@ -154,6 +154,10 @@ ash_status forward_enqueue(ash_hologram* h, int source, const float* phase, cons
 ash_status adjoint_enqueue(ash_hologram* h, const float2* y, float2* g_out, float* phase_out, const float* phase_in,
                            float* dphase, int epilogue, cudaStream_t s);
 cudaError_t coeff_images_enqueue(ash_hologram* h, cudaStream_t s);
+// A forward from the nearfield image that the last forward from a phase or a
+// field (or a fused adjoint) left in the handle, where the forward reads one.
+constexpr int kSrcImage = 2;
+bool forward_reads_image(const ash_hologram* h);
 // CG workspace: fp64 scalar slots, reduction partials, iterations per call.
 constexpr int kCgSlots = 13, kCgRedBlocks = 512, kCgMaxIters = 1024;
 

@@ -108,7 +108,8 @@ ash_status ash_zsub_sweep(ash_hologram* h, const float* phase, int mode, const f
       st = cuda_fail(e, "calibration sweep");
       break;
     }
-    st = forward_enqueue(h, kSrcPhase, phase, nullptr, h->E, s);
+    // the offsets share the phase's nearfield image (6 us each at 1024^2)
+    st = forward_enqueue(h, k > 0 && forward_reads_image(h) ? kSrcImage : kSrcPhase, phase, nullptr, h->E, s);
     if (st != ASH_OK) break;
     k_abs2<<<(N + 255) / 256, 256, 0, s>>>(h->E, intensity + (size_t)k * N, N);
     if ((e = cudaGetLastError()) != cudaSuccess) st = cuda_fail(e, "calibration sweep");
