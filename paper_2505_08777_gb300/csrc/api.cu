@@ -181,10 +181,11 @@ bool use_tc_adj(const ash_hologram* h) {
 // 82 / 49, 901 x 611 N = 230 90 / 85. A forward step and an adjoint tile cost
 // the same however few spots they have: with fewer than 64 they pay only where
 // most tiles need one strip (forward: 742 x 486 N = 27 25 / 33, 1024^2 N = 20
-// 52 / 36). Degree 2 (one mixed term): forward 220^2 N = 30 12.5 / 13.8,
+// 52 / 36, 800^2 N = 12 31 / 27; adjoint 16 / 31, 39 / 22, 27 / 18). Degree 2
+// (one mixed term): forward 220^2 N = 30 12.5 / 13.8,
 // 300^2 N = 200 28 / 17; adjoint 256^2 N = 100 13.5 / 16.4, 300^2 N = 200
 // 24 / 20.
-constexpr int kSepSideFwd = 400, kSepSideAdj = 560, kSepSide2 = 200, kSepFewSpots = 64, kSepFewSide = 900;
+constexpr int kSepSideFwd = 400, kSepSideAdj = 560, kSepSide2 = 200, kSepFewSpots = 64, kSepFewSide = 800;
 constexpr size_t kSepMaxBytes = (size_t)8 << 30;   // of phase polynomials, and of partial dL/dC an eighth
 constexpr long long kSepTerms2Fwd = 6LL << 20, kSepTerms2Adj = 10LL << 20;
 bool sep_pays(const ash_hologram* h, int side4, long long terms2) {
