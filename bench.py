@@ -123,6 +123,10 @@ def ncu_traffic(kernel):
     return None
 
 
+# terms per clock and SM of the separable kernels' tensor-core products
+SEP_TERMS_PER_CLK_SM = 128
+
+
 def roofline_alu(achieved, D, rates, kernel, algorithmic):
     """roofline object of an ALU-bound transform: peak = the FP32/SFU
     roofline R_terms = SMs x f_clk x min(FP32 / (D + 7), MUFU / 2) from the
@@ -506,7 +510,19 @@ def main():
                                 f"spots into TMEM, sincos + packed complex MAC, arg epilogue)") if adj_tc else
                                f"k_adjoint<D={p.D},P={P}> (pixel-stationary adjoint, arg epilogue)"}
     achieved = gterm[dom]
+    sep = max(p.noll) <= 15 and min(p.nx, p.ny) >= 560 and p.N >= 64   # the automatic choice of the separable kernels
+    if sep:
+        kernel_names = {"forward": "k_sep_forward (tile rows on tcgen05 split-f16 MMA, 64 sincos per spot and tile)",
+                        "adjoint": "k_sep_adjoint (tile sums on tcgen05 split-f16 MMA, 64 sincos per spot and tile)"}
     roofline = roofline_alu(achieved, p.D, rates, kernel_names[dom], f"N*M = {NM} terms")
+    if sep:
+        # R_terms counts one sin / cos per term; these kernels are bounded by their tensor-core products instead
+        mhz = max_sm_mhz()[0]
+        peak = rates["sms"] * SEP_TERMS_PER_CLK_SM * mhz * 1e6 / 1e9
+        roofline.update({"bound": "tensor", "r_terms": roofline["peak"], "frac_r_terms": roofline["frac"],
+                         "r_terms_basis": roofline["peak_basis"], "peak": peak, "frac": achieved / peak,
+                         "peak_basis": f"split-f16 products of a (128 spots, 32 x 32 tile) step: 131072 terms in 1024 "
+                                       f"clocks of the tensor core, {SEP_TERMS_PER_CLK_SM} terms/clk/SM at {mhz:.0f} MHz"})
     roofline["per_kernel_frac"] = {k: v / roofline["peak"] for k, v in gterm.items()}
     if clk.get("sm_mhz"):
         roofline["frac_at_sampled_clock"] = achieved / (roofline["peak"] * clk["sm_mhz"] / max_sm_mhz()[0])

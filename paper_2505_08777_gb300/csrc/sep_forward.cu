@@ -212,6 +212,14 @@ __global__ void k_sep_scan(const unsigned char* __restrict__ strips, int U, int 
 // apply Q_k(v) and Y(v). The low parts of the operands enter for k = 0, 1
 // only: |Q_2|, |Q_3| < 0.01. A, B and D have two buffers each, so the
 // generators, the tensor core and the summers work on different steps.
+//
+// Bound: the FP32 pipe, about 2100 clocks of a 3600-clock step (128 spots of a
+// tile, one strip) against 1024 of tensor core and 1400 of shared memory; at
+// 1024^2, N = 1024: FMA pipe 58 % busy, issue 56 %, tensor core 27 %, DRAM 9 %.
+// The rest is the hand-over between the roles. Kernel times, before (one
+// sine and cosine per term) / now: 1024^2 N = 400 252 / 60 us, 1024^2 N = 1024
+// 571 / 104, 1920 x 1152 N = 2000 2365 / 430. Two uniform CTAs per SM took 75
+// (540), one uniform CTA with lookahead 92 (858), MMAs issued by a generator 74.
 constexpr int kFwdThreads = 640;
 // Registers: 20 warps launch with 96 a thread; the summers take 120, the
 // generators keep 96, the last warpgroup drops to 40.
@@ -271,6 +279,12 @@ __device__ __forceinline__ void sep_sum_pair(const SepPoly& q, float R1s, float 
   acc.sr = fma2(sn, Tr, acc.sr);
 }
 
+// The coefficient gradient runs on the same steps: the summers keep the 14
+// moments of degree <= 4 of their spot instead of its field and fold them with
+// the modes' tile polynomials once per (spot block, tile), so that its time is
+// the summers' (FP32; 1024^2 N = 400 D = 10: 301 -> 146 us, N = 1024: 569 -> 236,
+// before: a sine and cosine and 14 multiply-adds per term).
+//
 // Moments of a tile over its pixels, Im(conj(gE) f K) mx^k my^l summed: m0[l]
 // (k = 0), m1, m2, m3.
 struct SepMoments {
@@ -736,7 +750,8 @@ __global__ void k_sep_gradc_reduce(const float* __restrict__ part, int rows, int
 }
 
 // E_n = the sum of the CTAs' partial rows, in a fixed order: row-lane k of the
-// 32 x 32 threads adds rows k, k + 32, ..., then a fixed-shape tree.
+// 32 x 32 threads adds rows k, k + 32, ..., then a fixed-shape tree. Latency
+// bound: 4.4 us for the 304 rows of N = 400 (1.2 MB from L2).
 __global__ void k_sep_forward_reduce(const float2* __restrict__ part, int rows, int npad, int N,
                                      float2* __restrict__ E) {
   __shared__ float2 acc[32][33];
