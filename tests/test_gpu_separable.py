@@ -1,7 +1,6 @@
 """GPU parity of the separable tile transforms (csrc/sep_forward.cu,
 csrc/sep_adjoint.cu) at the sizes where the automatic choice takes them:
-remainders of 32 and 128 spots (7, 20, 1: four copies of the last
-block's spots; 64, 33, 44: two), ragged last tiles, row strips from 1 to 32
+remainders of 32 and 128 spots, ragged last tiles, row strips from 1 to 32
 (coefficients scaled), bases of degree 2 and 4, few spots on a large grid,
 bands, and the same calls under capture.
 
