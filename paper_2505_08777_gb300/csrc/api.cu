@@ -208,13 +208,16 @@ bool use_tc_grad(const ash_hologram* h) {
   return h->variant == 2 || h->g.N >= kTcFwdMinSpots;
 }
 
-// The moments take u^4 as u^2 - 1/8 over a tile: with degree 4 the dropped part
-// of dL/dC, (16 / R)^4 of a quartic mode's scale, is below 1e-6 from this side
-// (2.5e-6 at 700).
-constexpr int kSepSideGrad4 = 900;
+// The moments take u^4 as u^2 - 1/8 over a tile, off by up to 1/8. What that
+// drops of dL/dC scales with (16 / R)^4 for a quartic mode and, through the
+// mixed terms of the second moments (Q_2 < 0.005 in a strip), with
+// 0.005 / 8 (16 / R)^2 for any: from this side both are below 1e-6 (degree 4:
+// 2.5e-6 at 700; degree 2: dL/dC off by 7.9e-6 against the other kernel's
+// 3.1e-6 at side 354, 3.0e-6 against 1.5e-6 at 460, in the same time).
+constexpr int kSepSideGrad = 900;
 bool use_sep_grad(const ash_hologram* h) {
   const int side = h->g.nx < h->g.ny_full ? h->g.nx : h->g.ny_full;
-  return use_sep_adj(h) && h->sep_dpart && (h->sep_ord < 4 || side >= kSepSideGrad4);
+  return use_sep_adj(h) && h->sep_dpart && side >= kSepSideGrad;
 }
 
 // Whether any kernel but the separable ones may read czs and rot.

@@ -33,7 +33,7 @@ CASES = [
     (233, 201, 231, [2, 3, 4, 5, 6], 1.0),
     (930, 901, 67, LOW, 1.0),
     (577, 590, 172, LOW, 6.0),
-    (901, 930, 20, LOW, 1.0),
+    (901, 930, 20, [2, 3, 4, 5, 6], 1.0),
     (905, 903, 161, LOW, 1.0),
 ]
 
