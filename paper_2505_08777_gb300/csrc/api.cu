@@ -457,7 +457,7 @@ ash_status enqueue_adjoint(ash_hologram* h, const float2* y, float2* g_out, floa
   p.out.dphase = dphase;
   p.out.epilogue = epilogue;
   if (use_sep_adj(h)) {
-    cudaError_t e = sep_launch_scale(y, h->g.N, h->sep_ys, h->sep_scale, s);
+    cudaError_t e = sep_launch_scale(y, h->g.N, h->sep_ys, h->sep_scale, h->sep_tickets, h->g.T, s);
     if (e == cudaSuccess) e = sep_launch_adjoint(sep_adj_params(h, y, p.out), s);
     return e == cudaSuccess ? ASH_OK : cuda_fail(e, "separable adjoint launch");
   }
@@ -1027,10 +1027,7 @@ ash_status create_impl(ash_hologram** out, int nx, int ny, int row0, int ny_full
     // pixels outside the grid stay 0 in every nearfield image
     CREATE_CUDA(cudaMemsetAsync(h->fimg, 0, tc_fimg_float4s(g) * sizeof(float4), s));
   }
-  if (h->sep_ok) {
-    CREATE_CUDA(sep_build_table(g, h->terms, h->term_off, h->sep_tab, s));
-    CREATE_CUDA(cudaMemsetAsync(h->sep_tickets, 0, (size_t)g.T * sizeof(int), s));
-  }
+  if (h->sep_ok) CREATE_CUDA(sep_build_table(g, h->terms, h->term_off, h->sep_tab, s));
   CREATE_CUDA(enqueue_tc_coeff(h, s));
   k_amp_image<<<g.T, g.NT, 0, s>>>(g, amp, h->amp_img);
   CREATE_CUDA(cudaGetLastError());
@@ -1415,7 +1412,7 @@ ash_status ash_profile(ash_hologram* h, const float* phase, const float* y, floa
   ap.out.epilogue = kEpiPhase;
   const TcAdjParams tp = tc_adj_params(h, y2, ap.out);
   const SepAdjParams spa = sep_adj_params(h, y2, ap.out);
-  if (e == cudaSuccess && sa) e = sep_launch_scale(y2, h->g.N, h->sep_ys, h->sep_scale, s);
+  if (e == cudaSuccess && sa) e = sep_launch_scale(y2, h->g.N, h->sep_ys, h->sep_scale, h->sep_tickets, h->g.T, s);
   if (e == cudaSuccess) {
     cudaEventRecord(ev[4], s);
     e = sa ? sep_launch_adjoint(spa, s) : tca ? tc_launch_adjoint(h->tc_na, tp, h->tadj.G, s) : launch_adjoint(h->g.D, ap, h->sched.G, s);

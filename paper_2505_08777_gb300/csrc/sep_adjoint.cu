@@ -191,7 +191,6 @@ __global__ void __launch_bounds__(kAdjThreads, 1) k_sep_adjoint(const SepAdjPara
           const int g_lo = adj_owner(W, G, p.cost[u0]);
           const int g_hi = adj_owner(W, G, p.cost[u1] - sep_chunk_cost(p.strips[u1 - 1]));
           const bool last = atomicAdd(&p.tickets[x.tile], 1) == g_hi - g_lo;
-          if (last) p.tickets[x.tile] = 0;
           flag[0] = last ? g_lo : -1;
           flag[1] = g_hi;
         }
@@ -463,19 +462,21 @@ __global__ void __launch_bounds__(kAdjThreads, 1) k_sep_adjoint(const SepAdjPara
 }
 
 // One warp per chunk of 32 spots (1.4 us, its launch; the adjoint fetches the
-// result with the phase polynomials).
+// result with the phase polynomials). It also sets the split tiles' counts to
+// zero, so that an adjoint whose wait ran out leaves none behind for the next.
 __global__ void k_sep_scale(const float2* __restrict__ y, int N, int chunks, float* __restrict__ ys,
-                            float* __restrict__ scale) {
+                            float* __restrict__ scale, int* __restrict__ tickets, int T) {
   pdl_begin();
+  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < T; k += gridDim.x * blockDim.x) tickets[k] = 0;
   const int c = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
   if (c < chunks) sep_scale_chunk(y, N, c, ys, scale);
 }
 
 }  // namespace
 
-cudaError_t sep_launch_scale(const float2* y, int N, float* ys, float* scale, cudaStream_t s) {
+cudaError_t sep_launch_scale(const float2* y, int N, float* ys, float* scale, int* tickets, int T, cudaStream_t s) {
   const int chunks = sep_blocks(N) * (kSepSpots / kSepChunk);
-  return launch_pdl(k_sep_scale, (chunks + 3) / 4, 128, 0, s, y, N, chunks, ys, scale);
+  return launch_pdl(k_sep_scale, (chunks + 3) / 4, 128, 0, s, y, N, chunks, ys, scale, tickets, T);
 }
 
 cudaError_t sep_adjoint_prepare() {

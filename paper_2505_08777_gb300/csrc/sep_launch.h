@@ -71,13 +71,14 @@ struct SepAdjParams {
   const float* ys;               // [4 nb][re, im][32] y / scale
   const float* scale;            // [4 nb] power of two per chunk of 32 spots
   float2* split;                 // [G][2][kTilePix] partial sums of tiles split between CTAs
-  int* tickets;                  // [T] CTAs done with a split tile (left at 0)
+  int* tickets;                  // [T] CTAs done with a split tile (0 at the start)
   int G;
 };
 cudaError_t sep_prepare();
 cudaError_t sep_adjoint_prepare();
-// y divided by a power of two (scale) per chunk of 32 spots.
-cudaError_t sep_launch_scale(const float2* y, int N, float* ys, float* scale, cudaStream_t s);
+// y divided by a power of two (scale) per chunk of 32 spots; the counts of the
+// T tiles set to 0. Goes before every adjoint.
+cudaError_t sep_launch_scale(const float2* y, int N, float* ys, float* scale, int* tickets, int T, cudaStream_t s);
 cudaError_t sep_launch_adjoint(const SepAdjParams& p, cudaStream_t s);
 cudaError_t sep_launch_forward(const SepFwdParams& p, cudaStream_t s);          // partial sums
 cudaError_t sep_launch_forward_reduce(const SepFwdParams& p, cudaStream_t s);   // E from them
