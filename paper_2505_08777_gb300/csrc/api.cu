@@ -194,11 +194,23 @@ bool sep_pays(const ash_hologram* h, int side4, long long terms2) {
   if (h->sep_ord <= 2) return side >= kSepSide2 && (long long)g.nx * g.ny * g.N >= terms2;
   return side >= side4 && (g.N >= kSepFewSpots || side >= kSepFewSide);
 }
-bool use_sep_fwd(const ash_hologram* h) {
-  return h->sep_ok && h->variant == 0 && sep_pays(h, kSepSideFwd, kSepTerms2Fwd);
+// WGS loops (and the batches made of them) take the separable transforms from
+// this side only, whatever the degree. An iteration divides by the spots'
+// amplitudes, so where one passes near zero the loop multiplies the transforms'
+// rounding, of either kind, by 100 and more (weights of 512^2 N = 196, five
+// iterations: 2e-7 off at most starting points, 1.8e-5 at one, where the
+// other kernels' rounding moved them by 3.7e-5); small holograms keep the
+// results that they had. Without the line a batch of 16 holograms of 256^2 to
+// 512^2 takes 1.93 instead of 2.13 ms.
+constexpr int kSepSideLoop = 560;
+bool sep_in_loops(const ash_hologram* h) {
+  return (h->g.nx < h->g.ny_full ? h->g.nx : h->g.ny_full) >= kSepSideLoop;
 }
-bool use_sep_adj(const ash_hologram* h) {
-  return h->sep_ok && h->variant == 0 && sep_pays(h, kSepSideAdj, kSepTerms2Adj);
+bool use_sep_fwd(const ash_hologram* h, bool loop = false) {
+  return h->sep_ok && h->variant == 0 && (!loop || sep_in_loops(h)) && sep_pays(h, kSepSideFwd, kSepTerms2Fwd);
+}
+bool use_sep_adj(const ash_hologram* h, bool loop = false) {
+  return h->sep_ok && h->variant == 0 && (!loop || sep_in_loops(h)) && sep_pays(h, kSepSideAdj, kSepTerms2Adj);
 }
 // The coefficient-gradient moments on the tensor cores need one K-atom,
 // D <= 12 and a polynomial basis of total degree <= 4 (the tile polynomials);
@@ -222,13 +234,14 @@ bool use_sep_grad(const ash_hologram* h) {
 
 // Whether any kernel but the separable ones may read czs and rot.
 bool needs_tc_images(const ash_hologram* h) {
-  return h->tc_ok && (h->tc_pinned || !(use_sep_fwd(h) && use_sep_adj(h) && use_sep_grad(h)));
+  return h->tc_ok && (h->tc_pinned || !(use_sep_fwd(h, true) && use_sep_adj(h, true) && use_sep_grad(h)));
 }
 
 // Whether the handle's current kernel choice runs any FMA-pipe kernel (they
 // read the register-image basis dz; the tensor-core kernels do not).
 bool needs_fma_image(const ash_hologram* h) {
-  return !((use_sep_fwd(h) || use_tc_fwd(h)) && (use_sep_adj(h) || use_tc_adj(h)) && (use_sep_grad(h) || use_tc_grad(h)));
+  return !((use_sep_fwd(h, true) || use_tc_fwd(h)) && (use_sep_adj(h, true) || use_tc_adj(h)) &&
+           (use_sep_grad(h) || use_tc_grad(h)));
 }
 
 // CTA range starts that give every CTA the same estimated time rather than
@@ -405,16 +418,17 @@ cudaError_t launch_gradc(int D, const GradCParams& p, dim3 grid, cudaStream_t s)
   return cudaErrorInvalidValue;
 }
 
-// forward transform into E (device complex [N]).
+// forward transform into E (device complex [N]); loop: as a WGS loop runs it.
 ash_status enqueue_forward(ash_hologram* h, int source, const float* phase, const float2* field, float2* E,
-                           cudaStream_t s) {
-  if (use_sep_fwd(h) || use_tc_fwd(h)) {
+                           cudaStream_t s, bool loop = false) {
+  const bool sep = use_sep_fwd(h, loop);
+  if (sep || use_tc_fwd(h)) {
     cudaError_t e = cudaSuccess;
     if (source != kSrcImg) {
       e = tc_field_img(h->g, h->amp_img, source == kSrcPhase ? phase : nullptr, field, h->fimg, s);
       if (e != cudaSuccess) return cuda_fail(e, "nearfield image launch");
     }
-    if (use_sep_fwd(h)) {
+    if (sep) {
       const SepFwdParams sp = sep_fwd_params(h, E);
       e = sep_launch_forward(sp, s);
       if (e == cudaSuccess) e = sep_launch_forward_reduce(sp, s);
@@ -447,7 +461,7 @@ ash_status enqueue_forward(ash_hologram* h, int source, const float* phase, cons
 }
 
 ash_status enqueue_adjoint(ash_hologram* h, const float2* y, float2* g_out, float* phase_out, const float* phase_in,
-                           float* dphase, int epilogue, cudaStream_t s) {
+                           float* dphase, int epilogue, cudaStream_t s, bool loop = false) {
   AdjParams p{};
   p.v = view_of(h);
   p.y = y;
@@ -456,7 +470,7 @@ ash_status enqueue_adjoint(ash_hologram* h, const float2* y, float2* g_out, floa
   p.out.phase_in = phase_in;
   p.out.dphase = dphase;
   p.out.epilogue = epilogue;
-  if (use_sep_adj(h)) {
+  if (use_sep_adj(h, loop)) {
     cudaError_t e = sep_launch_scale(y, h->g.N, h->sep_ys, h->sep_scale, h->sep_tickets, h->g.T, s);
     if (e == cudaSuccess) e = sep_launch_adjoint(sep_adj_params(h, y, p.out), s);
     return e == cudaSuccess ? ASH_OK : cuda_fail(e, "separable adjoint launch");
@@ -487,20 +501,22 @@ ash_status enqueue_adjoint(ash_hologram* h, const float2* y, float2* g_out, floa
 // metrics. When both transforms run on the tensor cores the adjoint also
 // writes the next forward's nearfield (kEpiFimg), so only the first forward
 // converts a phase.
-bool wgs_fused_field(const ash_hologram* h) { return (use_sep_fwd(h) || use_tc_fwd(h)) && (use_sep_adj(h) || use_tc_adj(h)); }
+bool wgs_fused_field(const ash_hologram* h) {
+  return (use_sep_fwd(h, true) || use_tc_fwd(h)) && (use_sep_adj(h, true) || use_tc_adj(h));
+}
 
 ash_status enqueue_wgs_body(ash_hologram* h, int iters, cudaStream_t s) {
   const bool tc = wgs_fused_field(h);
   const int adj_epi = tc ? (kEpiPhase | kEpiFimg) : kEpiPhase;
-  ash_status st = enqueue_forward(h, kSrcPhase, h->wgs_phase, nullptr, h->wgs_E, s);
+  ash_status st = enqueue_forward(h, kSrcPhase, h->wgs_phase, nullptr, h->wgs_E, s, true);
   if (st != ASH_OK) return st;
   for (int it = 0; it < iters; ++it) {
     cudaError_t e = launch_pdl(k_wgs_update, 1, 1024, 0, s, h->wgs_E, h->wgs_w, h->wgs_T, h->y, h->g.N,
                                h->wgs_feedback, h->wgs_fix ? h->wgs_u : nullptr, h->wgs_fix ? nullptr : h->wgs_u);
     if (e != cudaSuccess) return cuda_fail(e, "wgs update launch");
-    st = enqueue_adjoint(h, h->y, nullptr, h->wgs_phase, nullptr, nullptr, adj_epi, s);
+    st = enqueue_adjoint(h, h->y, nullptr, h->wgs_phase, nullptr, nullptr, adj_epi, s, true);
     if (st != ASH_OK) return st;
-    st = enqueue_forward(h, tc ? kSrcImg : kSrcPhase, h->wgs_phase, nullptr, h->wgs_E, s);
+    st = enqueue_forward(h, tc ? kSrcImg : kSrcPhase, h->wgs_phase, nullptr, h->wgs_E, s, true);
     if (st != ASH_OK) return st;
   }
   cudaError_t e = launch_pdl(k_metrics, 1, 1024, 0, s, h->wgs_E, h->wgs_T, h->g.N, h->sum_a2,
@@ -1358,9 +1374,10 @@ int ash_wgs_launches(const ash_hologram* h, int iters) {
   // forward: tensor-core (nearfield image unless fused, kernel, reduce if
   // split) or FMA (kernel, reduction); adjoint: kernel (+ fix-up)
   const bool fused = wgs_fused_field(h);
-  const int fwd_first = use_sep_fwd(h) ? 3 : use_tc_fwd(h) ? 2 + (h->tfwd_split ? 1 : 0) : 2;
-  const int fwd = use_sep_fwd(h) ? (fused ? 2 : 3) : use_tc_fwd(h) ? (fused ? 1 : 2) + (h->tfwd_split ? 1 : 0) : 2;
-  const int adj = use_sep_adj(h) ? 2 : use_tc_adj(h) ? 1 + (h->tadj_split ? 1 : 0) : 1 + (h->split_tiles ? 1 : 0);
+  const bool sep = use_sep_fwd(h, true);
+  const int fwd_first = sep ? 3 : use_tc_fwd(h) ? 2 + (h->tfwd_split ? 1 : 0) : 2;
+  const int fwd = sep ? (fused ? 2 : 3) : use_tc_fwd(h) ? (fused ? 1 : 2) + (h->tfwd_split ? 1 : 0) : 2;
+  const int adj = use_sep_adj(h, true) ? 2 : use_tc_adj(h) ? 1 + (h->tadj_split ? 1 : 0) : 1 + (h->split_tiles ? 1 : 0);
   return fwd_first + iters * (1 + adj + fwd) + 1;   // + metrics
 }
 
