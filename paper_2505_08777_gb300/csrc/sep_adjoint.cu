@@ -35,11 +35,18 @@ constexpr int kAdjThreads = 896;
 // to 40, the generators take 80.
 static_assert(2 * 72 + 40 + 4 * 80 <= 7 * 72);
 constexpr int kAdjBufs = 3, kAdjSlots = 8;
+// Barriers of the steps' MMAs. A wait names a phase by its parity, so a barrier
+// may not come round again before every waiter has seen it: the generators of
+// step it wait for step it - 3, and nothing of step it holds back step it + 1
+// (other generators, another issuer), which with one barrier per D buffer is
+// that barrier's next phase. With eight it is step it + 5, whose sums go where
+// step it + 1's were, read after step it's.
+constexpr int kAdjFull = 8;
 constexpr uint32_t kAA = 32768, kAB = 16384, kASlot = 2048 + 256;
 constexpr uint32_t kAdjB = kAdjBufs * kAA, kAdjSum = kAdjB + kAdjBufs * kAB;   // sums of the planes: [4][32][33] float2
 constexpr uint32_t kAdjSlot0 = kAdjSum + 4 * 32 * 33 * 8, kAdjTail = kAdjSlot0 + kAdjSlots * kASlot;
 constexpr size_t kAdjSmem = 1024 + kAdjTail + 512;
-static_assert(30 * 8 + 16 + kAdjSlots * 16 <= 512 && kAdjTail % 16 == 0);
+static_assert(kAdjFull == 8 && (kAdjFull + 26) * 8 + 16 + kAdjSlots * 16 <= 512 && kAdjTail % 16 == 0);
 static_assert(kAdjSum % 16 == 0 && kAdjSlot0 % 16 == 0 && kAdjTail % 8 == 0);
 
 // A step's record, read as one 16-byte word.
@@ -86,12 +93,12 @@ __device__ __forceinline__ int adj_owner(long long W, int G, int c) {
 __global__ void __launch_bounds__(kAdjThreads, 1) k_sep_adjoint(const SepAdjParams p) {
   extern __shared__ uint8_t raw[];
   uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(raw) + 1023) & ~(uintptr_t)1023);
-  uint64_t* full = reinterpret_cast<uint64_t*>(sm + kAdjTail);   // [4] MMAs of a step done
-  uint64_t* empty = full + 4;                                    // [8] its D and record read
-  uint64_t* ready = full + 12;                                   // [8] its operands written
-  uint64_t* listed = full + 20;                                  // [8] its record and spots written
-  uint64_t* summed = full + 28;                                  // the adders' meeting point at a tile's end
-  uint32_t* slot = reinterpret_cast<uint32_t*>(full + 30);
+  uint64_t* full = reinterpret_cast<uint64_t*>(sm + kAdjTail);   // [8] MMAs of a step done
+  uint64_t* empty = full + kAdjFull;                             // [8] its D and record read
+  uint64_t* ready = empty + 8;                                   // [8] its operands written
+  uint64_t* listed = ready + 8;                                  // [8] its record and spots written
+  uint64_t* summed = listed + 8;                                 // the adders' meeting point at a tile's end
+  uint32_t* slot = reinterpret_cast<uint32_t*>(summed + 2);
   AdjStep* steps = reinterpret_cast<AdjStep*>(slot + 4);         // [8]
   const int t = threadIdx.x, w = t >> 5, lane = t & 31;
   const int N = p.a.g.N, nb = p.nb, npad = nb * kSepSpots, U = p.a.g.T * nb;
@@ -100,7 +107,7 @@ __global__ void __launch_bounds__(kAdjThreads, 1) k_sep_adjoint(const SepAdjPara
     reinterpret_cast<uint4*>(sm + (k >> 9) * kAA + 16384 + 8192)[k & 511] = make_uint4(0, 0, 0, 0);
   if (w == 0) tmem_alloc(slot, 512);
   if (t == 0) {
-    for (int k = 0; k < 29; ++k) mbar_init(full + k, (k >= 4 && k < 12) || k == 28 ? 8 : 1);
+    for (uint64_t* b = full; b <= summed; ++b) mbar_init(b, (b >= empty && b < ready) || b == summed ? 8 : 1);
     fence_mbar_init();
   }
   fence_async_smem();
@@ -132,7 +139,7 @@ __global__ void __launch_bounds__(kAdjThreads, 1) k_sep_adjoint(const SepAdjPara
     for (int i = 0; i < 16; ++i) acc[i] = make_float2(0.0f, 0.0f);
     for (uint32_t it = 0; blockIdx.x < G; ++it) {
       const int sl = it & 7, d = it & 3;
-      ok = ok && sep_wait(&full[d], (it >> 2) & 1);
+      ok = ok && sep_wait(&full[sl], (it >> 3) & 1);
       ok = __all_sync(0xffffffffu, ok);
       if (!ok) break;
       const AdjStep x = adj_step(steps + sl);
@@ -262,10 +269,10 @@ __global__ void __launch_bounds__(kAdjThreads, 1) k_sep_adjoint(const SepAdjPara
         for (int ks = 0; ks < 8; ks += 2) umma_f16(dst, a + ks, b + ks, umma_idesc_f16(128, 128), ks > 0);
 #pragma unroll
         for (int ks = 0; ks < 8; ks += 2) umma_f16(dst + 64, al + ks, b + ks, umma_idesc_f16(128, 64), 1u);
-        umma_commit(&full[d]);
+        umma_commit(&full[sl]);
       }
       // nothing in flight when the CTA gives up its memory
-      if (it >= 3) ok = sep_wait(&full[(it - 3) & 3], ((it - 3) >> 2) & 1) && ok;
+      if (it >= 3) ok = sep_wait(&full[(it - 3) & 7], ((it - 3) >> 3) & 1) && ok;
     } else if (w == 8 && lane == 0) {
       // --- steps of this CTA: the chunks whose place in the cost prefix lies in [c0, c1) ---
       const int c0 = blockIdx.x < G ? (int)(W * blockIdx.x / G) : 0;
@@ -345,7 +352,7 @@ __global__ void __launch_bounds__(kAdjThreads, 1) k_sep_adjoint(const SepAdjPara
       const int sl = it & 7;
       ok = ok && sep_wait(&listed[sl], (it >> 3) & 1);
       // the MMAs of step it - 3 are done: its X is free
-      if (it >= 3) ok = ok && sep_wait(&full[(it - 3) & 3], ((it - 3) >> 2) & 1);
+      if (it >= 3) ok = ok && sep_wait(&full[(it - 3) & 7], ((it - 3) >> 3) & 1);
       AdjStep x{-4, 0u, -1, 0.0f};
       if (ok) x = adj_step(steps + sl);
       if (x.tile >= 0) {
