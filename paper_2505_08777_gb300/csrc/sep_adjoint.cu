@@ -53,7 +53,7 @@ static_assert(kAdjSum % 16 == 0 && kAdjSlot0 % 16 == 0 && kAdjTail % 8 == 0);
 struct __align__(16) AdjStep {
   int tile;        // negative: no more steps
   uint32_t bits;   // s | ls << 8 | a << 16 | end << 18: strip s of 2^ls, buffer of W
-  int used;        // the last step that used that buffer before this chunk (negative: none)
+  int used;        // 2 (the last step that used that buffer before this chunk, or -1) + (that chunk had several strips)
   float scale;     // 2^e: y is divided by it
   __device__ int s() const { return (int)(bits & 255u); }
   __device__ int ls() const { return (int)(bits >> 8 & 255u); }
@@ -287,7 +287,7 @@ __global__ void __launch_bounds__(kAdjThreads, 1) k_sep_adjoint(const SepAdjPara
       int cc = sep_chunk_cost(ls), c = (c0 - pos + cc - 1) / cc, s = 0, a = 0;
       pos += c * cc;
       int ls1 = u + 1 < U ? p.strips[u + 1] : 0;   // of the next unit, fetched early
-      int used[kAdjBufs] = {-1, -1, -1};   // last steps of the last three chunks
+      int used[kAdjBufs] = {-2, -2, -2};   // of the last three chunks, as AdjStep::used
       uint32_t it = 0;
       for (;; ++it) {
         const int sl = it & 7;
@@ -309,7 +309,7 @@ __global__ void __launch_bounds__(kAdjThreads, 1) k_sep_adjoint(const SepAdjPara
           // an end for each group of generators (-1, -2) and each issuer
           for (uint32_t k = it; k < it + 3; ++k)
             if (k >= 8) ok = ok && sep_wait(&empty[k & 7], ((k >> 3) - 1) & 1);
-          for (uint32_t k = it; k < it + 3; ++k) put_step(steps + (k & 7), -1 - (int)(k - it), 0, -1, 0.0f);
+          for (uint32_t k = it; k < it + 3; ++k) put_step(steps + (k & 7), -1 - (int)(k - it), 0, -2, 0.0f);
           mbar_arrive(&listed[it & 7]);
           mbar_arrive(&listed[(it + 1) & 7]);
           break;
@@ -333,7 +333,7 @@ __global__ void __launch_bounds__(kAdjThreads, 1) k_sep_adjoint(const SepAdjPara
           a = a == kAdjBufs - 1 ? 0 : a + 1;
           used[0] = used[1];
           used[1] = used[2];
-          used[2] = (int)it;
+          used[2] = 2 * (int)it + (ls > 0 ? 1 : 0);
         }
       }
       for (uint32_t k = it > 5 ? it - 5 : 0; k < it; ++k) ok = sep_wait(&listed[k & 7], (k >> 3) & 1) && ok;
@@ -353,7 +353,7 @@ __global__ void __launch_bounds__(kAdjThreads, 1) k_sep_adjoint(const SepAdjPara
       ok = ok && sep_wait(&listed[sl], (it >> 3) & 1);
       // the MMAs of step it - 3 are done: its X is free
       if (it >= 3) ok = ok && sep_wait(&full[(it - 3) & 7], ((it - 3) >> 3) & 1);
-      AdjStep x{-4, 0u, -1, 0.0f};
+      AdjStep x{-4, 0u, -2, 0.0f};
       if (ok) x = adj_step(steps + sl);
       if (x.tile >= 0) {
         const int xs = x.s(), xl = x.ls();
@@ -363,11 +363,13 @@ __global__ void __launch_bounds__(kAdjThreads, 1) k_sep_adjoint(const SepAdjPara
         const float2 c11 = word(kWC11), c21 = word(kWC21), c12 = word(kWC12), c22 = word(kWC22), n31 = word(kWN31),
                      c13 = word(kWC13);
         if (xs == 0) {
-          // W's buffer: the MMAs of its last user are done (step it - 3: above;
-          // more than 7 steps ago: the record's slot was free; they are issued by
-          // three threads, so a later step's say nothing)
-          if (x.used >= 0 && (int)it - x.used > 3 && (int)it - x.used < 8)
-            ok = ok && sep_wait(&empty[x.used & 7], (x.used >> 3) & 1);
+          // W's buffer: the MMAs of all strips of its last user are done. Those of
+          // step it - 3: above. More than 7 steps ago: the record's slot was free.
+          // Else by its last step's sums having been read, which is after all
+          // earlier steps'; the MMAs are issued by three threads, so that another
+          // step's being done says nothing.
+          const int used = x.used >> 1, ago = (int)it - used;
+          if (used >= 0 && ago < 8 && (ago > 3 || (x.used & 1))) ok = ok && sep_wait(&empty[used & 7], (used >> 3) & 1);
           const float2 yr = word(16), yi = word(17), nyi = sub2(make_float2(0.0f, 0.0f), yi);
           const float2 base = word(kWBase), ay = word(kWAy), y2 = word(kWY2), y3 = word(kWY3), y4 = word(kWY4);
           const float2 ayl = make_float2(__uint_as_float(__float_as_uint(lo.x) & 0xffff0000u),

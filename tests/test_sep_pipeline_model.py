@@ -120,9 +120,9 @@ class Adjoint(Model):
 
     SLOTS, BUFS, DBUFS = 8, 3, 4
 
-    def __init__(self, rng, chunks, ends, nfull=ADJ_FULL, x_wait=True):
+    def __init__(self, rng, chunks, ends, nfull=ADJ_FULL, x_wait=True, w_wait=True):
         super().__init__(rng)
-        self.nf, self.x_wait = nfull, x_wait
+        self.nf, self.x_wait, self.w_wait = nfull, x_wait, w_wait
         self.steps = []                      # (chunk, strip, last step that used W's buffer, tile end)
         last = []
         for c, ls in enumerate(chunks):
@@ -200,7 +200,8 @@ class Adjoint(Model):
                 c, s, used, _ = self.steps[it]
                 check(it < self.BUFS or self.done[it - self.BUFS], f"X of step {it - 3} overwritten early")
                 if s == 0:
-                    if used >= 0 and 3 < it - used < 8:
+                    several = self.w_wait and used >= 0 and self.steps[used][1] > 0
+                    if used >= 0 and it - used < 8 and (it - used > 3 or several):
                         yield wait(self.empty[used % S], used // S)
                     check(used < 0 or all(self.done[k] for k in range(used + 1) if self.steps[k][0] == c - self.BUFS),
                           f"W of chunk {c - self.BUFS} overwritten early")
@@ -400,3 +401,18 @@ def caught(make):
 def test_planted_mistakes_are_caught():
     assert caught(lambda r: Adjoint(r, *schedule(r), nfull=4))
     assert caught(lambda r: Adjoint(r, *schedule(r), x_wait=False))
+
+
+# A chunk of two strips, then chunks of one: W's buffer is free again three
+# steps after the second strip, whose MMAs another thread issued than the
+# first strip's.
+SHORT = [1, 0, 0, 0, 1, 0, 0, 0, 1, 0, 0, 0]
+
+
+@pytest.mark.parametrize("seed", range(40))
+def test_first_strips_are_done_before_w_is_rewritten(seed):
+    Adjoint(random.Random(seed), SHORT, set()).play()
+
+
+def test_waiting_for_the_last_strip_alone_is_caught():
+    assert caught(lambda r: Adjoint(r, SHORT, set(), w_wait=False))
