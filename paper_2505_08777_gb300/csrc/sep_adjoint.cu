@@ -309,12 +309,14 @@ __global__ void __launch_bounds__(kAdjThreads, 1) k_sep_adjoint(const SepAdjPara
           // an end for each group of generators (-1, -2) and each issuer
           for (uint32_t k = it; k < it + 3; ++k)
             if (k >= 8) ok = ok && sep_wait(&empty[k & 7], ((k >> 3) - 1) & 1);
+          if (!ok) break;
           for (uint32_t k = it; k < it + 3; ++k) put_step(steps + (k & 7), -1 - (int)(k - it), 0, -2, 0.0f);
           mbar_arrive(&listed[it & 7]);
           mbar_arrive(&listed[(it + 1) & 7]);
           break;
         }
         if (it >= 8) ok = ok && sep_wait(&empty[sl], ((it >> 3) - 1) & 1);
+        if (!ok) break;   // the slot may still be read
         uint8_t* dst = sm + kAdjSlot0 + sl * kASlot;
         uint32_t end = 0;
         if (((s + 1) >> ls) && (pos + cc >= c1 || (c + 1 == sep_chunks(N, b) && b + 1 == nb))) {
@@ -336,7 +338,10 @@ __global__ void __launch_bounds__(kAdjThreads, 1) k_sep_adjoint(const SepAdjPara
           used[2] = 2 * (int)it + (ls > 0 ? 1 : 0);
         }
       }
-      for (uint32_t k = it > 5 ? it - 5 : 0; k < it; ++k) ok = sep_wait(&listed[k & 7], (k >> 3) & 1) && ok;
+      // every copy has landed when the CTA gives up its memory (after the ends,
+      // those of steps up to it - 6 have been read, and others' slots hold the ends)
+      const uint32_t open = ok ? 5 : 8;
+      for (uint32_t k = it > open ? it - open : 0; k < it; ++k) ok = sep_wait(&listed[k & 7], (k >> 3) & 1) && ok;
     }
   } else {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 80;");

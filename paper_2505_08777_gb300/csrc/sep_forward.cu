@@ -593,8 +593,9 @@ __global__ void __launch_bounds__(kFwdThreads, 1) k_sep_forward(const SepFwdPara
         const bool more = pos < c1;
         if (!more) {
           // an end for each of the two issuers
-          for (uint32_t k = it; k < it + 2; ++k) {
+          for (uint32_t k = it; k < it + 2; ++k)
             if (k >= 4) ok = ok && sep_wait(&empty[k & 3], ((k >> 2) - 1) & 1);
+          for (uint32_t k = it; ok && k < it + 2; ++k) {
             steps[k & 3] = SepStep{0, -1, 0, 0, 0};
             mbar_arrive(&listed[k & 3]);
           }
@@ -602,6 +603,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) k_sep_forward(const SepFwdPara
         }
         // slot it & 3 was step it - 4's
         if (it >= 4) ok = ok && sep_wait(&empty[it & 3], ((it >> 2) - 1) & 1);
+        if (!ok) break;   // the slot may still be read
         steps[it & 3] = x;
         mbar_expect_tx(&listed[it & 3], kFSlot);
         bulk_g2s(sm + kFwdSlots + (it & 3) * kFSlot, p.poly + ((size_t)x.tile * nb + x.b) * (16 * kSepSpots), kFSlot,
@@ -609,7 +611,10 @@ __global__ void __launch_bounds__(kFwdThreads, 1) k_sep_forward(const SepFwdPara
         pos += c;
         ++x.s;
       }
-      for (uint32_t k = it > 2 ? it - 2 : 0; k < it; ++k) ok = sep_wait(&listed[k & 3], (k >> 2) & 1) && ok;
+      // every copy has landed when the CTA gives up its memory (after the ends,
+      // those of steps up to it - 3 have been read, and others' slots hold the ends)
+      const uint32_t open = ok ? 2 : 4;
+      for (uint32_t k = it > open ? it - open : 0; k < it; ++k) ok = sep_wait(&listed[k & 3], (k >> 2) & 1) && ok;
     }
     __syncwarp();
   } else {

@@ -12,9 +12,15 @@ copies and MMAs landing late) and checks that
 * operands, accumulators and step records are overwritten only when all
   their readers are past them, and read only when complete.
 
-The numbers of barriers are read from the sources. Mistakes planted in the
-model (four barriers for the adjoint's MMAs, which the generators' wait can
-find two phases on; an operand buffer taken back early) have to be caught.
+In further runs one wait runs out, as all do after about a second, and the
+others in turn where they depend on it: every role has to end, no copy may go
+to a slot that is still in use, and no copy or MMA may be in flight when the
+last role ends, for the memory belongs to the next block then.
+
+The numbers of barriers and what the listers do after a wait that ran out are
+read from the sources. Mistakes planted in the model (four barriers for the
+adjoint's MMAs, which the generators' wait can find two phases on; an operand
+buffer taken back early; listers that run on) have to be caught.
 """
 import pathlib
 import random
@@ -29,7 +35,15 @@ def constant(name, file):
     return int(re.search(rf"\b{name} = (\d+)", (CSRC / file).read_text()).group(1))
 
 
+def lister_leaves(file):
+    """Whether the lister leaves its loop before it writes a step into a slot whose wait ran out."""
+    text = (CSRC / file).read_text()
+    text = text[text.index("// --- steps of this CTA"):]
+    return re.search(r"sep_wait\(&empty[^;]*;\s*if \(!ok\) break;[^;]*(;[^;]*){0,8}mbar_expect_tx", text) is not None
+
+
 ADJ_FULL = constant("kAdjFull", "sep_adjoint.cu")
+ADJ_LEAVES, FWD_LEAVES = lister_leaves("sep_adjoint.cu"), lister_leaves("sep_forward.cu")
 
 
 class Violation(AssertionError):
@@ -60,22 +74,30 @@ class Barrier:
 
 
 class Meeting:
-    """A named barrier of n warps (bar.sync, barrier.red)."""
+    """A named barrier of n warps that also tells whether one of them stops (barrier.red.or)."""
 
     def __init__(self, n):
-        self.n, self.come, self.gen = n, 0, 0
+        self.n, self.come, self.gen, self.stop = n, 0, 0, {0: False}
 
-    def arrive(self):
+    def arrive(self, stop=False):
+        gen = self.gen
+        self.stop[gen] = self.stop.get(gen, False) or stop
         self.come += 1
         if self.come == self.n:
             self.come, self.gen = 0, self.gen + 1
-            return self.gen
-        return self.gen + 1
+        return gen
+
+    def met(self, gen):
+        return self.gen > gen
 
 
 class Model:
-    def __init__(self, rng):
-        self.rng, self.procs, self.later = rng, {}, []
+    """Roles are generators that yield None (a step), (barrier, phase) (a wait: they are sent whether it was
+    over before it ran out) or a function (a named barrier). `fails`: one wait runs out, and then those that
+    nothing ends any more."""
+
+    def __init__(self, rng, fails=False):
+        self.rng, self.fails, self.failed, self.procs, self.later = rng, fails, False, {}, []
 
     def add(self, name, gen):
         self.procs[name] = [gen, None]
@@ -86,17 +108,40 @@ class Model:
         self.later.append(item)
         return item
 
+    def see(self, cond, what):
+        """What holds for the values, as long as no wait has run out."""
+        check(cond or self.failed, what)
+
+    def resume(self, name, answer):
+        g = self.procs[name]
+        try:
+            g[1] = g[0].send(answer)
+        except StopIteration:
+            g[1] = "end"
+
+    @staticmethod
+    def can(at):
+        return at is None or (at[0].passed(at[1]) if isinstance(at, tuple) else at != "end" and at())
+
     def play(self):
         speed = {n: 10 ** self.rng.uniform(-2, 0) for n in self.procs}
         speed["async"] = 10 ** self.rng.uniform(-2, 0)
-        for gen in self.procs.values():
-            gen[1] = next(gen[0], "end")
+        for n in self.procs:
+            self.resume(n, None)
+        left = self.rng.randint(1, 1200) if self.fails else -1
         while True:
             live = [n for n, g in self.procs.items() if g[1] != "end"]
-            ready = [n for n in live if self.procs[n][1] is None or self.procs[n][1]()]
+            ready = [n for n in live if self.can(self.procs[n][1])]
             land = [x for x in self.later if x[1] is None or x[1] not in self.later]
             if not live:
+                check(not land, "copies or MMAs in flight at the end")
                 return
+            waits = [n for n in live if isinstance(self.procs[n][1], tuple) and n not in ready]
+            left -= 1
+            if waits and (left == 0 or self.failed and not ready and not land):
+                self.failed = True
+                self.resume(self.rng.choice(waits), False)
+                continue
             check(ready or land, "every role waits: " + ", ".join(sorted(live)))
             names = ready + (["async"] if land else [])
             pick = self.rng.choices(names, [speed[n] for n in names])[0]
@@ -107,12 +152,7 @@ class Model:
                 self.later.remove(x)
                 x[0]()
             else:
-                g = self.procs[pick]
-                g[1] = next(g[0], "end")
-
-
-def wait(bar, phase):
-    return lambda: bar.passed(phase)
+                self.resume(pick, True)
 
 
 class Adjoint(Model):
@@ -120,9 +160,9 @@ class Adjoint(Model):
 
     SLOTS, BUFS, DBUFS = 8, 3, 4
 
-    def __init__(self, rng, chunks, ends, nfull=ADJ_FULL, x_wait=True, w_wait=True):
-        super().__init__(rng)
-        self.nf, self.x_wait, self.w_wait = nfull, x_wait, w_wait
+    def __init__(self, rng, chunks, ends, nfull=ADJ_FULL, x_wait=True, w_wait=True, leaves=ADJ_LEAVES, fails=False):
+        super().__init__(rng, fails)
+        self.nf, self.x_wait, self.w_wait, self.leaves = nfull, x_wait, w_wait, leaves
         self.steps = []                      # (chunk, strip, last step that used W's buffer, tile end)
         last = []
         for c, ls in enumerate(chunks):
@@ -138,10 +178,10 @@ class Adjoint(Model):
         self.listed = [Barrier(1) for _ in range(self.SLOTS)]
         self.summed = Barrier(8)
         self.slot = [None] * self.SLOTS      # step whose record it holds
-        self.wrote = [0] * n                 # generator warps done with a step's operands
+        self.copying = [False] * self.SLOTS
+        self.wrote = [0] * n                 # generator warps past a step's operands
         self.issued, self.done = [False] * n, [False] * n
         self.read = [0] * n                  # adder warps done with a step's sums
-        self.left = {}                       # steps past which a role is
         self.meet = [Meeting(8), Meeting(8)]
         self.add("lister", self.lister())
         for k in range(3):
@@ -156,6 +196,7 @@ class Adjoint(Model):
         old = it - self.SLOTS
         if 0 <= old < self.n:
             check(self.read[old] == 8 and self.wrote[old] == 8 and self.issued[old], f"record of step {old} rewritten early")
+        check(not self.copying[it % self.SLOTS], "a copy goes to a slot whose last copy is in flight")
         self.slot[it % self.SLOTS] = (it, end)
 
     def record(self, it):
@@ -163,73 +204,84 @@ class Adjoint(Model):
         return self.slot[it % self.SLOTS][1]
 
     def lister(self):
-        S = self.SLOTS
-        for it in range(self.n):
+        S, ok, it = self.SLOTS, True, 0
+        while it < self.n:
             if it >= S:
-                yield wait(self.empty[it % S], it // S - 1)
+                ok = ok and (yield self.empty[it % S], it // S - 1)
+            if not ok and self.leaves:
+                break
             self.put(it, 0)
             bar = self.listed[it % S]
             bar.tx += 1
+            self.copying[it % S] = True
             bar.arrive()
 
-            def land(bar=bar):
+            def land(bar=bar, it=it):
+                self.copying[it % S] = False
                 bar.tx -= 1
                 bar.turn()
             self.queue(land)
             yield None
-        it = self.n
-        for k in range(it, it + 3):
-            if k >= S:
-                yield wait(self.empty[k % S], k // S - 1)
-        for k in range(it, it + 3):
-            self.put(k, -1 - (k - it))
-        self.listed[it % S].arrive()
-        self.listed[(it + 1) % S].arrive()
-        yield None
-        for k in range(max(0, it - 5), it):
-            yield wait(self.listed[k % S], k // S)
+            it += 1
+        if it == self.n:
+            for k in range(it, it + 3):
+                if k >= S:
+                    ok = ok and (yield self.empty[k % S], k // S - 1)
+            if ok or not self.leaves:
+                for k in range(it, it + 3):
+                    self.put(k, -1 - (k - it))
+                self.listed[it % S].arrive()
+                self.listed[(it + 1) % S].arrive()
+                yield None
+        for k in range(max(0, it - (5 if ok else 8)), it):
+            ok = (yield self.listed[k % S], k // S) and ok
 
     def generator(self, g, w):
-        S, it = self.SLOTS, g
+        S, it, ok = self.SLOTS, g, True
         while True:
-            yield wait(self.listed[it % S], it // S)
+            ok = ok and (yield self.listed[it % S], it // S)
             if it >= 3 and self.x_wait:
-                yield wait(self.full[(it - 3) % self.nf], (it - 3) // self.nf)
-            end = self.record(it)
+                ok = ok and (yield self.full[(it - 3) % self.nf], (it - 3) // self.nf)
+            end = self.record(it) if ok else -4
             if end == 0:
                 c, s, used, _ = self.steps[it]
-                check(it < self.BUFS or self.done[it - self.BUFS], f"X of step {it - 3} overwritten early")
+                self.see(it < self.BUFS or self.done[it - self.BUFS], f"X of step {it - 3} overwritten early")
                 if s == 0:
                     several = self.w_wait and used >= 0 and self.steps[used][1] > 0
                     if used >= 0 and it - used < 8 and (it - used > 3 or several):
-                        yield wait(self.empty[used % S], used // S)
-                    check(used < 0 or all(self.done[k] for k in range(used + 1) if self.steps[k][0] == c - self.BUFS),
-                          f"W of chunk {c - self.BUFS} overwritten early")
+                        ok = ok and (yield self.empty[used % S], used // S)
+                    self.see(used < 0 or all(self.done[k] for k in range(used + 1) if self.steps[k][0] == c - self.BUFS),
+                             f"W of chunk {c - self.BUFS} overwritten early")
                 self.wrote[it] += 1
                 yield None
-            gen = self.meet[g].arrive()
-            yield lambda: self.meet[g].gen >= gen
-            if w == 0:
+            elif not ok and it < self.n:
+                self.wrote[it] += 1          # past it, without a look at its record
+            meet = self.meet[g]
+            gen = meet.arrive(end < 0)
+            yield lambda: meet.met(gen)
+            if w == 0 and ok:
                 self.ready[it % S].arrive()
                 if end == -1:
                     self.ready[(it + 2) % S].arrive()
-            if end < 0:
+            if meet.stop[gen]:
                 return
             it += 2
 
     def issuer(self, k):
-        S, it, behind = self.SLOTS, k, None
+        S, it, behind, ok = self.SLOTS, k, None, True
         while True:
-            yield wait(self.ready[it % S], it // S)
-            if self.record(it) < 0:
+            ok = yield self.ready[it % S], it // S
+            if not ok or self.record(it) < 0:
                 break
             c, s, _, _ = self.steps[it]
             if 1 <= s <= 3:
-                yield wait(self.ready[(it - s) % S], (it - s) // S)
+                ok = ok and (yield self.ready[(it - s) % S], (it - s) // S)
             if it >= self.DBUFS:
-                yield wait(self.empty[(it - self.DBUFS) % S], (it - self.DBUFS) // S)
-                check(self.read[it - self.DBUFS] == 8, f"sums of step {it - self.DBUFS} overwritten early")
-            check(self.wrote[it] == 8 and self.wrote[it - s] == 8, f"MMAs of step {it} before its operands")
+                ok = ok and (yield self.empty[(it - self.DBUFS) % S], (it - self.DBUFS) // S)
+            if not ok:
+                break
+            self.see(it < self.DBUFS or self.read[it - self.DBUFS] == 8, f"sums of step {it - self.DBUFS} overwritten early")
+            self.see(self.wrote[it] == 8 and self.wrote[it - s] == 8, f"MMAs of step {it} before its operands")
             self.issued[it] = True
 
             def land(it=it):
@@ -239,13 +291,14 @@ class Adjoint(Model):
             yield None
             it += 3
         if it >= 3:
-            yield wait(self.full[(it - 3) % self.nf], (it - 3) // self.nf)
+            yield self.full[(it - 3) % self.nf], (it - 3) // self.nf
 
     def adder(self, w):
         meets = 0
         for it in range(self.n):
-            yield wait(self.full[it % self.nf], it // self.nf)
-            check(self.done[it], f"sums of step {it} read before they are complete")
+            if not (yield self.full[it % self.nf], it // self.nf):
+                return
+            self.see(self.done[it], f"sums of step {it} read before they are complete")
             self.record(it)
             yield None
             self.read[it] += 1
@@ -253,22 +306,23 @@ class Adjoint(Model):
             if self.steps[it][3]:
                 for _ in range(2 if it + 1 < self.n else 1):
                     self.summed.arrive()
-                    yield wait(self.summed, meets)
+                    if not (yield self.summed, meets):
+                        return
                     meets += 1
 
 
 class Forward(Model):
     """One CTA: steps of the given tiles (a number per step)."""
 
-    def __init__(self, rng, tiles):
-        super().__init__(rng)
-        self.tiles = tiles
+    def __init__(self, rng, tiles, leaves=FWD_LEAVES, fails=False):
+        super().__init__(rng, fails)
+        self.tiles, self.leaves = tiles, leaves
         n = self.n = len(tiles)
         self.full = [Barrier(1) for _ in range(2)]
         self.empty = [Barrier(8) for _ in range(4)]
         self.ready = [Barrier(1) for _ in range(4)]
         self.listed = [Barrier(1) for _ in range(4)]
-        self.slot = [None] * 4
+        self.slot, self.copying = [None] * 4, [False] * 4
         self.wrote, self.read = [0] * n, [0] * n
         self.issued, self.done = [False] * n, [False] * n
         self.meets = [Meeting(8) for _ in range(2)]
@@ -282,6 +336,7 @@ class Forward(Model):
     def put(self, it, end):
         if 0 <= it - 4 < self.n:
             check(self.read[it - 4] == 8 and self.wrote[it - 4] == 8 and self.issued[it - 4], f"record of step {it - 4} rewritten early")
+        check(not self.copying[it & 3], "a copy goes to a slot whose last copy is in flight")
         self.slot[it & 3] = (it, end)
 
     def record(self, it):
@@ -289,62 +344,76 @@ class Forward(Model):
         return self.slot[it & 3][1]
 
     def lister(self):
-        for it in range(self.n):
+        ok, it = True, 0
+        while it < self.n:
             if it >= 4:
-                yield wait(self.empty[it & 3], (it >> 2) - 1)
+                ok = ok and (yield self.empty[it & 3], (it >> 2) - 1)
+            if not ok and self.leaves:
+                break
             self.put(it, False)
             bar = self.listed[it & 3]
             bar.tx += 1
+            self.copying[it & 3] = True
             bar.arrive()
 
-            def land(bar=bar):
+            def land(bar=bar, it=it):
+                self.copying[it & 3] = False
                 bar.tx -= 1
                 bar.turn()
             self.queue(land)
             yield None
-        for k in (self.n, self.n + 1):
-            if k >= 4:
-                yield wait(self.empty[k & 3], (k >> 2) - 1)
-            self.put(k, True)
-            self.listed[k & 3].arrive()
-        yield None
-        for k in range(max(0, self.n - 2), self.n):
-            yield wait(self.listed[k & 3], k >> 2)
+            it += 1
+        if it == self.n:
+            for k in (it, it + 1):
+                if k >= 4:
+                    ok = ok and (yield self.empty[k & 3], (k >> 2) - 1)
+            if ok or not self.leaves:
+                for k in (it, it + 1):
+                    self.put(k, True)
+                    self.listed[k & 3].arrive()
+                yield None
+        for k in range(max(0, it - (2 if ok else 4)), it):
+            ok = (yield self.listed[k & 3], k >> 2) and ok
 
     def generator(self, w):
-        it = 0
+        it, ok = 0, True
         while True:
-            yield wait(self.listed[it & 3], it >> 2)
+            ok = ok and (yield self.listed[it & 3], it >> 2)
             if it >= 2:
-                yield wait(self.full[it & 1], (it >> 1) - 1)
-            gen = self.meets[0].arrive()
-            yield lambda: self.meets[0].gen >= gen
+                ok = ok and (yield self.full[it & 1], (it >> 1) - 1)
+            first, second = self.meets
+            gen = first.arrive(not ok)
+            yield lambda: first.met(gen)
+            if first.stop[gen]:
+                return
             if self.record(it):
                 if w == 0:
                     self.ready[it & 3].arrive()
                 return
-            check(it < 2 or self.done[it - 2], f"A of step {it - 2} overwritten early")
+            self.see(it < 2 or self.done[it - 2], f"A of step {it - 2} overwritten early")
             if it == 0 or self.tiles[it] != self.tiles[it - 1]:
                 old = [k for k in range(it) if self.tiles[k] < self.tiles[it] - 1]
-                check(all(self.done[k] for k in old), "B of an older tile overwritten early")
+                self.see(all(self.done[k] for k in old), "B of an older tile overwritten early")
             self.wrote[it] += 1
-            gen = self.meets[1].arrive()
-            yield lambda: self.meets[1].gen >= gen
+            gen = second.arrive()
+            yield lambda: second.met(gen)
             if w == 0:
                 self.ready[it & 3].arrive()
             it += 1
 
     def issuer(self, d):
-        it, behind = d, None
+        it, behind, ok = d, None, True
         while True:
-            yield wait(self.listed[it & 3], it >> 2)
-            if self.record(it):
+            ok = yield self.listed[it & 3], it >> 2
+            if not ok or self.record(it):
                 break
-            yield wait(self.ready[it & 3], it >> 2)
+            ok = yield self.ready[it & 3], it >> 2
             if it >= 2:
-                yield wait(self.empty[(it - 2) & 3], (it - 2) >> 2)
-                check(self.read[it - 2] == 8, f"sums of step {it - 2} overwritten early")
-            check(self.wrote[it] == 8, f"MMAs of step {it} before its operands")
+                ok = ok and (yield self.empty[(it - 2) & 3], (it - 2) >> 2)
+            if not ok:
+                break
+            self.see(it < 2 or self.read[it - 2] == 8, f"sums of step {it - 2} overwritten early")
+            self.see(self.wrote[it] == 8, f"MMAs of step {it} before its operands")
             self.issued[it] = True
 
             def land(it=it):
@@ -354,15 +423,15 @@ class Forward(Model):
             yield None
             it += 2
         if it >= 2:
-            yield wait(self.full[d], (it - 2) >> 1)
+            yield self.full[d], (it - 2) >> 1
 
     def summer(self, w):
         for it in range(self.n + 1):
-            yield wait(self.ready[it & 3], it >> 2)
-            if self.record(it):
+            if not (yield self.ready[it & 3], it >> 2) or self.record(it):
                 return
-            yield wait(self.full[it & 1], it >> 1)
-            check(self.done[it], f"sums of step {it} read before they are complete")
+            if not (yield self.full[it & 1], it >> 1):
+                return
+            self.see(self.done[it], f"sums of step {it} read before they are complete")
             yield None
             self.read[it] += 1
             self.empty[it & 3].arrive()
@@ -379,13 +448,24 @@ def test_adjoint_roles(seed):
     Adjoint(rng, *schedule(rng)).play()
 
 
-@pytest.mark.parametrize("seed", range(40))
-def test_forward_roles(seed):
-    rng = random.Random(seed)
+def tiles_of(rng):
     tiles = [0]
     for _ in range(rng.randint(0, 24)):
         tiles.append(tiles[-1] + (rng.random() < 0.5))
-    Forward(rng, tiles).play()
+    return tiles
+
+
+@pytest.mark.parametrize("seed", range(40))
+def test_forward_roles(seed):
+    rng = random.Random(seed)
+    Forward(rng, tiles_of(rng)).play()
+
+
+@pytest.mark.parametrize("seed", range(60))
+def test_every_role_ends_after_a_wait_that_ran_out(seed):
+    rng = random.Random(seed)
+    Adjoint(rng, *schedule(rng), fails=True).play()
+    Forward(rng, tiles_of(rng), fails=True).play()
 
 
 def caught(make):
@@ -401,6 +481,8 @@ def caught(make):
 def test_planted_mistakes_are_caught():
     assert caught(lambda r: Adjoint(r, *schedule(r), nfull=4))
     assert caught(lambda r: Adjoint(r, *schedule(r), x_wait=False))
+    assert caught(lambda r: Adjoint(r, *schedule(r), fails=True, leaves=False))
+    assert caught(lambda r: Forward(r, tiles_of(r), fails=True, leaves=False))
 
 
 # A chunk of two strips, then chunks of one: W's buffer is free again three
