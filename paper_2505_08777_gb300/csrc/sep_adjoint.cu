@@ -126,13 +126,15 @@ __global__ void __launch_bounds__(kAdjThreads, 1) k_sep_adjoint(const SepAdjPara
     const int pl = w & 3, hc = w >> 2;
     const uint32_t ta = tmem + ((uint32_t)(pl * 32) << 16) + 32u * hc;
     float2* sums = reinterpret_cast<float2*>(sm + kAdjSum);
-    // (an mbarrier, not a named one: a warp whose wait runs out leaves alone)
+    // (an mbarrier, not a named one: a warp whose wait runs out leaves alone, and
+    // so do then the others, before they read what it has not written)
     uint32_t meets = 0;
-    auto add_sync = [&]() {
+    auto add_sync = [&]() -> bool {
       __syncwarp();
       if (lane == 0) mbar_arrive(summed);
       ok = ok && sep_wait(summed, meets & 1);
       ++meets;
+      return ok = __all_sync(0xffffffffu, ok);
     };
     float2 acc[16];
 #pragma unroll
@@ -172,7 +174,7 @@ __global__ void __launch_bounds__(kAdjThreads, 1) k_sep_adjoint(const SepAdjPara
         mine[i] = mul2(acc[i], dup2(c));
         acc[i] = make_float2(0.0f, 0.0f);
       }
-      add_sync();
+      if (!add_sync()) break;
       const TcAdjParams& o = p.a;
       const Geometry& g = o.g;
       const int tx = x.tile % g.tiles_x, ty = x.tile / g.tiles_x;
@@ -191,7 +193,7 @@ __global__ void __launch_bounds__(kAdjThreads, 1) k_sep_adjoint(const SepAdjPara
 #pragma unroll
         for (int q = 0; q < 4; ++q) dst[q * 256] = v[q];
         __threadfence();
-        add_sync();
+        if (!add_sync()) break;
         int* flag = reinterpret_cast<int*>(slot + 1);   // [2]: the tile's first CTA if this is the last to come, its last CTA
         if (t == 0) {
           const int u0 = x.tile * nb, u1 = u0 + nb;
@@ -201,7 +203,7 @@ __global__ void __launch_bounds__(kAdjThreads, 1) k_sep_adjoint(const SepAdjPara
           flag[0] = last ? g_lo : -1;
           flag[1] = g_hi;
         }
-        add_sync();
+        if (!add_sync()) break;
         const int g_lo = flag[0], g_hi = flag[1];
         out = g_lo >= 0;
         if (out) {
@@ -241,7 +243,7 @@ __global__ void __launch_bounds__(kAdjThreads, 1) k_sep_adjoint(const SepAdjPara
         }
       }
       if (x.end() & 8) break;
-      add_sync();   // `sums` is rewritten at the next tile's end
+      if (!add_sync()) break;   // `sums` is rewritten at the next tile's end
     }
   } else if (w < 12) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");

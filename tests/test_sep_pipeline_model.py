@@ -17,10 +17,10 @@ others in turn where they depend on it: every role has to end, no copy may go
 to a slot that is still in use, and no copy or MMA may be in flight when the
 last role ends, for the memory belongs to the next block then.
 
-The numbers of barriers and what the listers do after a wait that ran out are
-read from the sources. Mistakes planted in the model (four barriers for the
+The numbers of barriers and what listers and adders do after a wait that ran
+out are read from the sources. Mistakes planted in the model (four barriers for the
 adjoint's MMAs, which the generators' wait can find two phases on; an operand
-buffer taken back early; listers that run on) have to be caught.
+buffer taken back early; listers and adders that run on) have to be caught.
 """
 import pathlib
 import random
@@ -43,6 +43,9 @@ def lister_leaves(file):
 
 
 ADJ_FULL = constant("kAdjFull", "sep_adjoint.cu")
+# meetings of the adjoint's adders: all of them are left if the wait ran out
+ADDERS = (CSRC / "sep_adjoint.cu").read_text()
+ADDERS_LEAVE = ADDERS.count("if (!add_sync()) break;") == len(re.findall(r"\badd_sync\(\)", ADDERS))
 ADJ_LEAVES, FWD_LEAVES = lister_leaves("sep_adjoint.cu"), lister_leaves("sep_forward.cu")
 
 
@@ -160,9 +163,11 @@ class Adjoint(Model):
 
     SLOTS, BUFS, DBUFS = 8, 3, 4
 
-    def __init__(self, rng, chunks, ends, nfull=ADJ_FULL, x_wait=True, w_wait=True, leaves=ADJ_LEAVES, fails=False):
+    def __init__(self, rng, chunks, ends, nfull=ADJ_FULL, x_wait=True, w_wait=True, leaves=ADJ_LEAVES,
+                 adders_leave=ADDERS_LEAVE, fails=False):
         super().__init__(rng, fails)
         self.nf, self.x_wait, self.w_wait, self.leaves = nfull, x_wait, w_wait, leaves
+        self.adders_leave, self.sums, self.flag = adders_leave, [0] * 8, -1
         self.steps = []                      # (chunk, strip, last step that used W's buffer, tile end)
         last = []
         for c, ls in enumerate(chunks):
@@ -303,12 +308,24 @@ class Adjoint(Model):
             yield None
             self.read[it] += 1
             self.empty[it % self.SLOTS].arrive()
-            if self.steps[it][3]:
-                for _ in range(2 if it + 1 < self.n else 1):
-                    self.summed.arrive()
-                    if not (yield self.summed, meets):
-                        return
-                    meets += 1
+            if not self.steps[it][3]:
+                continue
+            # the end of a tile split between CTAs: planes summed, partial sums
+            # stored, the tile's CTAs counted by thread 0, their sums read
+            self.sums[w] = it
+            for what in ("planes", "partial sums", "flag", "done")[: 4 if it + 1 < self.n else 3]:
+                if what == "flag" and w == 0:
+                    self.flag = it
+                self.summed.arrive()
+                ok = yield self.summed, meets
+                meets += 1
+                if not ok and self.adders_leave:
+                    return
+                if what == "planes":
+                    check(all(x == it for x in self.sums), "another warp's sums read before they are written")
+                if what == "flag":
+                    check(self.flag == it, "the tile's CTAs read before thread 0 has counted them")
+                yield None
 
 
 class Forward(Model):
@@ -483,6 +500,7 @@ def test_planted_mistakes_are_caught():
     assert caught(lambda r: Adjoint(r, *schedule(r), x_wait=False))
     assert caught(lambda r: Adjoint(r, *schedule(r), fails=True, leaves=False))
     assert caught(lambda r: Forward(r, tiles_of(r), fails=True, leaves=False))
+    assert caught(lambda r: Adjoint(r, *schedule(r), fails=True, adders_leave=False))
 
 
 # A chunk of two strips, then chunks of one: W's buffer is free again three
