@@ -318,6 +318,13 @@ cudaError_t enqueue_tc_gradc(ash_hologram* h, const float* phase, const float2* 
 // tc-layout nearfield the previous tensor-core adjoint wrote (kEpiFimg).
 constexpr int kSrcImg = kSrcImage;
 
+cudaError_t capturing(cudaStream_t s, bool* captured) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  const cudaError_t e = cudaStreamIsCapturing(s, &cap);
+  *captured = cap != cudaStreamCaptureStatusNone;
+  return e;
+}
+
 cudaError_t enqueue_tc_coeff(ash_hologram* h, cudaStream_t s) {
   if (!h->tc_ok) return cudaSuccess;
   if (h->sep_ok) {
@@ -325,9 +332,16 @@ cudaError_t enqueue_tc_coeff(ash_hologram* h, cudaStream_t s) {
                                            h->sep_acost, s);
     if (e != cudaSuccess) return e;
   }
-  // the other tensor-core kernels' images only where one of them is in use
-  h->tc_stale = !needs_tc_images(h);
-  if (h->tc_stale) return cudaSuccess;
+  // The other tensor-core kernels' images only where one of them is in use. Not
+  // left out of a captured call: its replays change the coefficients unseen, so
+  // they keep the images up to date, and the flag speaks of the other calls.
+  bool captured = false;
+  const cudaError_t e = capturing(s, &captured);
+  if (e != cudaSuccess) return e;
+  if (!captured) {
+    h->tc_stale = !needs_tc_images(h);
+    if (h->tc_stale) return cudaSuccess;
+  }
   return tc_build_coeff(h->g, h->tc_layout, h->coeff, h->anchors, h->czs, h->rot, s);
 }
 
@@ -422,6 +436,10 @@ cudaError_t launch_gradc(int D, const GradCParams& p, dim3 grid, cudaStream_t s)
 ash_status enqueue_forward(ash_hologram* h, int source, const float* phase, const float2* field, float2* E,
                            cudaStream_t s, bool loop = false) {
   const bool sep = use_sep_fwd(h, loop);
+  if (!sep) {
+    const ash_status st = fresh_tc_images(h, s);
+    if (st != ASH_OK) return st;
+  }
   if (sep || use_tc_fwd(h)) {
     cudaError_t e = cudaSuccess;
     if (source != kSrcImg) {
@@ -475,6 +493,8 @@ ash_status enqueue_adjoint(ash_hologram* h, const float2* y, float2* g_out, floa
     if (e == cudaSuccess) e = sep_launch_adjoint(sep_adj_params(h, y, p.out), s);
     return e == cudaSuccess ? ASH_OK : cuda_fail(e, "separable adjoint launch");
   }
+  const ash_status st = fresh_tc_images(h, s);
+  if (st != ASH_OK) return st;
   if (use_tc_adj(h)) {
     const TcAdjParams tp = tc_adj_params(h, y, p.out);
     cudaError_t e = tc_launch_adjoint(h->tc_na, tp, h->tadj.G, s);
@@ -550,12 +570,14 @@ ash_status ensure_fma_image(ash_hologram* h) {
   return ASH_OK;
 }
 
-ash_status ensure_tc_images(ash_hologram* h) {
-  if (!h->tc_ok || !h->tc_stale) return ASH_OK;
-  ASH_CUDA(cudaDeviceSynchronize());
-  ASH_CUDA(tc_build_coeff(h->g, h->tc_layout, h->coeff, h->anchors, h->czs, h->rot, h->home));
-  ASH_CUDA(cudaStreamSynchronize(h->home));
-  h->tc_stale = false;
+
+ash_status fresh_tc_images(ash_hologram* h, cudaStream_t s) {
+  // (a loop's own graph finds them rebuilt on the caller's stream)
+  if (!h->tc_stale || !needs_tc_images(h) || s == h->capture) return ASH_OK;
+  ASH_CUDA(tc_build_coeff(h->g, h->tc_layout, h->coeff, h->anchors, h->czs, h->rot, s));
+  bool captured = false;
+  ASH_CUDA(capturing(s, &captured));
+  if (!captured) h->tc_stale = false;
   return ASH_OK;
 }
 
@@ -1276,7 +1298,9 @@ ash_status ash_wgs_iterate(ash_hologram* h, float* phase, float* w, const float*
   ASH_CUDA(cudaMemcpyAsync(h->wgs_T, target, N * 4, cudaMemcpyDeviceToDevice, s));
   if (iters >= 2) {
     cudaGraphExec_t exec = nullptr;
-    ash_status st = cached_graph(h, iters, enqueue_wgs_body, iters, &exec);
+    ash_status st = fresh_tc_images(h, s);   // not in the loop's graph
+    if (st != ASH_OK) return st;
+    st = cached_graph(h, iters, enqueue_wgs_body, iters, &exec);
     if (st != ASH_OK) return st;
     ASH_CUDA(cudaGraphLaunch(exec, s));
   } else {
@@ -1308,6 +1332,8 @@ ash_status ash_grad(ash_hologram* h, const float* phase, const float* grad_E, fl
     ASH_CUDA(sep_launch_gradc(sp, s));
     ASH_CUDA(sep_launch_gradc_reduce(sp, s));
   } else if (dcoeff && use_tc_grad(h)) {
+    const ash_status st = fresh_tc_images(h, s);
+    if (st != ASH_OK) return st;
     ASH_CUDA(enqueue_tc_gradc(h, phase, gE, dcoeff, s));
   } else if (dcoeff) {
     if (!h->dz) return set_error(ASH_ERR_DEVICE, "FMA-pipe moments without their basis image");
@@ -1344,11 +1370,10 @@ ash_status ash_set_kernel_variant(ash_hologram* h, int variant) {
   if (variant == 2 && !h->tc_ok)
     return set_error(ASH_ERR_UNSUPPORTED, "tensor-core kernels need D <= %d (D = %d)", kTcMaxModes, h->g.D);
   h->variant = variant;
+  // a caller's graph captured in this variant reads the images whenever it is
+  // replayed, in any variant
+  if (variant == 2) h->tc_pinned = true;
   clear_graphs(h);
-  if (needs_tc_images(h)) {
-    const ash_status st = ensure_tc_images(h);
-    if (st != ASH_OK) return st;
-  }
   if (needs_fma_image(h)) return ensure_fma_image(h);
   return ASH_OK;
 }
@@ -1387,10 +1412,11 @@ ash_status ash_profile(ash_hologram* h, const float* phase, const float* y, floa
   if (injected_failure()) return set_error(ASH_ERR_INJECTED, "injected failure");
   cudaStream_t s = as_stream(stream);
   if (needs_fma_image(h) && !h->dz) return set_error(ASH_ERR_DEVICE, "FMA-pipe kernels without their basis image");
+  ash_status st = fresh_tc_images(h, s);
+  if (st != ASH_OK) return st;
   cudaEvent_t ev[12];
   for (int q = 0; q < 12; ++q) ASH_CUDA(cudaEventCreate(&ev[q]));
   const float2* y2 = reinterpret_cast<const float2*>(y);
-  ash_status st = ASH_OK;
   cudaError_t e = cudaSuccess;
   // forward kernel, then its reduction
   FwdParams fp{};

@@ -596,8 +596,10 @@ ash_status build_group(ash_batch* b, long long solo_terms, cudaStream_t s) {
     // the persistent kernels read the register-image basis or the
     // tensor-core spot images
     h->tc_pinned = true;
-    ash_status st = ensure_tc_images(h);
+    const bool stale = h->tc_stale;
+    ash_status st = fresh_tc_images(h, s);
     if (st != ASH_OK) return st;
+    if (stale) BCUDA(cudaStreamSynchronize(s));   // the loop may run on another stream
     st = ensure_fma_image(h);
     if (st != ASH_OK) return st;
     BatchHolo bh{};
@@ -713,8 +715,12 @@ std::string tune_key(const ash_batch* b) {
 
 // The batch's WGS loop for `iters` iterations (standalone members' loops
 // and the persistent group's launches) captured and instantiated.
-ash_status capture_loop(ash_batch* b, int iters, cudaGraphExec_t* exec, int* kernels) {
+ash_status capture_loop(ash_batch* b, int iters, cudaGraphExec_t* exec, int* kernels, cudaStream_t s) {
   cudaGraph_t graph = nullptr;
+  for (ash_hologram* h : b->solo) {   // not in the loop's graph
+    const ash_status st = fresh_tc_images(h, s);
+    if (st != ASH_OK) return st;
+  }
   BCUDA(cudaStreamBeginCapture(b->capture, cudaStreamCaptureModeThreadLocal));
   ash_status st = ASH_OK;
   const int lanes = (int)std::min<size_t>(b->solo.size(), kBatchLanes);
@@ -969,7 +975,7 @@ ash_status ash_batch_wgs(ash_batch* b, float* const* phases, float* const* weigh
     exec = it->second;
   } else {
     int kernels = 0;
-    ash_status st = capture_loop(b, iters, &exec, &kernels);
+    ash_status st = capture_loop(b, iters, &exec, &kernels, s);
     if (st != ASH_OK) return st;
     b->graphs[iters] = exec;
     b->graph_kernels[iters] = kernels;
@@ -1091,7 +1097,7 @@ ash_status ash_batch_tune(ash_batch* b, const float* const* phases, const char* 
       }
       // the whole loop of this choice, as the graph ash_batch_wgs runs
       cudaGraphExec_t exec = nullptr;
-      if ((st = capture_loop(b, kTimedIters, &exec, nullptr)) != ASH_OK) break;
+      if ((st = capture_loop(b, kTimedIters, &exec, nullptr, s)) != ASH_OK) break;
       float ms = 0.0f;
       st = elapsed(
           [&]() -> ash_status {

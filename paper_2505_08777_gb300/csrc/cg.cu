@@ -236,7 +236,9 @@ ash_status ash_cg_refine(ash_hologram* h, float* phase, const float* t, int iter
   ASH_CUDA(cudaMemcpyAsync(h->cg_scal, init, sizeof init, cudaMemcpyHostToDevice, s));
   if (iters >= 1) {
     cudaGraphExec_t exec = nullptr;
-    ash_status st = cached_graph(h, -iters, enqueue_cg_body, iters, &exec);
+    ash_status st = fresh_tc_images(h, s);   // not in the loop's graph
+    if (st != ASH_OK) return st;
+    st = cached_graph(h, -iters, enqueue_cg_body, iters, &exec);
     if (st != ASH_OK) return st;
     ASH_CUDA(cudaGraphLaunch(exec, s));
   } else {

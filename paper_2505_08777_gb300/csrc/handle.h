@@ -42,7 +42,7 @@ struct ash_hologram {
   ash::TcFwdSched tfwd{};       // forward units (spot block, pixel chunk)
   bool tfwd_split = false;      // some spot block's pixels span two CTA ranges
   bool tc_stale = false;        // czs and rot are older than the coefficients (no kernel in use reads them)
-  bool tc_pinned = false;       // a batch's persistent kernels read them
+  bool tc_pinned = false;       // a batch's persistent kernels or a caller's graph of variant 2 may read them
   float* zs = nullptr;
   float* czs = nullptr;
   float4* fimg = nullptr;
@@ -133,9 +133,9 @@ int graph_kernel_nodes(cudaGraph_t g);
 // The FMA-pipe kernels' register-image basis: rebuilt from the monomial
 // tables if it was released (synchronises the device).
 ash_status ensure_fma_image(ash_hologram* h);
-// The tensor-core spot images (czs, rot), if they are older than the
-// coefficients (synchronises the device).
-ash_status ensure_tc_images(ash_hologram* h);
+// The tensor-core spot images (czs, rot), rebuilt on `s` if the kernels in use
+// read them and they are older than the coefficients.
+ash_status fresh_tc_images(ash_hologram* h, cudaStream_t s);
 // Record a message for ash_last_error() (any translation unit).
 void record_error(const char* msg);
 // Map a CUDA error to ASH_ERR_CUDA with a message.
