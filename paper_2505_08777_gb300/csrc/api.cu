@@ -325,13 +325,16 @@ cudaError_t capturing(cudaStream_t s, bool* captured) {
   return e;
 }
 
-cudaError_t enqueue_tc_coeff(ash_hologram* h, cudaStream_t s) {
+// The coefficients' images. forward_only: nothing but a forward reads them
+// before the next call of this.
+cudaError_t enqueue_tc_coeff(ash_hologram* h, cudaStream_t s, bool forward_only = false) {
   if (!h->tc_ok) return cudaSuccess;
   if (h->sep_ok) {
     const cudaError_t e = sep_build_params(h->g, h->sep_tab, h->coeff, h->sep_poly, h->sep_strips, h->sep_cost,
                                            h->sep_acost, s);
     if (e != cudaSuccess) return e;
   }
+  if (forward_only && use_sep_fwd(h)) return cudaSuccess;
   // The other tensor-core kernels' images only where one of them is in use. Not
   // left out of a captured call: its replays change the coefficients unseen, so
   // they keep the images up to date, and the flag speaks of the other calls.
@@ -643,7 +646,9 @@ ash_status adjoint_enqueue(ash_hologram* h, const float2* y, float2* g_out, floa
                            float* dphase, int epilogue, cudaStream_t s) {
   return enqueue_adjoint(h, y, g_out, phase_out, phase_in, dphase, epilogue, s);
 }
-cudaError_t coeff_images_enqueue(ash_hologram* h, cudaStream_t s) { return enqueue_tc_coeff(h, s); }
+cudaError_t coeff_images_enqueue(ash_hologram* h, cudaStream_t s, bool forward_only) {
+  return enqueue_tc_coeff(h, s, forward_only);
+}
 bool forward_reads_image(const ash_hologram* h) { return use_sep_fwd(h) || use_tc_fwd(h); }
 }  // namespace ash
 

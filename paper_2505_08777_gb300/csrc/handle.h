@@ -153,7 +153,8 @@ ash_status forward_enqueue(ash_hologram* h, int source, const float* phase, cons
                            cudaStream_t s);
 ash_status adjoint_enqueue(ash_hologram* h, const float2* y, float2* g_out, float* phase_out, const float* phase_in,
                            float* dphase, int epilogue, cudaStream_t s);
-cudaError_t coeff_images_enqueue(ash_hologram* h, cudaStream_t s);
+// forward_only: nothing but a forward reads the images before the next call.
+cudaError_t coeff_images_enqueue(ash_hologram* h, cudaStream_t s, bool forward_only = false);
 // A forward from the nearfield image that the last forward from a phase or a
 // field (or a fused adjoint) left in the handle, where the forward reads one.
 constexpr int kSrcImage = 2;

@@ -103,7 +103,11 @@ ash_status ash_zsub_sweep(ash_hologram* h, const float* phase, int mode, const f
   for (int k = 0; k < K && st == ASH_OK; ++k) {
     k_zsub_shift<<<blocks, 256, 0, s>>>(h->coeff_bak, h->coeff, N, D, mode, deltas[k]);
     cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess) e = coeff_images_enqueue(h, s);
+    // (what the adjoint and the moments read is built with the restored
+    // coefficients: per offset it cost more than a separable forward saves; seven
+    // offsets of 880 x 890 N = 8 549 / 319 us, 400^2 N = 64 556 / 311, before the
+    // separable forward 531 / 501)
+    if (e == cudaSuccess) e = coeff_images_enqueue(h, s, true);
     if (e != cudaSuccess) {
       st = cuda_fail(e, "calibration sweep");
       break;

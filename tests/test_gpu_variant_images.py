@@ -109,3 +109,25 @@ def test_variant_change_inside_a_capture(setup):
     h.set_coefficients(Cs[1])
     graph.replay()
     assert torch.equal(E, _want(amp, ph, Cs[1]))
+
+
+def test_images_reach_the_calls_that_read_them():
+    # a separable forward beside a tensor-core adjoint, moment pass and loop
+    p = random_problem(78, 470, 450, 300, NOLL)
+    ph, amp = torch.from_numpy(p.phase0).cuda(), torch.from_numpy(p.amp).cuda()
+    C1 = torch.from_numpy((p.coeff * np.float32(0.5)).astype(np.float32)).cuda()
+    y = torch.polar(torch.ones(p.N), torch.arange(p.N, dtype=torch.float32)).cuda()
+    t = torch.ones(p.N, device="cuda")
+    fresh = _holo(amp, C1)
+
+    def loop(h):
+        x, w = ph.clone(), t.clone()
+        h.wgs(x, w, t, 2)
+        assert h.graph_kernels(2) == h.wgs_launches(2)
+        return x
+    calls = [lambda h: h.adjoint(y)[0], lambda h: h.grad(ph, y)[1], loop,
+             lambda h: (h.zsub_sweep(ph, 1, [0.5]), h.adjoint(y)[0])[1]]
+    for call in calls:
+        h = _holo(amp, torch.from_numpy(p.coeff).cuda())
+        h.forward_coeff(C1, ph)
+        assert torch.equal(call(h), call(fresh))
