@@ -338,13 +338,14 @@ cudaError_t enqueue_tc_coeff(ash_hologram* h, cudaStream_t s, bool forward_only 
   // The other tensor-core kernels' images only where one of them is in use. Not
   // left out of a captured call: its replays change the coefficients unseen, so
   // they keep the images up to date, and the flag speaks of the other calls.
+  const bool needed = needs_tc_images(h);
   bool captured = false;
-  const cudaError_t e = capturing(s, &captured);
-  if (e != cudaSuccess) return e;
-  if (!captured) {
-    h->tc_stale = !needs_tc_images(h);
-    if (h->tc_stale) return cudaSuccess;
+  if (!needed || h->tc_stale) {
+    const cudaError_t e = capturing(s, &captured);
+    if (e != cudaSuccess) return e;
   }
+  if (!captured) h->tc_stale = !needed;
+  if (!captured && !needed) return cudaSuccess;
   return tc_build_coeff(h->g, h->tc_layout, h->coeff, h->anchors, h->czs, h->rot, s);
 }
 

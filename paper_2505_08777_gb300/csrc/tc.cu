@@ -175,12 +175,9 @@ cudaError_t tc_build_zs(const Geometry& g, const TcLayout& L, const float* dz, f
 cudaError_t tc_build_coeff(const Geometry& g, const TcLayout& L, const float* coeff, const float2* anchors, float* czs,
                            float2* rot, cudaStream_t s) {
   const int nc64 = tc_spot_chunks(g.N);
-  k_tc_build_czs<<<blocks_for((long long)(nc64 + 2) * kTcChunk, 256), 256, 0, s>>>(coeff, g.N, L, nc64,
-                                                                                 tc_fwd_rep(g.N), czs);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  const long long nr = (long long)g.N * g.T;
-  k_tile_rotations<<<blocks_for(nr, 256), 256, 0, s>>>(coeff, anchors, g.N, g.D, g.T, rot);
+  const unsigned nczs = blocks_for((long long)(nc64 + 2) * kTcChunk, 256), nrot = blocks_for((long long)g.N * g.T, 256);
+  k_tc_build_coeff<<<nczs + nrot, 256, 0, s>>>(coeff, g.N, L, nc64, tc_fwd_rep(g.N), czs, (int)nczs, anchors, g.D, g.T,
+                                               rot);
   return cudaGetLastError();
 }
 

@@ -107,9 +107,8 @@ static __global__ void k_tc_build_zs(const Geometry G, const TcLayout L, const f
 // The two chunks after the nc64 main ones hold the last 128-spot block with
 // its first 128 / rep spots repeated rep times.
 constexpr double kInv2PiD = 0.15915494309189533576888376337251;
-static __global__ void k_tc_build_czs(const float* __restrict__ coeff, int N, const TcLayout L, int nc64, int rep,
-                                      float* __restrict__ czs) {
-  const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+__device__ __forceinline__ void build_czs(long long e, const float* __restrict__ coeff, int N, const TcLayout& L,
+                                          int nc64, int rep, float* __restrict__ czs) {
   if (e >= (long long)(nc64 + 2) * kTcChunk) return;
   const int jc = (int)(e / kTcChunk), r = (int)(e % kTcChunk), D = L.D;
   int n = jc * kTcChunk + r;
@@ -180,9 +179,9 @@ static __global__ void k_tc_field_img(const Geometry G, const float* __restrict_
 
 // rot[tile][n] = exp(+i 2 pi base(n, tile)): the per-(spot, tile) phase of
 // the anchor pixel, reduced exactly in turns.
-static __global__ void k_tile_rotations(const float* __restrict__ coeff, const float2* __restrict__ anchors, int N,
-                                        int D, int T, float2* __restrict__ rot) {
-  const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+__device__ __forceinline__ void tile_rotation(long long i, const float* __restrict__ coeff,
+                                              const float2* __restrict__ anchors, int N, int D, int T,
+                                              float2* __restrict__ rot) {
   if (i >= (long long)N * T) return;
   const int tile = (int)(i / N), n = (int)(i % N);
   float c[kMaxModes];
@@ -193,6 +192,18 @@ static __global__ void k_tile_rotations(const float* __restrict__ coeff, const f
   }
   // modes beyond D have c = 0 and contribute exactly 0 turns
   rot[i] = cis_turns(base_turns<kMaxModes>(c, a));
+}
+
+// Both of the coefficients' images: the first nczs CTAs build czs, the others
+// rot. One launch for the two: a gradient step of a small hologram is bound by
+// its launches from the host, and one on the separable kernels has two more
+// for their own tables.
+static __global__ void __launch_bounds__(256) k_tc_build_coeff(const float* __restrict__ coeff, int N, const TcLayout L,
+                                                               int nc64, int rep, float* __restrict__ czs, int nczs,
+                                                               const float2* __restrict__ anchors, int D, int T,
+                                                               float2* __restrict__ rot) {
+  if ((int)blockIdx.x < nczs) build_czs((long long)blockIdx.x * 256 + threadIdx.x, coeff, N, L, nc64, rep, czs);
+  else tile_rotation((long long)((int)blockIdx.x - nczs) * 256 + threadIdx.x, coeff, anchors, N, D, T, rot);
 }
 
 // --- pieces shared by the two kernels ------------------------------------------
