@@ -181,16 +181,22 @@ bool use_tc_adj(const ash_hologram* h) {
 // 82 / 49, 901 x 611 N = 230 90 / 85. A forward step and an adjoint tile cost
 // the same however few spots they have: with fewer than 64 they pay only where
 // most tiles need one strip (forward: 742 x 486 N = 27 25 / 33, 1024^2 N = 20
-// 52 / 36, 800^2 N = 12 31 / 27; adjoint 16 / 31, 39 / 22, 27 / 18). Degree 2
+// 52 / 36, 800^2 N = 12 31 / 27; adjoint 16 / 31, 39 / 22, 27 / 18), and not
+// with one or two (calls, 1024^2: adjoint N = 1 18.3 / 21.3, 3 32.8 / 22.0; loop
+// of 5 iterations N = 1 300 / 370, 2 375 / 386, 3 384 / 382; 3000 x 2000:
+// adjoint N = 4 92 / 95, 8 104 / 95). Degree 2
 // (one mixed term): forward 220^2 N = 30 12.5 / 13.8,
 // 300^2 N = 200 28 / 17; adjoint 256^2 N = 100 13.5 / 16.4, 300^2 N = 200
 // 24 / 20.
 constexpr int kSepSideFwd = 400, kSepSideAdj = 560, kSepSide2 = 200, kSepFewSpots = 64, kSepFewSide = 800;
 constexpr size_t kSepMaxBytes = (size_t)8 << 30;   // of phase polynomials, and of partial dL/dC an eighth
 constexpr long long kSepTerms2Fwd = 6LL << 20, kSepTerms2Adj = 10LL << 20;
+constexpr int kSepFewest = 3, kSepFewestLarge = 8;
+constexpr long long kSepLarge = 4LL << 20;   // pixels
 bool sep_pays(const ash_hologram* h, int side4, long long terms2) {
   const Geometry& g = h->g;
   const int side = g.nx < g.ny_full ? g.nx : g.ny_full;
+  if (g.N < (side4 == kSepSideAdj && (long long)g.nx * g.ny > kSepLarge ? kSepFewestLarge : kSepFewest)) return false;
   if (h->sep_ord <= 2) return side >= kSepSide2 && (long long)g.nx * g.ny * g.N >= terms2;
   return side >= side4 && (g.N >= kSepFewSpots || side >= kSepFewSide);
 }
@@ -206,11 +212,19 @@ constexpr int kSepSideLoop = 560;
 bool sep_in_loops(const ash_hologram* h) {
   return (h->g.nx < h->g.ny_full ? h->g.nx : h->g.ny_full) >= kSepSideLoop;
 }
+// Strong aberrations need many strips, whose time the other kernels do not pay.
+// Mean cost of a step and of a chunk against one strip, by the coefficients at
+// the handle's creation, up to which the separable kernels serve; times of the
+// other kernels over theirs: forward 700^2 N = 200 1.12 at 3.4, 900^2 1.05 at
+// 3.6, 460^2 N = 1000 1.00 at 3.7, 560^2 N = 64 1.07 at 3.0, 700^2 0.85 at 3.7,
+// 560^2 N = 300 0.69 at 5.7; adjoint 900^2 N = 300 1.00 at 3.0, 1200^2 1.03 at
+// 2.9, 700^2 1.16 at 2.4 and 0.60 at 5.3, N = 64 1.19 at 2.9 and 0.71 at 6.5.
+constexpr double kSepCostFwd = 3.0, kSepCostAdj = 2.8;
 bool use_sep_fwd(const ash_hologram* h, bool loop = false) {
-  return h->sep_ok && h->variant == 0 && (!loop || sep_in_loops(h)) && sep_pays(h, kSepSideFwd, kSepTerms2Fwd);
+  return h->sep_ok && h->sep_cheap_fwd && h->variant == 0 && (!loop || sep_in_loops(h)) && sep_pays(h, kSepSideFwd, kSepTerms2Fwd);
 }
 bool use_sep_adj(const ash_hologram* h, bool loop = false) {
-  return h->sep_ok && h->variant == 0 && (!loop || sep_in_loops(h)) && sep_pays(h, kSepSideAdj, kSepTerms2Adj);
+  return h->sep_ok && h->sep_cheap_adj && h->variant == 0 && (!loop || sep_in_loops(h)) && sep_pays(h, kSepSideAdj, kSepTerms2Adj);
 }
 // The coefficient-gradient moments on the tensor cores need one K-atom,
 // D <= 12 and a polynomial basis of total degree <= 4 (the tile polynomials);
@@ -1081,6 +1095,22 @@ ash_status create_impl(ash_hologram** out, int nx, int ny, int row0, int ny_full
   // stream-ordered allocations and set-up must be complete before the handle
   // is used from another stream (the graph capture stream, or the caller's)
   CREATE_CUDA(cudaStreamSynchronize(s));
+  if (h->sep_ok) {
+    // whether the strips that the coefficients need are few enough
+    int cost = 0, acost = 0;
+    const size_t U = (size_t)g.T * sep_blocks(N);
+    CREATE_CUDA(cudaMemcpyAsync(&cost, h->sep_cost + U, sizeof cost, cudaMemcpyDeviceToHost, s));
+    CREATE_CUDA(cudaMemcpyAsync(&acost, h->sep_acost + U, sizeof acost, cudaMemcpyDeviceToHost, s));
+    CREATE_CUDA(cudaStreamSynchronize(s));
+    const double chunks = (double)g.T * ((N + kSepChunk - 1) / kSepChunk);
+    h->sep_cheap_fwd = cost <= kSepCostFwd * sep_step_cost(0) * U;
+    h->sep_cheap_adj = acost <= kSepCostAdj * sep_chunk_cost(0) * chunks;
+    if (!h->sep_cheap_fwd && !h->sep_cheap_adj) h->sep_ok = false;
+    if (h->tc_stale && needs_tc_images(h)) {
+      if ((st = fresh_tc_images(h, s)) != ASH_OK) return fail(st);
+      CREATE_CUDA(cudaStreamSynchronize(s));
+    }
+  }
 #undef CREATE_CUDA
   // the register-image basis serves only the FMA-pipe kernels: when every
   // transform of this handle runs on the tensor cores, it is released (and

@@ -66,6 +66,8 @@ struct ash_hologram {
   float* tpoly = nullptr;       // tile polynomials of the basis
   // separable tile transforms (polynomial bases of total degree <= 4)
   bool sep_ok = false;
+  bool sep_cheap_fwd = true;    // the coefficients at creation need few strips (api.cu: kSepCostFwd)
+  bool sep_cheap_adj = true;
   int sep_ord = 0;              // total degree of the basis
   int sep_G = 0;                // forward CTAs
   float* sep_tab = nullptr;     // basis polynomials per tile

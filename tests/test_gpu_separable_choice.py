@@ -1,0 +1,68 @@
+"""Where the automatic choice takes the separable transforms: not for one or two
+spots, and not where the coefficients that a handle is created with need many
+row strips. A handle that it leaves to the other kernels returns bit for bit
+what their forced variant returns (1: few spots, 2 from 256); one created with
+weak aberrations keeps the separable kernels when stronger ones are set, up to
+the 32 strips of a tile, within the transforms' tolerance."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from gpu_helpers import REL_TOL, assert_close, oracle_inputs  # noqa: E402
+from oracle import transform  # noqa: E402
+from workloads import random_problem  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+LOW = list(range(2, 12))
+
+
+def _problem(nx, ny, N, noll, scale):
+    p = random_problem(nx + 3 * ny + N, nx, ny, N, noll, defocus_max=5.0)
+    p.coeff = np.ascontiguousarray(p.coeff * np.float32(scale))
+    y = torch.polar(torch.ones(N), torch.arange(N, dtype=torch.float32)).cuda()
+    return p, torch.from_numpy(p.phase0).cuda(), y
+
+
+def _holo(p, coeff, variant=0):
+    from paper_2505_08777_gb300 import Hologram
+    h = Hologram(torch.from_numpy(p.amp).cuda(), torch.from_numpy(coeff).cuda(), noll=p.noll)
+    h.set_variant(variant)
+    return h
+
+
+def _calls(h, ph, y):
+    dph, dC = h.grad(ph, y)
+    x, w, t = ph.clone(), torch.ones(len(y), device="cuda"), torch.ones(len(y), device="cuda")
+    E, met = h.wgs(x, w, t, 2)
+    assert h.graph_kernels(2) == h.wgs_launches(2)
+    h.check()
+    return h.forward(ph), h.adjoint(y)[0], h.zsub_sweep(ph, 1, [0.5, -0.5]), dph, dC, x, w, E
+
+
+@pytest.mark.parametrize("nx,ny,N,noll,scale,variant", [
+    (901, 930, 1, LOW, 1.0, 1),
+    (930, 901, 2, LOW, 1.0, 1),
+    (3000, 2000, 2, [2, 3, 4, 5, 6], 1.0, 1),
+    (577, 590, 260, LOW, 30.0, 2),
+])
+def test_left_to_the_other_kernels(nx, ny, N, noll, scale, variant):
+    p, ph, y = _problem(nx, ny, N, noll, scale)
+    got, want = (_calls(_holo(p, p.coeff, v), ph, y) for v in (0, variant))
+    assert all(torch.equal(a, b) for a, b in zip(got, want))
+
+
+@pytest.mark.parametrize("nx,ny,N,scale", [(577, 590, 100, 30.0), (640, 600, 97, 6.0), (905, 903, 161, 30.0)])
+def test_stronger_coefficients_set_later(nx, ny, N, scale):
+    p, ph, y = _problem(nx, ny, N, LOW, scale)
+    Z, C, A = oracle_inputs(p)
+    h = _holo(p, np.ascontiguousarray(p.coeff / np.float32(100.0)))
+    other = _holo(p, p.coeff, 2)
+    h.set_coefficients(torch.from_numpy(p.coeff).cuda())
+    E, g = h.forward(ph), h.adjoint(y)[0]
+    assert not torch.equal(g, other.adjoint(y)[0])      # another kernel's rounding
+    assert_close(E.cpu().numpy(), transform.forward(transform.field(A, p.phase0), C, Z, workers=8), REL_TOL, "forward")
+    assert_close(g.cpu().numpy(), transform.adjoint(y.cpu().numpy().astype(np.complex128), C, Z, workers=8), REL_TOL,
+                 "adjoint")
+    h.check()
