@@ -6,6 +6,7 @@
 #include <map>
 #include <mutex>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "ash.h"
@@ -125,6 +126,50 @@ void release(ash_hologram* h) {
   h->capture = nullptr;
 }
 
+constexpr size_t kSepMaxBytes = (size_t)8 << 30;   // of phase polynomials, and of partial dL/dC an eighth
+// The separable kernels' workspace, one allocation: 64 B per (tile, spot of a
+// full block) and what is left of it small, but for the gradient's partial sums
+// (left out above an eighth of kSepMaxBytes). False, without an error, if
+// it cannot be had.
+bool sep_workspace(ash_hologram* h) {
+  const size_t T = (size_t)h->g.T, D = (size_t)h->g.D, nb = (size_t)sep_blocks(h->g.N), npad = nb * kSepSpots;
+  const size_t rows = (size_t)kSepFwdRows * h->sep_G, dp = rows * D * npad;
+  for (int pass = 0; pass < 2; ++pass) {
+    uint8_t* p = static_cast<uint8_t*>(h->sep_block);
+    size_t at = 0;
+    auto take = [&](auto** out, size_t n) {
+      if (pass) *out = reinterpret_cast<std::decay_t<decltype(*out)>>(p + at);
+      at += (n * sizeof(**out) + 255) & ~(size_t)255;
+    };
+    take(&h->sep_tab, T * D * kSepTab);
+    take(&h->sep_poly, T * 16 * npad);
+    take(&h->sep_strips, T * nb);
+    take(&h->sep_cost, T * nb + 1);
+    take(&h->sep_acost, T * nb + 2);
+    take(&h->sep_split, 2 * (size_t)h->sep_G * kTilePix);
+    take(&h->sep_ys, 2 * npad);
+    take(&h->sep_scale, npad / kSepChunk);
+    if (dp * sizeof(float) <= kSepMaxBytes / 8) take(&h->sep_dpart, dp);
+    take(&h->sep_tickets, T);
+    take(&h->sep_part, rows * npad);
+    h->sep_bytes = at;
+    if (!pass) {
+      const std::string error = g_last_error;
+      if (ws_alloc(h, &h->sep_block, at) != ASH_OK) {
+        g_last_error = error;
+        return false;
+      }
+    }
+  }
+  return true;
+}
+
+void drop_sep_workspace(ash_hologram* h) {
+  free_one(h, h->sep_block, h->sep_bytes);
+  h->sep_block = nullptr;
+  h->sep_dpart = nullptr;
+}
+
 cudaError_t prepare(int D, LaunchInfo* li) {
   switch (range_of(D)) {
     case 0: return prepare_r0(D, li);
@@ -189,7 +234,6 @@ bool use_tc_adj(const ash_hologram* h) {
 // 300^2 N = 200 28 / 17; adjoint 256^2 N = 100 13.5 / 16.4, 300^2 N = 200
 // 24 / 20.
 constexpr int kSepSideFwd = 400, kSepSideAdj = 560, kSepSide2 = 200, kSepFewSpots = 64, kSepFewSide = 800;
-constexpr size_t kSepMaxBytes = (size_t)8 << 30;   // of phase polynomials, and of partial dL/dC an eighth
 constexpr long long kSepTerms2Fwd = 6LL << 20, kSepTerms2Adj = 10LL << 20;
 constexpr int kSepFewest = 3, kSepFewestLarge = 8;
 constexpr long long kSepLarge = 4LL << 20;   // pixels
@@ -986,21 +1030,6 @@ ash_status create_impl(ash_hologram** out, int nx, int ny, int row0, int ny_full
     if ((st = ws(h, &h->tadj_begin, tadj_begin.size())) != ASH_OK) return fail(st);
     if ((st = ws(h, &h->tadj_groups, tadj_groups.size() + 1)) != ASH_OK) return fail(st);
   }
-  if (h->sep_ok) {
-    const size_t npad = (size_t)sep_blocks(N) * kSepSpots;
-    if ((st = ws(h, &h->sep_tab, (size_t)g.T * D * kSepTab)) != ASH_OK) return fail(st);
-    if ((st = ws(h, &h->sep_poly, (size_t)g.T * 16 * npad)) != ASH_OK) return fail(st);
-    if ((st = ws(h, &h->sep_strips, (size_t)g.T * sep_blocks(N))) != ASH_OK) return fail(st);
-    if ((st = ws(h, &h->sep_cost, (size_t)g.T * sep_blocks(N) + 1)) != ASH_OK) return fail(st);
-    if ((st = ws(h, &h->sep_acost, (size_t)g.T * sep_blocks(N) + 2)) != ASH_OK) return fail(st);
-    if ((st = ws(h, &h->sep_split, 2 * (size_t)h->sep_G * kTilePix)) != ASH_OK) return fail(st);
-    if ((st = ws(h, &h->sep_ys, 2 * npad)) != ASH_OK) return fail(st);
-    if ((st = ws(h, &h->sep_scale, npad / kSepChunk)) != ASH_OK) return fail(st);
-    const size_t dp = (size_t)kSepFwdRows * h->sep_G * D * npad;
-    if (dp * sizeof(float) <= kSepMaxBytes / 8 && (st = ws(h, &h->sep_dpart, dp)) != ASH_OK) return fail(st);
-    if ((st = ws(h, &h->sep_tickets, (size_t)g.T)) != ASH_OK) return fail(st);
-    if ((st = ws(h, &h->sep_part, (size_t)kSepFwdRows * h->sep_G * npad)) != ASH_OK) return fail(st);
-  }
   if (h->tgrad_ok) {
     if ((st = ws(h, &h->tpoly, tc_tpoly_floats(g, h->tgrad_ord))) != ASH_OK) return fail(st);
     if ((st = ws(h, &h->tgrad_part, (size_t)h->tgrad.G * 2 * kTcRows * tc_grad_dp(D))) != ASH_OK) return fail(st);
@@ -1031,6 +1060,8 @@ ash_status create_impl(ash_hologram** out, int nx, int ny, int row0, int ny_full
     if ((st = ws(h, &h->terms, spec->terms.size() + 1)) != ASH_OK) return fail(st);
     if ((st = ws(h, &h->term_off, spec->off.size())) != ASH_OK) return fail(st);
   }
+  // last, so that a handle whose memory does not reach serves as without it
+  if (h->sep_ok && !sep_workspace(h)) h->sep_ok = false;
   ce = cudaStreamCreateWithFlags(&h->capture, cudaStreamNonBlocking);
   if (ce != cudaSuccess) return fail(cuda_fail(ce, "capture stream"));
 
@@ -1105,7 +1136,10 @@ ash_status create_impl(ash_hologram** out, int nx, int ny, int row0, int ny_full
     const double chunks = (double)g.T * ((N + kSepChunk - 1) / kSepChunk);
     h->sep_cheap_fwd = cost <= kSepCostFwd * sep_step_cost(0) * U;
     h->sep_cheap_adj = acost <= kSepCostAdj * sep_chunk_cost(0) * chunks;
-    if (!h->sep_cheap_fwd && !h->sep_cheap_adj) h->sep_ok = false;
+    if (!h->sep_cheap_fwd && !h->sep_cheap_adj) {
+      h->sep_ok = false;
+      drop_sep_workspace(h);
+    }
     if (h->tc_stale && needs_tc_images(h)) {
       if ((st = fresh_tc_images(h, s)) != ASH_OK) return fail(st);
       CREATE_CUDA(cudaStreamSynchronize(s));

@@ -70,6 +70,8 @@ struct ash_hologram {
   bool sep_cheap_adj = true;
   int sep_ord = 0;              // total degree of the basis
   int sep_G = 0;                // forward CTAs
+  void* sep_block = nullptr;    // the allocation that holds the following
+  size_t sep_bytes = 0;
   float* sep_tab = nullptr;     // basis polynomials per tile
   float* sep_poly = nullptr;    // phase polynomials per (tile, spot)
   unsigned char* sep_strips = nullptr;   // per (tile, spot block): log2 of its row strips

@@ -66,3 +66,39 @@ def test_stronger_coefficients_set_later(nx, ny, N, scale):
     assert_close(g.cpu().numpy(), transform.adjoint(y.cpu().numpy().astype(np.complex128), C, Z, workers=8), REL_TOL,
                  "adjoint")
     h.check()
+
+
+def test_a_handle_without_memory_for_them_serves_on_the_other_kernels():
+    from paper_2505_08777_gb300 import _lib
+    lib = _lib.load()
+    sizes, refuse = [], set()
+    stream = torch.cuda.current_stream().cuda_stream
+
+    def alloc(ctx, n, s):
+        sizes.append(n)
+        if len(sizes) - 1 in refuse:
+            return None
+        return torch.cuda.caching_allocator_alloc(n, 0, stream)
+
+    hooks = _lib.ALLOC_FN(alloc), _lib.FREE_FN(lambda ctx, p, s: torch.cuda.caching_allocator_delete(p))
+    p, ph, y = _problem(905, 903, 300, LOW, 1.0)
+    assert lib.ash_set_allocator(*hooks, None) == 0
+    try:
+        full = _holo(p, p.coeff)
+        block = sizes[-1]                               # taken last
+        E_sep, full_bytes = full.forward(ph), full.workspace_bytes()
+        full.close()
+        count = len(sizes)
+        sizes.clear()
+        refuse.add(count - 1)
+        h = _holo(p, p.coeff)
+        assert len(sizes) == count and sizes[-1] == block
+        assert h.workspace_bytes() == full_bytes - block
+        got = _calls(h, ph, y)
+        h.close()
+    finally:
+        torch.cuda.synchronize()
+        lib.ash_set_allocator(_lib.ALLOC_FN(0), _lib.FREE_FN(0), None)
+    want = _calls(_holo(p, p.coeff, 2), ph, y)
+    assert all(torch.equal(a, b) for a, b in zip(got, want))
+    assert_close(E_sep.cpu().numpy(), want[0].cpu().numpy(), 1e-5, "separable forward")
