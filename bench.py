@@ -510,10 +510,11 @@ def main():
                                 f"spots into TMEM, sincos + packed complex MAC, arg epilogue)") if adj_tc else
                                f"k_adjoint<D={p.D},P={P}> (pixel-stationary adjoint, arg epilogue)"}
     achieved = gterm[dom]
-    sep = max(p.noll) <= 15 and min(p.nx, p.ny) >= 560 and p.N >= 64   # the automatic choice of the separable kernels
-    if sep:
-        kernel_names = {"forward": "k_sep_forward (tile rows on tcgen05 split-f16 MMA, 64 sincos per spot and tile)",
-                        "adjoint": "k_sep_adjoint (tile sums on tcgen05 split-f16 MMA, 64 sincos per spot and tile)"}
+    if linfo["kernels"] & 16:
+        kernel_names["forward"] = "k_sep_forward (tile rows on tcgen05 split-f16 MMA, 64 sincos per spot and tile)"
+    if linfo["kernels"] & 32:
+        kernel_names["adjoint"] = "k_sep_adjoint (tile sums on tcgen05 split-f16 MMA, 64 sincos per spot and tile)"
+    sep = bool(linfo["kernels"] & (16 if dom == "forward" else 32))
     roofline = roofline_alu(achieved, p.D, rates, kernel_names[dom], f"N*M = {NM} terms")
     if sep:
         # R_terms counts one sin / cos per term; these kernels are bounded by their tensor-core products instead

@@ -418,8 +418,9 @@ ash_status ash_wgs_iterate(ash_hologram *h, float *phase, float *w, const float 
  *               (forward pass with D moments, tiles recomputed; the phases
  *               C_n . Z_m come from the tensor cores when the operand row
  *               fits one K-atom, D <= 12 and the basis is a polynomial of
- *               total degree <= 4, else from the FMA pipe).
- * The tensor-core moment pass overwrites the handle's nearfield image (no
+ *               total degree <= 4, else from the FMA pipe; large grids of such a
+ *               basis: the separable kernels' row sums).
+ * The tensor-core and separable moment passes overwrite the handle's nearfield image (no
  * other state of the handle changes).
  *   phase   device float[ny*nx];  grad_E device float[2*N];
  *   dphase  device float[ny*nx] or NULL;  dcoeff device float[N*D] or NULL.
@@ -436,15 +437,25 @@ ash_status ash_grad(ash_hologram *h, const float *phase, const float *grad_E, fl
  *    the tensor-core forward splits spot blocks, bit 3: the tensor-core
  *    forward's CTAs claim their ranges by SM), kernels in use (adjoint:
  *    1 FMA or 2 tensor core, plus 4 if the forward and 8 if the
- *    coefficient-gradient moments use the tensor core), pixels per thread}.
+ *    coefficient-gradient moments use the tensor core; in place of these the
+ *    separable tile kernels serve the forward if 16 is set, the adjoint if 32,
+ *    the moments if 64, and inside ash_wgs_iterate the forward if 128 and the
+ *    adjoint if 256), pixels per thread}.
  */
 ash_status ash_hologram_launch_info(const ash_hologram *h, int *out);
 
 /*
  * Kernel variant of the forward and adjoint transforms and of the
  * coefficient-gradient moments: 0 = automatic (the faster measured family
- * per pass: tensor cores when the operand row fits one K-atom, for the
- * forward and the moments from N = 64 spots, for the adjoint from N = 256),
+ * per pass: the separable tile kernels for polynomial bases of total degree
+ * <= 4 from N = 3 spots on grids whose shorter side is long enough (degree
+ * 3 and 4: the forward from 400, the adjoint from 560, from 800 with fewer
+ * than 64 spots, the moments from 900; degree <= 2: from 200 and 6 and 10 Mi
+ * terms; ash_wgs_iterate: from 560 for every degree), unless the coefficients
+ * at creation vary so strongly that most tiles need several row strips; else
+ * tensor cores when the operand row fits one K-atom, for the
+ * forward and the moments from N = 64 spots, for the adjoint from N = 256;
+ * else the FMA pipe),
  * 1 = FMA-pipe kernels, 2 = tensor-core kernels (available for every D a
  * handle accepts: one K-atom per operand row for D <= 10 and for D = 11
  * with both tilts, two otherwise; the moments stay on the FMA pipe where

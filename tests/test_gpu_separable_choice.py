@@ -102,3 +102,25 @@ def test_a_handle_without_memory_for_them_serves_on_the_other_kernels():
     want = _calls(_holo(p, p.coeff, 2), ph, y)
     assert all(torch.equal(a, b) for a, b in zip(got, want))
     assert_close(E_sep.cpu().numpy(), want[0].cpu().numpy(), 1e-5, "separable forward")
+
+
+# launch-info bits: 16 / 32 / 64 separable forward, adjoint, moments; 128 / 256 forward and adjoint of a loop
+@pytest.mark.parametrize("nx,ny,N,noll,scale,bits", [
+    (417, 403, 65, LOW, 0.05, 16),
+    (399, 700, 65, LOW, 0.05, 0),
+    (561, 577, 129, LOW, 0.05, 16 | 32 | 128 | 256),
+    (577, 590, 260, LOW, 30.0, 0),
+    (640, 700, 63, LOW, 0.05, 0),
+    (803, 801, 7, LOW, 0.1, 16 | 32 | 128 | 256),
+    (905, 903, 161, LOW, 0.1, 16 | 32 | 64 | 128 | 256),
+    (901, 930, 2, LOW, 1.0, 0),
+    (233, 201, 231, [2, 3, 4, 5, 6], 1.0, 16 | 32),
+    (901, 930, 20, [2, 3, 4, 5, 6], 1.0, 16 | 32 | 64 | 128 | 256),
+    (600, 600, 70, list(range(2, 17)), 0.05, 0),          # degree 5
+])
+def test_launch_info_tells_the_choice(nx, ny, N, noll, scale, bits):
+    p, _, _ = _problem(nx, ny, N, noll, scale)
+    h = _holo(p, p.coeff)
+    assert h.launch_info()["kernels"] & ~15 == bits
+    h.set_variant(2)
+    assert h.launch_info()["kernels"] & ~15 == 0
