@@ -304,10 +304,13 @@ __device__ __forceinline__ void spot_loss_body(const float2* __restrict__ E, con
   }
   sI = block_sum<1024>(sI, red);
   const double mu = sI / N, inv = mu > 0.0 ? 1.0 / mu : 0.0;
+  // (divided by mu, not multiplied by its reciprocal, which took 2 to 4 us less of
+  // the kernel's 18.5 at N = 400 and 25.5 at 1024: a single spot is exactly 1, and
+  // its gradient exactly 0)
   double sL = 0.0, sR = 0.0;
   for (int n = threadIdx.x; n < N; n += 1024) {
     const float2 e = E[n];
-    const double x = ((double)e.x * e.x + (double)e.y * e.y) * inv;
+    const double x = mu > 0.0 ? ((double)e.x * e.x + (double)e.y * e.y) / mu : 0.0;
     const double r = x - (double)t[n];
     sL += r * r;
     sR += r * x;
@@ -319,7 +322,7 @@ __device__ __forceinline__ void spot_loss_body(const float2* __restrict__ E, con
   const double c = sR / N, f = 4.0 * inv;
   for (int n = threadIdx.x; n < N; n += 1024) {
     const float2 e = E[n];
-    const double x = ((double)e.x * e.x + (double)e.y * e.y) * inv;
+    const double x = mu > 0.0 ? ((double)e.x * e.x + (double)e.y * e.y) / mu : 0.0;
     const double G = f * ((x - (double)t[n]) - c);
     gE[n] = make_float2((float)(G * e.x), (float)(G * e.y));
   }
