@@ -799,7 +799,10 @@ ash_status apply_choice(ash_batch* b, const TuneChoice& c, cudaStream_t s) {
   return st;
 }
 
-// Copies of many arrays of floats (a batch call's states) in one launch.
+// Copies of many arrays of floats (a batch call's states) in one launch, in the
+// order given: a launch's copies run side by side, so one to memory that an
+// earlier copy of the launch writes (members that share a tensor) begins the
+// next launch.
 constexpr int kCopies = 120;
 struct CopyList {
   const float* src[kCopies];
@@ -821,8 +824,17 @@ __global__ void __launch_bounds__(256) k_batch_copy(const __grid_constant__ Copy
 struct Copies {
   CopyList l;
   int count = 0;
+  uintptr_t lo = 0, hi = 0;   // span of the launch's destinations
   cudaStream_t s;
   cudaError_t err = cudaSuccess;
+  bool written(uintptr_t a, uintptr_t b) const {
+    if (count == 0 || b <= lo || a >= hi) return false;
+    for (int k = 0; k < count; ++k) {
+      const uintptr_t d = reinterpret_cast<uintptr_t>(l.dst[k]);
+      if (a < d + sizeof(float) * l.n[k] && d < b) return true;
+    }
+    return false;
+  }
   void flush() {
     if (count > 0 && err == cudaSuccess) {
       k_batch_copy<<<dim3(32, count), 256, 0, s>>>(l);
@@ -831,6 +843,10 @@ struct Copies {
     count = 0;
   }
   void add(float* dst, const float* src, size_t n) {
+    const uintptr_t a = reinterpret_cast<uintptr_t>(dst), b = a + sizeof(float) * n;
+    if (written(a, b)) flush();
+    lo = count ? std::min(lo, a) : a;
+    hi = count ? std::max(hi, b) : b;
     l.src[count] = src;
     l.dst[count] = dst;
     l.n[count] = (unsigned)n;
