@@ -216,18 +216,26 @@ __device__ __forceinline__ SepColumns sep_columns(const SepPoly& q, int s, int l
   return o;
 }
 
+// The exponent e by which values are scaled to |x| <= 1: the largest, with the
+// bits mx, is below 2^e. Over the whole range of floats (from 2^127 on |x| < 2, the
+// split a bit coarser); 2^-127 is the subnormal 0x00400000.
+__device__ __forceinline__ int sep_exponent(uint32_t mx) { return min(max((int)(mx >> 23), 0), 253) - 126; }
+__device__ __forceinline__ float pow2_up(int e) { return __uint_as_float((uint32_t)(127 + e) << 23); }
+__device__ __forceinline__ float pow2_down(int e) {
+  return __uint_as_float(e == 127 ? 0x00400000u : (uint32_t)(127 - e) << 23);
+}
+
 // y of the 32 spots of a chunk divided by a power of two (scale), so that
 // |y| <= 1: the 32 real, then the 32 imaginary parts; by one warp.
 __device__ __forceinline__ void sep_scale_chunk(const float2* __restrict__ y, int N, int c, float* __restrict__ ys,
                                                 float* __restrict__ scale) {
   const int lane = threadIdx.x & 31, n = c * 32 + lane;
   const float2 v = n < N ? __ldg(y + n) : make_float2(0.0f, 0.0f);
-  const uint32_t mx = __reduce_max_sync(0xffffffffu, __float_as_uint(hypotf(v.x, v.y)));
-  const int e = min(max((int)(mx >> 23), 27), 227) - 126;
-  const float inv = __uint_as_float((uint32_t)(127 - e) << 23);
+  const int e = sep_exponent(__reduce_max_sync(0xffffffffu, __float_as_uint(hypotf(v.x, v.y))));
+  const float inv = pow2_down(e);
   ys[c * 64 + lane] = v.x * inv;
   ys[c * 64 + 32 + lane] = v.y * inv;
-  if (lane == 0) scale[c] = __uint_as_float((uint32_t)(127 + e) << 23);
+  if (lane == 0) scale[c] = pow2_up(e);
 }
 
 }  // namespace ash

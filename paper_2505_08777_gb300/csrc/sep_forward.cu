@@ -639,9 +639,8 @@ __global__ void __launch_bounds__(kFwdThreads, 1) k_sep_forward(const SepFwdPara
       uint32_t m = 0;
 #pragma unroll
       for (int q = 0; q < 8; ++q) m = max(m, smax[q]);
-      // exponent e with max < 2^e, kept where 2^e and 2^-e are normal
-      const int e = min(max((int)(m >> 23), 27), 227) - 126;
-      const float inv = __uint_as_float((uint32_t)(127 - e) << 23);
+      const int e = sep_exponent(m);
+      const float inv = pow2_down(e);
       constexpr uint32_t S = 0x80008000u;
 #pragma unroll
       for (int k2 = 0; k2 < 2; ++k2) {
@@ -669,7 +668,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) k_sep_forward(const SepFwdPara
           put16(bh + kFB, r0 + 2, 4 + c, rl);
         }
       }
-      return __uint_as_float((uint32_t)(127 + e) << 23);
+      return pow2_up(e);
     };
 
     // A: X(u) of this thread's spot for its 16 columns, about the strip's row
