@@ -41,7 +41,8 @@ struct ash_hologram {
   bool tadj_split = false;      // some group's spots span two CTA ranges
   ash::TcFwdSched tfwd{};       // forward units (spot block, pixel chunk)
   bool tfwd_split = false;      // some spot block's pixels span two CTA ranges
-  bool tc_stale = false;        // czs and rot are older than the coefficients (no kernel in use reads them)
+  bool tc_stale = false;        // czs and rot are older than the coefficients
+  bool tc_unseen = false;       // or may be, by replays of a captured call: rebuilt before every read
   bool tc_pinned = false;       // a batch's persistent kernels or a caller's graph of variant 2 may read them
   float* zs = nullptr;
   float* czs = nullptr;

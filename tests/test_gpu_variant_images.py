@@ -71,6 +71,15 @@ def test_replayed_coefficients_reach_a_later_variant(setup):
     assert torch.equal(E, _want(amp, ph, Cs[2], 0))
     h.set_variant(2)
     assert torch.equal(h.forward(ph), _want(amp, ph, Cs[2]))
+    # also while the variant stays, and by a forward captured in it
+    later, E2 = _capture(lambda: h.forward(ph))
+    C.copy_(Cs[3])
+    graph.replay()
+    assert torch.equal(h.forward(ph), _want(amp, ph, Cs[3]))
+    C.copy_(Cs[1])
+    graph.replay()
+    later.replay()
+    assert torch.equal(E2, _want(amp, ph, Cs[1]))
 
 
 def test_captured_but_not_replayed_coefficients_do_not_count(setup):
