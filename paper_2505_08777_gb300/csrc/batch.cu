@@ -241,7 +241,8 @@ BatchKernel adj_kernel(int dmax) {
 // Branches of a batch's captured loop that the standalone members are dealt
 // to: they share nothing, and a small one leaves most of the chip idle (16
 // members of 256^2 to 512^2, 5 iterations: 3.17 ms in one chain, 1.93 in 8, with
-// the copies of k_batch_copy).
+// the copies of k_batch_copy; 2.13 since loops of that size are off the separable
+// kernels).
 constexpr int kBatchLanes = 8;
 
 struct ash_batch {

@@ -153,8 +153,12 @@ __device__ __forceinline__ SepPoly sep_unpack(const float* w) {
 }
 
 // sin and cos of two angles through the MUFU. Its error is a phase error of
-// -7.5e-8 of the angle (besides the random part), so the angles are kept to
-// [-pi, pi] and a little.
+// -7.5e-8 of the angle (besides the random part). The tilt and the base are
+// reduced to [-pi, pi], the pure powers over a tile are not: they are far below
+// 1 for ordinary aberrations, and with 1400 rad of defocus on 300^2 (70 rad) the
+// forward is 8.8e-7 off, where the kernels of one sine and cosine per term are
+// 1.2e-5 (at 20 rad 3.8e-7 and 2.2e-6). FP32 polynomials (rms 3.5e-8) in place of
+// the MUFU bring the adjoint from 3.1e-7 to 2.9e-7 and cost it 4 to 12 %.
 __device__ __forceinline__ void cis2(float2 x, float2& c, float2& s) {
   s.x = __sinf(x.x);
   c.x = __cosf(x.x);

@@ -124,3 +124,15 @@ def test_launch_info_tells_the_choice(nx, ny, N, noll, scale, bits):
     assert h.launch_info()["kernels"] & ~15 == bits
     h.set_variant(2)
     assert h.launch_info()["kernels"] & ~15 == 0
+
+
+@pytest.mark.parametrize("nx,ny,N,scale", [(905, 903, 161, 7.5), (620, 610, 260, 2.2)])
+def test_forward_alone_beside_the_other_adjoint(nx, ny, N, scale):
+    # strips enough for the adjoint's line, not for the forward's
+    p, ph, y = _problem(nx, ny, N, LOW, scale)
+    Z, C, A = oracle_inputs(p)
+    h = _holo(p, p.coeff)
+    assert h.launch_info()["kernels"] & ~15 == 16 | 128
+    got = _calls(h, ph, y)
+    assert_close(got[0].cpu().numpy(), transform.forward(transform.field(A, p.phase0), C, Z, workers=8), REL_TOL, "forward")
+    assert torch.equal(got[1], _holo(p, p.coeff, 2 if N >= 256 else 1).adjoint(y)[0])
