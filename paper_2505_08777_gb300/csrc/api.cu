@@ -508,7 +508,7 @@ ash_status enqueue_forward(ash_hologram* h, int source, const float* phase, cons
   if (sep || use_tc_fwd(h)) {
     cudaError_t e = cudaSuccess;
     if (source != kSrcImg) {
-      e = tc_field_img(h->g, h->amp_img, source == kSrcPhase ? phase : nullptr, field, h->fimg, s);
+      e = tc_field_img(h->g, h->amp_img, source == kSrcPhase ? phase : nullptr, field, h->fimg, s, sep);
       if (e != cudaSuccess) return cuda_fail(e, "nearfield image launch");
     }
     if (sep) {
@@ -1400,7 +1400,7 @@ ash_status ash_grad(ash_hologram* h, const float* phase, const float* grad_E, fl
     if (st != ASH_OK) return st;
   }
   if (dcoeff && use_sep_grad(h)) {
-    ASH_CUDA(tc_field_img(h->g, h->amp_img, phase, nullptr, h->fimg, s));
+    ASH_CUDA(tc_field_img(h->g, h->amp_img, phase, nullptr, h->fimg, s, true));
     const SepFwdParams sp = sep_grad_params(h, gE, dcoeff);
     ASH_CUDA(sep_launch_gradc(sp, s));
     ASH_CUDA(sep_launch_gradc_reduce(sp, s));
@@ -1504,7 +1504,7 @@ ash_status ash_profile(ash_hologram* h, const float* phase, const float* y, floa
   const bool tc = use_tc_fwd(h), tca = use_tc_adj(h), sf = use_sep_fwd(h), sa = use_sep_adj(h), sg = use_sep_grad(h);
   const TcFwdParams tf = tc_fwd_params(h, h->E);
   const SepFwdParams spf = sep_fwd_params(h, h->E);
-  if (sf || tc) e = tc_field_img(h->g, h->amp_img, phase, nullptr, h->fimg, s);
+  if (sf || tc) e = tc_field_img(h->g, h->amp_img, phase, nullptr, h->fimg, s, sf);
   cudaEventRecord(ev[0], s);
   if (e == cudaSuccess) e = sf ? sep_launch_forward(spf, s) : tc ? tc_launch_forward(h->tc_na, tf, h->tfwd.G, s) : launch_forward(h->g.D, fp, h->sched.G, s);
   cudaEventRecord(ev[1], s);

@@ -10,6 +10,13 @@ The coefficients are a weighted least-squares fit on Chebyshev nodes of r
 to float32. Running this file prints them and the worst absolute error of
 sin x and cos x over r in [-1/2, 1/2], evaluated with float32 rounding after
 every operation (an upper bound for the fused multiply-adds of the device).
+
+It also prints the coefficients of cis2_turns (sep_common.cuh), whose error over
+a turn has to vanish on average as well: with the zeros of sine and cosine
+taken out,
+    sin 2 pi r = r (1/4 - u) P(u),    cos 2 pi r = (1 - 16 u) Q(u),
+P of degree 5 and Q of degree 6, evaluated with a rounding per fused
+multiply-add as the device does.
 """
 import numpy as np
 
@@ -47,9 +54,44 @@ def evaluate(s, c, n=200001):
     return float(np.max(np.abs(sinx - np.sin(x)))), float(np.max(np.abs(cosx - np.cos(x))))
 
 
+ZEROS_S, ZEROS_C = 5, 6
+
+
+def fit_zeros():
+    k = np.arange(6000)
+    r = 0.5 * np.cos(np.pi * (k + 0.5) / len(k))
+    u = r * r
+    wp, wq = r * (0.25 - u), 1.0 - 16.0 * u
+    p = np.linalg.lstsq(np.vander(u, ZEROS_S + 1, increasing=True) * wp[:, None], np.sin(2 * np.pi * r), rcond=None)[0]
+    q = np.linalg.lstsq(np.vander(u, ZEROS_C + 1, increasing=True) * wq[:, None], np.cos(2 * np.pi * r), rcond=None)[0]
+    return p.astype(np.float32), q.astype(np.float32)
+
+
+def evaluate_zeros(p, q, n=2000001):
+    """Max and rms error of the sine, the same of the cosine, mean error of the cosine."""
+    f = np.float32
+
+    def fma(a, b, c):
+        return (np.float64(a) * np.float64(b) + np.float64(c)).astype(f)
+    r = np.linspace(-0.5, 0.5, n).astype(f)
+    u = r * r
+    P, Q = np.full_like(u, p[-1]), np.full_like(u, q[-1])
+    for a in p[-2::-1]:
+        P = fma(P, u, a)
+    for a in q[-2::-1]:
+        Q = fma(Q, u, a)
+    x = 2.0 * np.pi * r.astype(np.float64)
+    es, ec = (r * (f(0.25) - u)) * P - np.sin(x), fma(u, f(-16.0), f(1.0)) * Q - np.cos(x)
+    return np.abs(es).max(), np.sqrt(np.mean(es * es)), np.abs(ec).max(), np.sqrt(np.mean(ec * ec)), np.mean(ec)
+
+
 if __name__ == "__main__":
     s, c = fit()
     es, ec = evaluate(s, c)
     print("S:", ", ".join(f"{v:.9e}f" for v in s))
     print("C:", ", ".join(f"{v:.9e}f" for v in c))
     print(f"max |sin error| {es:.3e}, max |cos error| {ec:.3e}")
+    p, q = fit_zeros()
+    print("P:", ", ".join(f"{v:.9e}f" for v in p))
+    print("Q:", ", ".join(f"{v:.9e}f" for v in q))
+    print("sin max %.2e rms %.2e, cos max %.2e rms %.2e mean %.1e" % evaluate_zeros(p, q))

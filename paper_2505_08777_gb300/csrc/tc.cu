@@ -182,10 +182,10 @@ cudaError_t tc_build_coeff(const Geometry& g, const TcLayout& L, const float* co
 }
 
 cudaError_t tc_field_img(const Geometry& g, const float* amp_img, const float* phase, const float2* field,
-                         float4* fimg, cudaStream_t s) {
+                         float4* fimg, cudaStream_t s, bool exact) {
   const long long px = (long long)g.T * kTilePix;
   return launch_pdl(k_tc_field_img, blocks_for(px, 256), 256, 0, s, g, amp_img, phase, field,
-                    reinterpret_cast<float*>(fimg));
+                    reinterpret_cast<float*>(fimg), exact);
 }
 
 }  // namespace ash

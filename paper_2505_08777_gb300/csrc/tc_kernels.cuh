@@ -153,7 +153,7 @@ __device__ __forceinline__ float turns_of_phase(float ph) {
 // holds (A_2p, A_2p+1, phi_2p, phi_2p+1).
 static __global__ void k_tc_field_img(const Geometry G, const float* __restrict__ amp_img,
                                       const float* __restrict__ phase, const float2* __restrict__ field,
-                                      float* __restrict__ fimg) {
+                                      float* __restrict__ fimg, bool exact) {
   pdl_begin();
   const long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= (long long)G.T * kTilePix) return;
@@ -165,11 +165,12 @@ static __global__ void k_tc_field_img(const Geometry G, const float* __restrict_
     const size_t m = (size_t)px.j * G.nx + px.i;
     if (phase) {
       a = amp_img[px.img];
-      ph = turns_of_phase(phase[m]);
+      ph = exact ? exact_turns(phase[m]) : turns_of_phase(phase[m]);
     } else {
       const float2 f = field[m];
       a = hypotf(f.x, f.y);
-      ph = (f.x == 0.0f && f.y == 0.0f) ? 0.0f : atan2f(f.y, f.x) * 0.15915494309189535f;
+      ph = (f.x == 0.0f && f.y == 0.0f) ? 0.0f : atan2f(f.y, f.x);
+      ph = exact ? exact_turns(ph) : ph * 0.15915494309189535f;
     }
   }
   float* q = fimg + ((size_t)qc * 32 + (r >> 1)) * 4;

@@ -286,7 +286,9 @@ cudaError_t tc_field_img_batch(const TcFieldDesc* ds, const int* tiles0, int cou
 cudaError_t tc_build_zs(const Geometry& g, const TcLayout& L, const float* dz, float* zs, cudaStream_t s);
 cudaError_t tc_build_coeff(const Geometry& g, const TcLayout& L, const float* coeff, const float2* anchors, float* czs,
                            float2* rot, cudaStream_t s);
+// exact: for the separable kernels, whose spots are compared with kernels that
+// take the phase itself (the others keep their rounding).
 cudaError_t tc_field_img(const Geometry& g, const float* amp_img, const float* phase, const float2* field,
-                         float4* fimg, cudaStream_t s);
+                         float4* fimg, cudaStream_t s, bool exact = false);
 
 }  // namespace ash
