@@ -429,8 +429,9 @@ TcFwdParams tc_fwd_params(const ash_hologram* h, float2* E) {
   return p;
 }
 
-SepFwdParams sep_fwd_params(const ash_hologram* h, float2* E) {
+SepFwdParams sep_fwd_params(const ash_hologram* h, float2* E, bool exact = true) {
   SepFwdParams p{};
+  p.exact = exact;
   p.g = h->g;
   p.nb = sep_blocks(h->g.N);
   p.poly = h->sep_poly;
@@ -508,11 +509,11 @@ ash_status enqueue_forward(ash_hologram* h, int source, const float* phase, cons
   if (sep || use_tc_fwd(h)) {
     cudaError_t e = cudaSuccess;
     if (source != kSrcImg) {
-      e = tc_field_img(h->g, h->amp_img, source == kSrcPhase ? phase : nullptr, field, h->fimg, s, sep);
+      e = tc_field_img(h->g, h->amp_img, source == kSrcPhase ? phase : nullptr, field, h->fimg, s, sep && !loop);
       if (e != cudaSuccess) return cuda_fail(e, "nearfield image launch");
     }
     if (sep) {
-      const SepFwdParams sp = sep_fwd_params(h, E);
+      const SepFwdParams sp = sep_fwd_params(h, E, !loop);
       e = sep_launch_forward(sp, s);
       if (e == cudaSuccess) e = sep_launch_forward_reduce(sp, s);
       return e == cudaSuccess ? ASH_OK : cuda_fail(e, "separable forward launch");

@@ -233,7 +233,7 @@ __global__ void __launch_bounds__(kAdjThreads, 1) k_sep_adjoint(const SepAdjPara
           if (j >= g.ny) break;
           adjoint_epilogue(o.out, (size_t)j * g.nx + pi, v[q].x, v[q].y, amp[q]);
           if (o.out.epilogue & kEpiFimg) {
-            const float ph = (v[q].x == 0.0f && v[q].y == 0.0f) ? 0.0f : exact_turns(atan2f(v[q].y, v[q].x));
+            const float ph = (v[q].x == 0.0f && v[q].y == 0.0f) ? 0.0f : atan2f(v[q].y, v[q].x) * 0.15915494309189535f;
             // row 8 q + w of the tile, column lane
             float* f = reinterpret_cast<float*>(o.fimg + ((size_t)x.tile * kTcChunksPerTile + 4 * q + (w >> 1)) * 32 +
                                                 (w & 1) * 16 + (lane >> 1)) + (lane & 1);

@@ -239,8 +239,9 @@ struct SepStep {
 // The tensor core's fp32 accumulator truncates: measured over 256^2 to
 // 1920 x 1152 pixels, fields came out smaller by 1.9e-7 of themselves whatever
 // the input (phases 1.83e-7 to 2.2e-7, random fields 1.6e-7 to 1.8e-7), and by
-// 5e-8 at random. This makes up for the first.
-constexpr float kTruncation = 1.9e-7f;
+// 5e-8 at random; 2.8e-7 with the pixel phases of a loop. This makes up for the
+// first.
+constexpr float kTruncation = 1.9e-7f, kTruncationLoop = 1.0f + 2.4e-7f;
 
 // Sums over row pairs of c Tr, s Ti, c Ti, s Tr, with Y = c - i s.
 struct SepSum {
@@ -478,8 +479,8 @@ __global__ void __launch_bounds__(kFwdThreads, 1) k_sep_forward(const SepFwdPara
       } else {
         float2* o = part + pb * kSepSpots;
         const float re = (acc.cr.x + acc.cr.y) + (acc.si.x + acc.si.y), im = (acc.ci.x + acc.ci.y) - (acc.sr.x + acc.sr.y);
-        atomicAdd(&o->x, fmaf(re, kTruncation, re) * pscale);
-        atomicAdd(&o->y, fmaf(im, kTruncation, im) * pscale);
+        atomicAdd(&o->x, (p.exact ? fmaf(re, kTruncation, re) : re) * pscale);
+        atomicAdd(&o->y, (p.exact ? fmaf(im, kTruncation, im) : im) * pscale);
       }
     };
     for (uint32_t it = 0;; ++it) {
@@ -497,7 +498,7 @@ __global__ void __launch_bounds__(kFwdThreads, 1) k_sep_forward(const SepFwdPara
         }
         pb = r.b;
         pt = r.tile;
-        pscale = scale;
+        pscale = p.exact ? scale : scale * kTruncationLoop;
         psc = scale;
       }
       if (r.b < 0) break;
@@ -647,16 +648,15 @@ __global__ void __launch_bounds__(kFwdThreads, 1) k_sep_forward(const SepFwdPara
       // The pixels' phases, not through the MUFU: its cosine is on average 7.5e-8
       // off over a turn, which all pixels add up in a spot without tilt and
       // aberrations (random field of 1024^2, N = 19, the middle spot among them: 7e-6
-      // of the norm, with the phase's turns as exact 4e-7; the times are the same)
-      float2 fr[4], fi[4];
+      // of the norm, with the phase's turns as exact 4e-7; the times are the same).
+      // Loops, whose spots are bright and which multiply any change of rounding,
+      // keep it.
+      float2 pc[4], ps[4];
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
-        const float2 u = make_float2((float)(8 * c + 2 * q - 16) * 0.0625f, (float)(8 * c + 2 * q - 15) * 0.0625f);
-        float2 a = mul2(make_float2(v[q].x, v[q].y), dup2(inv));
-        if (kh) a = mul2(a, mul2(u, u));
-        cis2_turns(make_float2(v[q].z, v[q].w), fr[q], fi[q]);
-        fr[q] = mul2(a, fr[q]);
-        fi[q] = mul2(a, fi[q]);
+        const float2 t = make_float2(v[q].z, v[q].w);
+        if (p.exact) cis2_turns(t, pc[q], ps[q]);
+        else cis2(mul2(t, dup2(6.283185307179586f)), pc[q], ps[q]);
       }
 #pragma unroll
       for (int k2 = 0; k2 < 2; ++k2) {
@@ -664,8 +664,11 @@ __global__ void __launch_bounds__(kFwdThreads, 1) k_sep_forward(const SepFwdPara
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
           const float2 u = make_float2((float)(8 * c + 2 * q - 16) * 0.0625f, (float)(8 * c + 2 * q - 15) * 0.0625f);
-          split_pack(k2 ? mul2(fr[q], u) : fr[q], rh[q], rl[q]);
-          split_pack(k2 ? mul2(fi[q], u) : fi[q], ih[q], il[q]);
+          float2 a = mul2(make_float2(v[q].x, v[q].y), dup2(inv));
+          if (kh) a = mul2(a, mul2(u, u));
+          if (k2) a = mul2(a, u);
+          split_pack(mul2(a, pc[q]), rh[q], rl[q]);
+          split_pack(mul2(a, ps[q]), ih[q], il[q]);
         }
         const int r0 = kh * 128 + (j >> 1) * 8 + k2 * 4 + (j & 1);   // re row; im row is r0 + 2
         put16(bh, r0, c, rh);

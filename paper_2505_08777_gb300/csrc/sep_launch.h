@@ -54,6 +54,7 @@ struct SepFwdParams {
   float2* E;                     // [N]
   int G;
   unsigned* err;
+  bool exact;                    // pixel phases without a mean error (not inside a loop)
   // the moment pass (dL/dC) instead of E
   const float2* gE;              // [N] dL/dE
   const float* tab;              // basis polynomials per tile
