@@ -448,12 +448,13 @@ ash_status ash_hologram_launch_info(const ash_hologram *h, int *out);
  * Kernel variant of the forward and adjoint transforms and of the
  * coefficient-gradient moments: 0 = automatic (the faster measured family
  * per pass: the separable tile kernels for polynomial bases of total degree
- * <= 4 from N = 3 spots on grids whose shorter side is long enough (degree
- * 3 and 4: the forward from 400, the adjoint from 560, from 800 with fewer
- * than 64 spots, the moments from 900; degree <= 2: from 200 and 6 and 10 Mi
- * terms; ash_wgs_iterate: from 560 for every degree), unless the coefficients
- * at creation vary so strongly that most tiles need several row strips; else
- * tensor cores when the operand row fits one K-atom, for the
+ * <= 4, on grids whose shorter side is long enough (degree 3 and 4: the
+ * forward from 400, the adjoint from 560, both from 800 with fewer than 64
+ * spots, the moments from 900; degree <= 2: from 200, and 8 and 10 Mi terms;
+ * inside ash_wgs_iterate from 560), from 6 spots in the forward (16 for degree
+ * <= 2; of a field 12 and 24) and 4 in the adjoint (8 above 4 Mi pixels),
+ * unless the coefficients at creation vary so strongly that most tiles need
+ * several row strips; else tensor cores when the operand row fits one K-atom, for the
  * forward and the moments from N = 64 spots, for the adjoint from N = 256;
  * else the FMA pipe),
  * 1 = FMA-pipe kernels, 2 = tensor-core kernels (available for every D a

@@ -228,19 +228,27 @@ bool use_tc_adj(const ash_hologram* h) {
 // most tiles need one strip (forward: 742 x 486 N = 27 25 / 33, 1024^2 N = 20
 // 52 / 36, 800^2 N = 12 31 / 27; adjoint 16 / 31, 39 / 22, 27 / 18), and not
 // with one or two (calls, 1024^2: adjoint N = 1 18.3 / 21.3, 3 32.8 / 22.0; loop
-// of 5 iterations N = 1 300 / 370, 2 375 / 386, 3 384 / 382; 3000 x 2000:
-// adjoint N = 4 92 / 95, 8 104 / 95). Degree 2
+// of 5 iterations N = 1 300 / 370, 2 375 / 386, 3 384 / 382, 1920 x 1152 N = 3 with
+// the FMA forward 721 / 727; 3000 x 2000:
+// adjoint N = 4 92 / 95, 8 104 / 95); a field, which the FMA kernel reads without
+// sines and cosines, from more (1024^2 D = 5 N = 8 28.7 / 36.3, N = 16 34.8 / 36.9,
+// 800 x 800 N = 30 35 / 27; D = 10 800^2 N = 6 26.7 / 28.7, 1200 x 900 N = 12 45 /
+// 40). Degree 2
 // (one mixed term): forward 220^2 N = 30 12.5 / 13.8,
 // 300^2 N = 200 28 / 17; adjoint 256^2 N = 100 13.5 / 16.4, 300^2 N = 200
 // 24 / 20.
 constexpr int kSepSideFwd = 400, kSepSideAdj = 560, kSepSide2 = 200, kSepFewSpots = 64, kSepFewSide = 800;
-constexpr long long kSepTerms2Fwd = 6LL << 20, kSepTerms2Adj = 10LL << 20;
-constexpr int kSepFewest = 3, kSepFewestLarge = 8;
+constexpr long long kSepTerms2Fwd = 8LL << 20, kSepTerms2Adj = 10LL << 20;
+constexpr int kSepFewest = 6, kSepFewest2 = 16;            // forward, of degree 3 and 4 and of degree <= 2
+constexpr int kSepFewestField = 12, kSepFewestField2 = 24; // of a field
+constexpr int kSepFewestAdj = 4, kSepFewestLarge = 8;
 constexpr long long kSepLarge = 4LL << 20;   // pixels
 bool sep_pays(const ash_hologram* h, int side4, long long terms2) {
   const Geometry& g = h->g;
   const int side = g.nx < g.ny_full ? g.nx : g.ny_full;
-  if (g.N < (side4 == kSepSideAdj && (long long)g.nx * g.ny > kSepLarge ? kSepFewestLarge : kSepFewest)) return false;
+  const int fewest = side4 == kSepSideFwd ? (h->sep_ord <= 2 ? kSepFewest2 : kSepFewest)
+                                          : ((long long)g.nx * g.ny > kSepLarge ? kSepFewestLarge : kSepFewestAdj);
+  if (g.N < fewest) return false;
   if (h->sep_ord <= 2) return side >= kSepSide2 && (long long)g.nx * g.ny * g.N >= terms2;
   return side >= side4 && (g.N >= kSepFewSpots || side >= kSepFewSide);
 }
@@ -270,6 +278,10 @@ bool use_sep_fwd(const ash_hologram* h, bool loop = false) {
 bool use_sep_adj(const ash_hologram* h, bool loop = false) {
   return h->sep_ok && h->sep_cheap_adj && h->variant == 0 && (!loop || sep_in_loops(h)) && sep_pays(h, kSepSideAdj, kSepTerms2Adj);
 }
+// The forward of a complex field.
+bool use_sep_field(const ash_hologram* h) {
+  return use_sep_fwd(h) && h->g.N >= (h->sep_ord <= 2 ? kSepFewestField2 : kSepFewestField);
+}
 // The coefficient-gradient moments on the tensor cores need one K-atom,
 // D <= 12 and a polynomial basis of total degree <= 4 (the tile polynomials);
 // from N = 64, as the forward whose structure they share.
@@ -298,7 +310,7 @@ bool needs_tc_images(const ash_hologram* h) {
 // Whether the handle's current kernel choice runs any FMA-pipe kernel (they
 // read the register-image basis dz; the tensor-core kernels do not).
 bool needs_fma_image(const ash_hologram* h) {
-  return !((use_sep_fwd(h, true) || use_tc_fwd(h)) && (use_sep_adj(h, true) || use_tc_adj(h)) &&
+  return !(((use_sep_fwd(h, true) && use_sep_field(h)) || use_tc_fwd(h)) && (use_sep_adj(h, true) || use_tc_adj(h)) &&
            (use_sep_grad(h) || use_tc_grad(h)));
 }
 
@@ -387,7 +399,8 @@ cudaError_t capturing(cudaStream_t s, bool* captured) {
 // before the next call of this.
 cudaError_t enqueue_tc_coeff(ash_hologram* h, cudaStream_t s, bool forward_only = false) {
   if (!h->tc_ok) return cudaSuccess;
-  if (h->sep_ok) {
+  if (forward_only && !use_sep_fwd(h) && !use_tc_fwd(h)) return cudaSuccess;   // the FMA forward reads the coefficients
+  if (h->sep_ok && (use_sep_fwd(h) || !forward_only)) {
     const cudaError_t e = sep_build_params(h->g, h->sep_tab, h->coeff, h->sep_poly, h->sep_strips, h->sep_cost,
                                            h->sep_acost, s);
     if (e != cudaSuccess) return e;
@@ -501,7 +514,7 @@ cudaError_t launch_gradc(int D, const GradCParams& p, dim3 grid, cudaStream_t s)
 // forward transform into E (device complex [N]); loop: as a WGS loop runs it.
 ash_status enqueue_forward(ash_hologram* h, int source, const float* phase, const float2* field, float2* E,
                            cudaStream_t s, bool loop = false) {
-  const bool sep = use_sep_fwd(h, loop);
+  const bool sep = source == kSrcField ? use_sep_field(h) : use_sep_fwd(h, loop);
   if (!sep) {
     const ash_status st = fresh_tc_images(h, s);
     if (st != ASH_OK) return st;

@@ -53,6 +53,22 @@ def test_left_to_the_other_kernels(nx, ny, N, noll, scale, variant):
     assert all(torch.equal(a, b) for a, b in zip(got, want))
 
 
+@pytest.mark.parametrize("nx,ny,N,noll,other", [(901, 930, 11, LOW, True), (901, 930, 12, LOW, False),
+                                                (1030, 1000, 23, [2, 3, 4, 5, 6], True),
+                                                (1030, 1000, 24, [2, 3, 4, 5, 6], False)])
+def test_a_field_on_few_spots(nx, ny, N, noll, other):
+    p, ph, _ = _problem(nx, ny, N, noll, 0.1)
+    Z, C, A = oracle_inputs(p)
+    f = torch.polar(torch.from_numpy(p.amp).cuda(), ph)
+    h = _holo(p, p.coeff)
+    assert h.launch_info()["kernels"] & 16
+    E = h.forward_field(f)
+    assert torch.equal(E, _holo(p, p.coeff, 1).forward_field(f)) == other
+    ref = transform.forward(f.cpu().numpy().astype(np.complex128).ravel(), C, Z, workers=8)
+    assert_close(E.cpu().numpy(), ref, 1e-5, "field")
+    h.check()
+
+
 @pytest.mark.parametrize("nx,ny,N,scale", [(577, 590, 100, 30.0), (640, 600, 97, 6.0), (905, 903, 161, 30.0)])
 def test_stronger_coefficients_set_later(nx, ny, N, scale):
     p, ph, y = _problem(nx, ny, N, LOW, scale)
@@ -114,6 +130,10 @@ def test_a_handle_without_memory_for_them_serves_on_the_other_kernels():
     (803, 801, 7, LOW, 0.1, 16 | 32 | 128 | 256),
     (905, 903, 161, LOW, 0.1, 16 | 32 | 64 | 128 | 256),
     (901, 930, 2, LOW, 1.0, 0),
+    (901, 930, 3, LOW, 0.1, 0),
+    (901, 930, 4, LOW, 0.1, 32 | 64 | 256),
+    (901, 930, 6, LOW, 0.1, 16 | 32 | 64 | 128 | 256),
+    (1030, 1030, 15, [2, 3, 4, 5, 6], 1.0, 32 | 64 | 256),
     (233, 201, 231, [2, 3, 4, 5, 6], 1.0, 16 | 32),
     (901, 930, 20, [2, 3, 4, 5, 6], 1.0, 16 | 32 | 64 | 128 | 256),
     (600, 600, 70, list(range(2, 17)), 0.05, 0),          # degree 5
